@@ -113,15 +113,14 @@ int ensure_device(pmlbie_problem* prob) {
         (rc = upload(D.corr_w, H.corr_w)))
         return rc;
     const int M = prob->P.M;
-    std::vector<double2> cs(M / 2 + 1), tw(M), tw2(2 * M);
+    std::vector<double2> cs(M / 2 + 1), tw2(2 * M);
     for (int e = 0; e < 2 * M; ++e)
         tw2[e] = make_double2(std::cos(kPi * e / M), -std::sin(kPi * e / M));
     for (int j = 0; j <= M / 2; ++j) {
         double s = std::sin(kPi * j / M);
         cs[j] = make_double2(s * s, std::cos(2.0 * kPi * j / M));
     }
-    for (int e = 0; e < M; ++e) tw[e] = make_double2(std::cos(2.0 * kPi * e / M), -std::sin(2.0 * kPi * e / M));
-    if ((rc = upload(D.cos_tab, cs)) || (rc = upload(D.twid, tw)) || (rc = upload(D.twid2, tw2))) return rc;
+    if ((rc = upload(D.cos_tab, cs)) || (rc = upload(D.twid2, tw2)) || (rc = upload(D.twid_fx, fx_twiddles(M)))) return rc;
     {
         const int nr = rec_table_len(M);
         std::vector<double2> up(nr), dn(nr);
@@ -159,7 +158,7 @@ int ensure_device(pmlbie_problem* prob) {
 void free_device(pmlbie_problem* prob) {
     DeviceTables& D = prob->D;
     void* ptrs[] = {D.rho, D.z, D.I, D.Wu, D.Wphi, D.rho_t, D.nuc_r, D.nuc_z, D.bk, D.off, D.cls, D.near, D.near_lead,
-                    D.corr_target, D.corr_m, D.corr_coef, D.Da, D.Db, D.cos_tab, D.twid, D.twid2,
+                    D.corr_target, D.corr_m, D.corr_coef, D.Da, D.Db, D.cos_tab, D.twid2, D.twid_fx,
                     D.corr_start, D.corr_cmin, D.corr_w, D.rec_up, D.rec_dn, D.twid_ff, D.twid2_ff, D.cos_ff, D.exp_ff, D.trig_ff, D.wuc_ff,
                     D.wpc_ff};
     for (void* p : ptrs)

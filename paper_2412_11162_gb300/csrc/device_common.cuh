@@ -46,6 +46,12 @@ __device__ __forceinline__ double2 cexpi(double2 q) {
 }
 __device__ __forceinline__ double2 clog(double2 z) { return c2(log(hypot(z.x, z.y)), atan2(z.y, z.x)); }
 
+// every quantity of a close pair real (two physical nodes)
+__device__ __forceinline__ bool near_physical(const NearPair& q) {
+    return q.d2.y == 0.0 && q.rr.y == 0.0 && q.rho_t.y == 0.0 && q.rho_s.y == 0.0 && q.drt.y == 0.0 &&
+           q.nuc_r.y == 0.0 && q.nuc_z.y == 0.0;
+}
+
 // Geometry of a grid pair (l, m) from node tables: the symmetric sampling
 // quantities d~^2 and rho~_l rho~_m, and for both orientations the normal
 // factor N_D(psi) = nd0 + nds sin^2(psi/2) of the double layer at the source

@@ -378,6 +378,63 @@ bool solve_ld(std::vector<q128::real>& A, std::vector<q128::real>& b, int n) {
 
 }  // namespace
 
+// Twiddles of the fixed-point transforms (fxdft.cuh): cos and sin of pi e / M on
+// the first octant by their Taylor series in double-double arithmetic (106 bits;
+// 22 terms leave less than 2^-80 at pi/4), rounded to Q62, the other octants by
+// symmetry.
+namespace {
+struct Dd {
+    double h, l;
+};
+Dd dd_quick(double a, double b) {
+    const double s = a + b;
+    return {s, b - (s - a)};
+}
+Dd dd_mul(Dd a, Dd b) {
+    const double p = a.h * b.h;
+    return dd_quick(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+Dd dd_add(Dd a, Dd b) {
+    const double s = a.h + b.h, t = s - a.h;
+    return dd_quick(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
+}
+Dd dd_div(Dd a, double d) {
+    const double q = a.h / d;
+    return dd_quick(q, (std::fma(-q, d, a.h) + a.l) / d);
+}
+int64_t dd_q62(Dd a) {
+    const double t = a.h * 4611686018427387904.0, f = std::floor(t);
+    return (int64_t)f + (int64_t)std::floor((t - f) + a.l * 4611686018427387904.0 + 0.5);
+}
+}  // namespace
+
+std::vector<int4> fx_twiddles(int M) {
+    const int Q = M / 2;                     // quarter of the circle of 2M steps
+    std::vector<int64_t> C(Q / 2 + 1), S(Q / 2 + 1);
+    const Dd pi{3.141592653589793116, 1.2246467991473531772e-16};
+    for (int e = 0; e <= Q / 2; ++e) {
+        const Dd x = dd_div(dd_mul(pi, Dd{(double)e, 0.0}), M), x2 = dd_mul(x, x);
+        Dd c{1.0, 0.0}, s = x, tc = c, ts = x;
+        for (int k = 1; k <= 11; ++k) {
+            tc = dd_div(dd_mul(tc, x2), -(2.0 * k - 1.0) * (2.0 * k));
+            ts = dd_div(dd_mul(ts, x2), -(2.0 * k) * (2.0 * k + 1.0));
+            c = dd_add(c, tc);
+            s = dd_add(s, ts);
+        }
+        C[e] = dd_q62(c);
+        S[e] = dd_q62(s);
+    }
+    std::vector<int4> tw(3 * (size_t)M / 2);
+    for (int e = 0; e < 3 * M / 2; ++e) {
+        const int q = e / Q, r = e % Q;
+        const int64_t c0 = r <= Q / 2 ? C[r] : S[Q - r], s0 = r <= Q / 2 ? S[r] : C[Q - r];
+        const int64_t re = q == 0 ? c0 : q == 1 ? -s0 : -c0, im = -(q == 0 ? s0 : q == 1 ? c0 : -s0);
+        const int rl = (int)(uint32_t)(uint64_t)re, il = (int)(uint32_t)(uint64_t)im;
+        tw[e] = make_int4((int)((re - rl) >> 32), rl, (int)((im - il) >> 32), il);
+    }
+    return tw;
+}
+
 // ---------------------------------------------------------------------------
 // Alpert's log-singular end correction (j nodes, skip a): nodes x_k in (0, a)
 // and weights w_k with  sum_k w_k x_k^p = -zeta(-p, a)  and

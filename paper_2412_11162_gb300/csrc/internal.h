@@ -97,10 +97,10 @@ struct DeviceTables {
     int* corr_w = nullptr;
     double *Da = nullptr, *Db = nullptr;
     double2* cos_tab = nullptr;   // (sin^2(psi_j/2), cos psi_j), j = 0..M/2
-    double2* twid = nullptr;      // e^{-2 pi i e / M}, e = 0..M-1
     double2* twid2 = nullptr;     // e^{-2 pi i e / (2M)}, e = 0..2M-1
+    int4* twid_fx = nullptr;      // e^{-2 pi i e / (2M)}, e = 0..3M/2-1, Q62 balanced digits (fxdft.cuh)
     // float-float copies for the mixed path's kernels (kernels_ff.cu): the
-    // twiddles and angle table above as (re.hi, re.lo, im.hi, im.lo), the exp
+    // length-M and length-2M twiddles and the angle table above as (re.hi, re.lo, im.hi, im.lo), the exp
     // and sin / cos tables of ffloat.cuh, and per node h W_u / (2M) and
     // h W_phi / (2M) (column weight times the trapezoid factor of the modes)
     // coefficients of the Legendre-Q three-term recurrence of the close-pair
@@ -158,6 +158,9 @@ bool device_ready(const pmlbie_problem* prob);
 
 // host setup (host.cpp)
 int build_tables(pmlbie_problem* prob);
+// e^{-2 pi i e / (2M)}, e = 0..3M/2-1, as Q62 integers in balanced 32-bit digits
+// (re.high, re.low, im.high, im.low), correctly rounded to about one unit
+std::vector<int4> fx_twiddles(int M);
 void alpert_log_rule(int j, int a, std::vector<double>& x, std::vector<double>& w);
 
 // kernels (kernels.cu)

@@ -15,11 +15,13 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "internal.h"
 #include "device_common.cuh"
 #include "fp64_elem.cuh"
 #include "ffloat.cuh"
+#include "modal_fx.cuh"
 
 namespace pmlbie {
 
@@ -33,6 +35,11 @@ namespace {
 constexpr double kUpward = kRecUpward;
 
 // ---------------------------------------------------------------------------
+// FP64 transforms of the close pairs with a PML point (near_modes_kernel): the
+// Sec. 4.3 split cancels by up to 1e12 there, so that any change of rounding moves
+// the solutions of ill-conditioned modes; every other transform is fixed point
+// (fxdft.cuh).
+//
 // Warp-cooperative Stockham FFT (forward, e^{-2 pi i k n / M}) in shared
 // memory, radices 4, 2, 3 (M = 2^a 3^b).  x, y: two buffers of M elements;
 // returns the buffer holding the result.  tw[e] = e^{-2 pi i e / M}.
@@ -86,15 +93,6 @@ __device__ double2* warp_fft(double2* x, double2* y, int M, const double2* tw, i
         rem /= R;
     }
     return x;
-}
-
-// FFT of buf (length M) using scratch; the result ends in buf.
-__device__ void warp_fft_inplace(double2* buf, double2* scratch, int M, const double2* tw, int lane) {
-    double2* r = warp_fft(buf, scratch, M, tw, lane);
-    if (r != buf) {
-        for (int i = lane; i < M; i += 32) buf[i] = r[i];
-        __syncwarp();
-    }
 }
 
 // DFT of an even sequence x_0..x_{L-1} (x_k = x_{L-k}, L = 2K, K even) from
@@ -158,23 +156,6 @@ __device__ void warp_even_dft(double2* xh, double2* y, double2* scr, int K, cons
     __syncwarp();
 }
 
-// The double layer's normal factor nd0 + nds sin^2(psi/2) multiplies the
-// geometric factor g(psi) = e^{iq}(1 - iq) / |Delta|^3 (times constants); on
-// the M-point DFT, sin^2(psi/2) = (1 - cos psi)/2 acts as G_n -> G_n / 2 -
-// (G_{n-1} + G_{n+1}) / 4 (exact; G_{-1} = G_1 for even g, and n + 1 <= M/2
-// stays inside the spectrum).  sin2_mode gives that shifted spectrum, shared
-// by both orientations of a pair; nd_mode combines it with one orientation's
-// normal factor (real arithmetic when the factor is real: two physical nodes).
-__device__ __forceinline__ double2 sin2_mode(const double2* gh, int n) {
-    const double2 gn = gh[n], gm = gh[n == 0 ? 1 : n - 1], gp = gh[n + 1];
-    return c2(fma(0.5, gn.x, -0.25 * (gm.x + gp.x)), fma(0.5, gn.y, -0.25 * (gm.y + gp.y)));
-}
-__device__ __forceinline__ double2 nd_mode(double2 nd0, double2 nds, double2 gn, double2 s2, bool real) {
-    if (real) return c2(fma(nd0.x, gn.x, nds.x * s2.x), fma(nd0.x, gn.y, nds.x * s2.y));
-    return c2(fma(nd0.x, gn.x, fma(-nd0.y, gn.y, fma(nds.x, s2.x, -nds.y * s2.y))),
-              fma(nd0.x, gn.y, fma(nd0.y, gn.x, fma(nds.x, s2.y, nds.y * s2.x))));
-}
-
 // ---------------------------------------------------------------------------
 // Far pairs.  The kernel samples the ordered pairs (l, m) and (m, l) together:
 // |Delta| is symmetric in the two nodes, so S~ is, and K~ differs between the
@@ -188,65 +169,49 @@ __device__ __forceinline__ double2 nd_mode(double2 nd0, double2 nds, double2 gn,
 // far entries with their weighted modes, all others with zero (close pairs
 // and skipped pairs are filled in by the assembly).
 // ---------------------------------------------------------------------------
-struct FarArgs {
-    DeviceTables T;
-    int N, M, mode_lo, mode_hi;
-    double w1, w2, h;
-    double2* A;     // [mode][col][row], ld 2N
-    double2* raw;   // [mode][kernel][l][m]
-};
+// Shared memory of a far_kernel CTA with nw pairs, in double2: the twiddles of
+// one length-M transform, the angle table, and per pair the geometry, the scatter's
+// factors, four sequences of M/2 + 1 values and (four to an entry) flags and exponents.
+__host__ __device__ __forceinline__ size_t far_elems(int M, int nw) {
+    return (size_t)3 * M / 4 + (M / 2 + 1) + (size_t)nw * (12 + 4 * (size_t)(M / 2 + 1)) + (5 * (size_t)nw + 3) / 4;
+}
 
-// targets x sources of a CTA with nw pairs
-__host__ __device__ __forceinline__ int far_tile_m(int nw) { return nw >= 16 ? 4 : 2; }
-
-__global__ void __launch_bounds__(512, 2) far_kernel(FarArgs a) {
+// The samples are FP64; the transforms run on the integer pipe in block fixed
+// point (fxdft.cuh), and the scatter's normal factors carry the column weights.
+template <int NB>
+__global__ void __launch_bounds__(512, NB == 1 ? 2 : 1) far_kernel(FarArgs a) {
     extern __shared__ double2 smem[];
     const int M = a.M, N = a.N, K = M / 2, S1 = K + 1;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int TM = far_tile_m(nw), TL = nw / TM;
     const int l0 = blockIdx.x * TL, m0 = blockIdx.y * TM;
     if (l0 + TL - 1 < m0) return;               // the whole tile has l < m: mirrored elsewhere
-    double2* tw = smem;                         // M: e^{-2 pi i e / M}
-    double2* hs = tw + M;                       // K: even-DFT weights
-    double2* cs = hs + K;                       // K + 1: (sin^2(psi/2), cos psi)
+    int4* tw = reinterpret_cast<int4*>(smem);   // 3M/4: e^{-2 pi i e / M}
+    double2* cs = smem + 3 * M / 4;             // K + 1: (sin^2(psi/2), cos psi)
     PairGeom* geo = reinterpret_cast<PairGeom*>(cs + S1);                  // nw pairs
-    double2* bufs = cs + S1 + 6 * nw;           // per warp: 4 sequences of K+1, then 2 x K scratch
-    int* act = reinterpret_cast<int*>(bufs + nw * (4 * S1 + 2 * K));     // nw flags
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-        const double2 t = a.T.twid[i];
-        tw[i] = t;
-        if (i < K) hs[i] = c2(0.5 + t.y, 0.5 - t.y);
-    }
+    FarPairFx* pf = reinterpret_cast<FarPairFx*>(geo + nw);                // nw pairs
+    double2* bufs = reinterpret_cast<double2*>(pf + nw);                   // per pair: 4 sequences of K+1
+    int* act = reinterpret_cast<int*>(bufs + (size_t)nw * 4 * S1);         // nw flags
+    int* exs = act + nw;                        // per pair: the sequences' exponents
+    for (int i = threadIdx.x; i < 3 * M / 4; i += blockDim.x) tw[i] = a.T.twid_fx[2 * i];
     for (int i = threadIdx.x; i <= K; i += blockDim.x) cs[i] = a.T.cos_tab[i];
-    // warp w: target l = l0 + w % TL, source m = m0 + w / TL.  act bit 0: (l, m)
-    // is far; bit 1: (m, l) is far; bit 2: the warp owns its entries (l >= m);
-    // bit 3: real pair quantities.
-    if (lane == 0) {
-        const int l = l0 + warp % TL, m = m0 + warp / TL;
-        int f = 0;
-        if (l < N && m < N && l >= m) {
-            f = 4;
-            if (l > m) {
-                f |= (a.T.cls[(size_t)l * N + m] == kFar ? 1 : 0) | (a.T.cls[(size_t)m * N + l] == kFar ? 2 : 0);
-                if (f & 3) {
-                    const PairGeom g = grid_pair(a.T, l, m);
-                    geo[warp] = g;
-                    // bit 3: every pair quantity real (two physical nodes)
-                    if (g.d2.y == 0.0 && g.rr.y == 0.0 && g.nd0.y == 0.0 && g.nds.y == 0.0 && g.nd0t.y == 0.0 &&
-                        g.ndst.y == 0.0)
-                        f |= 8;
-                }
-            }
+    // all pairs by the lanes of warp 0: an FP64 instruction occupies its pipe for a
+    // whole warp whatever the active lanes
+    if (warp == 0 && lane < nw) {
+        PairGeom g;
+        FarPairFx o;
+        const int f = far_pair_setup(a, l0 + lane % TL, m0 + lane / TL, g, o);
+        if (f & 3) {
+            geo[lane] = g;
+            pf[lane] = o;
         }
-        act[warp] = f;
+        act[lane] = f;
     }
     __syncthreads();
 
     // samples j = 0..K of the CTA's pairs, spread over all its threads:
-    // S~ = e^{iq} / (4 pi |Delta|) and g = -(e^{iq}(1 - iq)) / (4 pi |Delta|^3)
-    // (region b: -g, its normal is -nu), q = omega |Delta|, both times the
-    // trapezoid factor 2 pi / M of the modes (c4 = (1 / 4 pi)(2 pi / M))
-    const double c4 = 0.5 / M;
+    // 4 pi S~ = e^{iq} / |Delta| and g = -(e^{iq}(1 - iq)) / |Delta|^3 (region b: -g, its
+    // normal is -nu), q = omega |Delta|
     // (pair w, angle j) over the CTA's threads, advanced without a division
     int w = threadIdx.x / S1, j = threadIdx.x - (threadIdx.x / S1) * S1;
     const int bstep = blockDim.x / S1, jstep = blockDim.x - bstep * S1;
@@ -258,13 +223,13 @@ __global__ void __launch_bounds__(512, 2) far_kernel(FarArgs a) {
         }
         if (!(act[w] & 3)) continue;
         const PairGeom& g = geo[w];
-        double2* buf = bufs + w * (4 * S1 + 2 * K);
+        double2* buf = bufs + (size_t)w * 4 * S1;
         const double2 sc = cs[j];
         if (g.d2.y == 0.0 && g.rr.y == 0.0) {
             // both nodes physical: real distance, e^{iq} = cos q + i sin q
             const double D2 = fma(4.0 * sc.x, g.rr.x, g.d2.x);
             const double iR = frsqrt(D2), R = D2 * iR;
-            const double gk = -c4 * (iR * iR * iR), f = c4 * iR;
+            const double gk = -(iR * iR * iR), f = iR;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const double q = (r == 0 ? a.w1 : a.w2) * R, gr = r == 0 ? gk : -gk;
@@ -278,80 +243,29 @@ __global__ void __launch_bounds__(512, 2) far_kernel(FarArgs a) {
         const double2 D2 = cadd(g.d2, cscale(g.rr, 4.0 * sc.x));
         double2 R, iR;
         fcsqrt_rcp(D2, R, iR);
-        const double2 gk = cscale(cmul(iR, cmul(iR, iR)), -c4);
+        const double2 gk = cscale(cmul(iR, cmul(iR, iR)), -1.0);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const double w = r == 0 ? a.w1 : a.w2;
             const double2 gr = r == 0 ? gk : c2(-gk.x, -gk.y);
             const double2 q = cscale(R, w);
             const double2 e = fcexpi(q);
-            buf[(2 * r) * S1 + j] = cscale(cmul(e, iR), c4);
+            buf[(2 * r) * S1 + j] = cmul(e, iR);
             buf[(2 * r + 1) * S1 + j] = cmul(cmul(gr, e), c2(1.0 + q.y, -q.x));   // (1 - i q)
         }
     }
     __syncthreads();
     if (act[warp] & 3) {
-        double2* buf = bufs + warp * (4 * S1 + 2 * K);
-        double2* y = buf + 4 * S1;
-        for (int s = 0; s < 4; ++s) warp_even_dft(buf + s * S1, y, y + K, K, tw, hs, 1, lane);
+        for (int s = 0; s < 4; ++s) {
+            double2* seq = bufs + ((size_t)warp * 4 + s) * S1;
+            const int ex =
+                fx_even_dft<NB>(reinterpret_cast<longlong2*>(seq), fx_quantise(seq, S1, lane), K, tw, 1, lane);
+            if (lane == 0) exs[4 * warp + s] = ex;
+        }
     }
     __syncthreads();
 
-    // scatter: thread (pair w, mode n) forms the eight entries of both
-    // orientations from the pair's spectra (kernel 0 S^a, 1 g^a, 2 S^b, 3 g^b)
-    const int nmodes = a.mode_hi - a.mode_lo;
-    const int lg = __ffs(nw) - 1, lgl = __ffs(TL) - 1;
-    const int total = nmodes << lg;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int w = idx & (nw - 1), n = idx >> lg;
-        const int f = act[w];
-        if (!(f & 4)) continue;
-        const int l = l0 + (w & (TL - 1)), m = m0 + (w >> lgl);
-        const int nn = a.mode_lo + n;
-        double2 sa = c2(0.0, 0.0), sb = sa, ka[2] = {sa, sa}, kb[2] = {sa, sa};
-        if (f & 3) {
-            const double2* b = bufs + w * (4 * S1 + 2 * K);
-            const PairGeom& g = geo[w];
-            const bool real = (f & 8) != 0;
-            sa = b[nn];
-            sb = b[2 * S1 + nn];
-            const double2 ga = b[S1 + nn], gb = b[3 * S1 + nn];
-            const double2 s2a = sin2_mode(b + S1, nn), s2b = sin2_mode(b + 3 * S1, nn);
-            if (f & 1) {
-                ka[0] = nd_mode(g.nd0, g.nds, ga, s2a, real);
-                kb[0] = nd_mode(g.nd0, g.nds, gb, s2b, real);
-            }
-            if (f & 2) {
-                ka[1] = nd_mode(g.nd0t, g.ndst, ga, s2a, real);
-                kb[1] = nd_mode(g.nd0t, g.ndst, gb, s2b, real);
-            }
-        }
-        for (int o = 0; o < 2; ++o) {
-            if (o == 1 && l == m) break;             // the diagonal entry once
-            const int tgt = o == 0 ? l : m, src = o == 0 ? m : l;
-            const bool on = (f >> o) & 1;
-            if (a.A) {
-                // blocks: K^a -> (t, s); -S^a -> (t, N+s); K^b -> (N+t, s); S^b -> (N+t, N+s)
-                const size_t ld = 2 * (size_t)N;
-                double2* col0 = a.A + (size_t)n * ld * ld + (size_t)src * ld;
-                double2* col1 = col0 + (size_t)N * ld;
-                const double wu = a.h * a.T.Wu[src], wp = a.h * a.T.Wphi[src];
-                const double2 z = c2(0.0, 0.0);
-                col0[tgt] = on ? cscale(ka[o], wu) : z;
-                col1[tgt] = on ? cscale(sa, -wp) : z;
-                col0[N + tgt] = on ? cscale(kb[o], wu) : z;
-                col1[N + tgt] = on ? cscale(sb, wp) : z;
-            }
-            if (a.raw) {
-                const size_t NN = (size_t)N * N, e = (size_t)tgt * N + src;
-                const double2 z = c2(0.0, 0.0);
-                a.raw[((size_t)n * 4 + 0) * NN + e] = on ? sa : z;
-                a.raw[((size_t)n * 4 + 1) * NN + e] = on ? ka[o] : z;
-                a.raw[((size_t)n * 4 + 2) * NN + e] = on ? sb : z;
-                a.raw[((size_t)n * 4 + 3) * NN + e] = on ? kb[o] : z;
-            }
-        }
-    }
+    far_scatter(a, nw, l0, m0, reinterpret_cast<const longlong2*>(bufs), exs, pf, act);
 }
 
 // ---------------------------------------------------------------------------
@@ -377,12 +291,9 @@ struct NearArgs {
     double2* out;    // [p][4][nmodes]
     double2 pa[8], pb[8];   // Taylor coefficients of cH1 (pa) and cH3 (pb)
     int hs_tab;             // keep the even-DFT weight table in shared memory
-    int only_subst;         // 1: the modes kernel handles only the pairs with the
-                            // Sec. 4.3 substitution (the mixed path's float-float
-                            // kernel takes the others)
     float4* pff;            // per-pair float-float quantities (kNearFF float4), or null
-    int share_mirror;       // 1: a general (non-packed, non-plain) grid pair and its
-                            // mirror are computed by one CTA (shared memory permitting)
+    int share_mirror;       // 1: a pair with a PML point and its mirror are computed by one
+                            // CTA (shared memory permitting)
     const int* lead;        // pairs whose Laplace modes a thread computes (HostTables::near_lead)
     int nlead;
 };
@@ -525,8 +436,7 @@ __device__ void near_pair_ff(const NearPair& q, double w1, double w2, float4* ou
     out[3] = c4(cscale(cmul(q.nuc_r, q.rho_t), 2.0), -e);
     out[4] = r4(ldexp(w1, e), ldexp(w2, e));
     out[5] = r4(ldexp(1.0 / w1, -e), ldexp(1.0 / w2, -e));
-    const bool phys = q.d2.y == 0.0 && q.rr.y == 0.0 && q.rho_t.y == 0.0 && q.rho_s.y == 0.0 && q.drt.y == 0.0 &&
-                      q.nuc_r.y == 0.0 && q.nuc_z.y == 0.0;
+    const bool phys = near_physical(q);
     out[6] = make_float4(__int_as_float(e), __int_as_float(phys ? 1 : 0), 0.0f, 0.0f);
 }
 
@@ -669,16 +579,11 @@ __global__ void __launch_bounds__(128) near_laplace_out_kernel(NearArgs a) {
     }
 }
 
-// Close pairs, stage 2 (one CTA of 4 warps per pair): samples of the smooth
-// factors f1, f3 and remainders r1, r3 (both regions; for PML pairs the
-// Taylor substitution of Sec. 4.3, otherwise H1 = cos q, H3 = cos q + q sin q),
-// their FFTs, and the convolution
+// Close pairs with a PML point, stage 2 (one CTA of 4 warps per pair), FP64
+// throughout (above): samples of the smooth factors f1, f3 and remainders r1, r3
+// (both regions; the Taylor substitution of Sec. 4.3), their FFTs, and the convolution
 //   S^_n = (1/2pi) sum_{|k| < M/2} Z^_{|n-k|} F1_k + R1_n   (K^_n with D^, F3, R3).
 // Correction pairs that are far by the criterion use the plain FFT.
-// Physical pairs (no point in the PML) have real Z^, D^, f1, f3 and purely
-// imaginary r1, r3, so the two regions are packed as real and imaginary parts
-// of one sequence: 4 sample transforms and 4 convolution transforms instead
-// of 8 and 8.
 // kExact: the diagnostic exact split on PML pairs (compiled into its own
 // variant so that the default one keeps its register budget)
 // Mirror sharing (a.share_mirror): a grid pair (l, m) of the general path and
@@ -716,20 +621,14 @@ __global__ void near_modes_kernel(NearArgs a) {
     NearPair q = a.np[p];
     const bool plain = (q.flags & kFlagFar) != 0;
     const bool subst = (q.flags & kFlagSubst) != 0;
-    if (a.only_subst && !subst) return;
-    // both points physical: every pair quantity is real (the two regions pack
-    // into one transform); a PML pair without the substitution (diagnostic
-    // exact split) takes the general path
-    const bool phys = q.d2.y == 0.0 && q.rr.y == 0.0 && q.rho_t.y == 0.0 && q.rho_s.y == 0.0 && q.drt.y == 0.0 &&
-                      q.nuc_r.y == 0.0 && q.nuc_z.y == 0.0;
-    const bool packed = !plain && !subst && phys;
+    // the other pairs: near_modes_fx_kernel or the float-float kernel
+    if (!subst && (plain || near_physical(q))) return;
     // mirror sharing (both pairs on the general path, same substitution flag)
     bool share = false;
     NearPair qm;
-    if (a.share_mirror && !plain && !packed && q.mirror >= 0) {
+    if (a.share_mirror && !plain && q.mirror >= 0) {
         qm = a.np[q.mirror];
-        const bool mphys = qm.d2.y == 0.0 && qm.rr.y == 0.0 && qm.rho_t.y == 0.0 && qm.rho_s.y == 0.0 &&
-                           qm.drt.y == 0.0 && qm.nuc_r.y == 0.0 && qm.nuc_z.y == 0.0;
+        const bool mphys = near_physical(qm);
         const bool msubst = (qm.flags & kFlagSubst) != 0;
         share = (qm.flags & kFlagFar) == 0 && msubst == subst && !(mphys && !msubst);
         if (share && q.mirror < p) return;    // computed by the mirror's CTA
@@ -751,32 +650,6 @@ __global__ void near_modes_kernel(NearArgs a) {
         fcsqrt_rcp(D2, R, iR);
         const double2 ND = cadd(nd0, cscale(nds, sc.x));
         const double2 NDm = cadd(nd0m, cscale(ndsm, sc.x));
-        if (packed) {
-            // real q = w R; H1 = cos q, i Z H2 = (i w / 4 pi) sin(q)/q, H3 = cos q + q sin q,
-            // i D H4 = -(i w^3 / 4 pi) N_D (sin q - q cos q)/q^3 (region b: -N_D)
-            double f1[2], r1[2], f3[2], r3[2];
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const double w = r == 0 ? a.w1 : a.w2;
-                const double qr = w * R.x, iq = iR.x / w;
-                double sn, cs;
-                fsincos(qr, &sn, &cs);
-                const double q2 = qr * qr;
-                const double sinc = fabs(qr) < 1e-3 ? 1.0 - q2 / 6.0 + q2 * q2 / 120.0 : sn * iq;
-                const double h4 = fabs(qr) < 1e-2
-                                      ? 1.0 / 3.0 - q2 / 30.0 + q2 * q2 / 840.0 - q2 * q2 * q2 / 45360.0
-                                      : (sn - qr * cs) * (iq * iq * iq);
-                f1[r] = cs;
-                r1[r] = w * kInv4Pi * sinc;
-                f3[r] = fma(qr, sn, cs);
-                r3[r] = (r == 0 ? -1.0 : 1.0) * w * w * w * kInv4Pi * h4 * ND.x;
-            }
-            seq[0 * S1 + j] = c2(f1[0], f1[1]);
-            seq[1 * S1 + j] = c2(r1[0], r1[1]);
-            seq[2 * S1 + j] = c2(f3[0], f3[1]);
-            seq[3 * S1 + j] = c2(r3[0], r3[1]);
-            continue;
-        }
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const double w = r == 0 ? a.w1 : a.w2;
@@ -838,15 +711,10 @@ __global__ void near_modes_kernel(NearArgs a) {
         }
     }
     __syncthreads();
-    // even-sequence DFTs of length M: packed pairs 4 (one per warp), plain
-    // pairs 0, 2, 4, 6, the others all 8
-    if (packed) {
-        warp_even_dft(seq + warp * S1, wyK, wyK + K, K, tw2, hs, 2, lane);
-    } else {
-        for (int s = warp; s < (share ? 10 : 8); s += 4) {
-            if (plain && (s & 1)) continue;
-            warp_even_dft(s < 8 ? seq + s * S1 : seqm + (s - 8) * S1, wyK, wyK + K, K, tw2, hs, 2, lane);
-        }
+    // even-sequence DFTs of length M: plain pairs 0, 2, 4, 6, the others all 8
+    for (int s = warp; s < (share ? 10 : 8); s += 4) {
+        if (plain && (s & 1)) continue;
+        warp_even_dft(s < 8 ? seq + s * S1 : seqm + (s - 8) * S1, wyK, wyK + K, K, tw2, hs, 2, lane);
     }
     __syncthreads();
     const double scale = 2.0 * kPi / M;
@@ -885,17 +753,13 @@ __global__ void near_modes_kernel(NearArgs a) {
     if (warp < 2) warp_even_dft(warp == 0 ? zZ : zD, slot, slot + M, M, tw2, hs, 1, lane);
     if (share && warp == 2) warp_even_dft(zDm, slot2, slot2 + M, M, tw2, hs, 1, lane);
     const double c = 1.0 / (2.0 * kPi * L2);
-    // packed: one pass with cS = F1a + i F1b and cK = F3a - i F3b (region b's -D^
-    // as the conjugate); otherwise one pass per region
-    const int passes = packed ? 1 : 2;
-    for (int r = 0; r < passes; ++r) {
+    for (int r = 0; r < 2; ++r) {
         for (int i = threadIdx.x; i <= M; i += blockDim.x) {
             bool in = i <= K - 1;
             double2 vS = c2(0.0, 0.0), vK = c2(0.0, 0.0);
             if (in) {
-                vS = cscale(seq[(packed ? 0 : 4 * r + 0) * S1 + i], scale);
-                vK = cscale(seq[(packed ? 2 : 4 * r + 2) * S1 + i], scale);
-                if (packed) vK.y = -vK.y;
+                vS = cscale(seq[(4 * r + 0) * S1 + i], scale);
+                vK = cscale(seq[(4 * r + 2) * S1 + i], scale);
             }
             cS[i] = vS;
             cK[i] = vK;
@@ -903,7 +767,7 @@ __global__ void near_modes_kernel(NearArgs a) {
         __syncthreads();
         if (warp >= 2) warp_even_dft(warp == 2 ? cS : cK, slot, slot + M, M, tw2, hs, 1, lane);
         __syncthreads();
-        const double sgn = r == 0 ? 1.0 : -1.0;      // region b: D^ -> -D^ (unpacked)
+        const double sgn = r == 0 ? 1.0 : -1.0;      // region b: D^ -> -D^
         for (int i = threadIdx.x; i <= M; i += blockDim.x) {
             cS[i] = cmul(zZ[i], cS[i]);
             if (share) cKm[i] = cscale(cmul(zDm[i], cK[i]), sgn);
@@ -915,27 +779,124 @@ __global__ void near_modes_kernel(NearArgs a) {
         __syncthreads();
         for (int t = threadIdx.x; t < nmodes; t += blockDim.x) {
             int n = a.mode_lo + t;
-            if (packed) {
-                // real parts from the convolutions, imaginary parts from the remainders
-                const double2 s0 = cscale(cS[n], c), k0 = cscale(cK[n], c);
-                const double2 rs = cscale(seq[1 * S1 + n], scale), rk = cscale(seq[3 * S1 + n], scale);
-                out[0 * (size_t)nmodes + t] = c2(s0.x, rs.x);
-                out[1 * (size_t)nmodes + t] = c2(k0.x, rk.x);
-                out[2 * (size_t)nmodes + t] = c2(s0.y, rs.y);
-                out[3 * (size_t)nmodes + t] = c2(k0.y, rk.y);
-            } else {
-                const double2 sv = cadd(cscale(cS[n], c), cscale(seq[(4 * r + 1) * S1 + n], scale));
-                out[(2 * r + 0) * (size_t)nmodes + t] = sv;
-                out[(2 * r + 1) * (size_t)nmodes + t] =
-                    cadd(cscale(cK[n], c), cscale(seq[(4 * r + 3) * S1 + n], scale));
-                if (share) {
-                    outm[(2 * r + 0) * (size_t)nmodes + t] = sv;
-                    outm[(2 * r + 1) * (size_t)nmodes + t] = cadd(cscale(cKm[n], c), cscale(seqm[r * S1 + n], scale));
-                }
+            const double2 sv = cadd(cscale(cS[n], c), cscale(seq[(4 * r + 1) * S1 + n], scale));
+            out[(2 * r + 0) * (size_t)nmodes + t] = sv;
+            out[(2 * r + 1) * (size_t)nmodes + t] = cadd(cscale(cK[n], c), cscale(seq[(4 * r + 3) * S1 + n], scale));
+            if (share) {
+                outm[(2 * r + 0) * (size_t)nmodes + t] = sv;
+                outm[(2 * r + 1) * (size_t)nmodes + t] = cadd(cscale(cKm[n], c), cscale(seqm[r * S1 + n], scale));
             }
         }
         __syncthreads();
     }
+}
+
+// Close pairs without a PML point (and correction pairs far by the criterion),
+// stage 2, FP64 samples: physical pairs have real Z^, D^, f1, f3 and purely
+// imaginary r1, r3 (H1 = cos q, H3 = cos q + q sin q), so the two regions are packed
+// as real and imaginary parts of one sequence; the transforms and the convolution
+// run in block fixed point (near_finish).  The FP64 path; the mixed path takes the
+// same pairs with float-float samples.  Mirror sharing as above.
+//
+// Threads of a CTA and its shared memory (double2): three quarters of the length-2M
+// twiddles, 7 sample sequences (M/2 + 1; packed pairs use 5), three Laplace-mode and
+// two convolution sequences (M + 1)
+__host__ __device__ constexpr int near_threads(int NB) { return NB <= 2 ? 128 : 256; }
+static size_t near_elems(int M) { return (size_t)3 * M / 2 + 7 * (size_t)(M / 2 + 1) + 5 * (size_t)(M + 1); }
+
+template <int NB>
+__global__ void __launch_bounds__(near_threads(NB), NB <= 2 ? 4 : NB <= 4 ? 2 : 1) near_modes_fx_kernel(NearArgs a) {
+    extern __shared__ double2 smem[];
+    const int M = a.M, K = M / 2, S1 = K + 1, S2 = M + 1, p = blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    int4* tw = reinterpret_cast<int4*>(smem);   // 3M/2: e^{-2 pi i e / (2M)}
+    double2* seq = smem + 3 * M / 2;    // 7 sequences of K+1 (samples, then spectra)
+    double2* zs = seq + 7 * S1;         // Z^, D^, the mirror's D^
+    double2* cv = zs + 3 * S2;          // S and K convolution
+    const NearPair q = a.np[p];
+    const bool plain = (q.flags & kFlagFar) != 0;
+    if ((q.flags & kFlagSubst) || !(plain || near_physical(q))) return;   // near_modes_kernel's
+    const bool packed = !plain;
+    bool share = false;
+    NearPair qm;
+    if (packed && q.mirror >= 0) {
+        qm = a.np[q.mirror];
+        share = (qm.flags & (kFlagFar | kFlagSubst)) == 0 && near_physical(qm);
+        if (share && q.mirror < p) return;    // computed by the mirror's CTA
+    }
+    for (int i = threadIdx.x; i < 3 * M / 2; i += blockDim.x) tw[i] = a.T.twid_fx[i];
+    double2* seqm = seq + 4 * S1;       // the mirror's r3
+    // sampling; N_D(psi) = [nu'_r (rho~' - rho~) - nu'_z dz] + 2 nu'_r rho~ sin^2(psi/2)
+    const double2 nd0 = cadd(cmul(q.nuc_r, q.drt), cscale(q.nuc_z, -q.dz));
+    const double2 nds = cscale(cmul(q.nuc_r, q.rho_t), 2.0);
+    double2 nd0m = c2(0.0, 0.0), ndsm = nd0m;
+    if (share) {
+        nd0m = cadd(cmul(qm.nuc_r, qm.drt), cscale(qm.nuc_z, -qm.dz));
+        ndsm = cscale(cmul(qm.nuc_r, qm.rho_t), 2.0);
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j <= K; j += blockDim.x) {
+        const double2 sc = a.T.cos_tab[j];
+        const double2 D2 = cadd(q.d2, cscale(q.rr, 4.0 * sc.x));
+        double2 R, iR;
+        fcsqrt_rcp(D2, R, iR);
+        const double2 ND = cadd(nd0, cscale(nds, sc.x));
+        const double2 NDm = cadd(nd0m, cscale(ndsm, sc.x));
+        if (packed) {
+            // real q = w R; H1 = cos q, i Z H2 = (i w / 4 pi) sin(q)/q, H3 = cos q + q sin q,
+            // i D H4 = -(i w^3 / 4 pi) N_D (sin q - q cos q)/q^3 (region b: -N_D)
+            double f1[2], r1[2], f3[2], r3[2], r3m[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const double w = r == 0 ? a.w1 : a.w2;
+                const double qr = w * R.x, iq = iR.x / w;
+                double sn, cs;
+                fsincos(qr, &sn, &cs);
+                const double q2 = qr * qr;
+                const double sinc = fabs(qr) < 1e-3 ? 1.0 - q2 / 6.0 + q2 * q2 / 120.0 : sn * iq;
+                const double h4 = fabs(qr) < 1e-2
+                                      ? 1.0 / 3.0 - q2 / 30.0 + q2 * q2 / 840.0 - q2 * q2 * q2 / 45360.0
+                                      : (sn - qr * cs) * (iq * iq * iq);
+                f1[r] = cs;
+                r1[r] = w * kInv4Pi * sinc;
+                f3[r] = fma(qr, sn, cs);
+                const double h4w = (r == 0 ? -1.0 : 1.0) * w * w * w * kInv4Pi * h4;
+                r3[r] = h4w * ND.x;
+                r3m[r] = h4w * NDm.x;
+            }
+            seq[0 * S1 + j] = c2(f1[0], f1[1]);
+            seq[1 * S1 + j] = c2(r1[0], r1[1]);
+            seq[2 * S1 + j] = c2(f3[0], f3[1]);
+            seq[3 * S1 + j] = c2(r3[0], r3[1]);
+            if (share) seqm[j] = c2(r3m[0], r3m[1]);
+            continue;
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const double w = r == 0 ? a.w1 : a.w2;
+            const double sg = r == 0 ? 1.0 : -1.0;     // region b normal -nu
+            const double2 qq = cscale(R, w);
+            const double2 e = fcexpi(qq);
+            const double2 iR3 = cmul(iR, cmul(iR, iR));
+            const double2 Dk = cscale(cmul(ND, iR3), -kInv4Pi * sg);
+            seq[(4 * r + 0) * S1 + j] = cscale(cmul(e, iR), kInv4Pi);
+            seq[(4 * r + 2) * S1 + j] = cmul(cmul(Dk, e), c2(1.0 + qq.y, -qq.x));
+        }
+    }
+    __syncthreads();
+    NearShape sh;
+    sh.packed = packed;
+    sh.plain = plain;
+    sh.share = share;
+    sh.mode_lo = a.mode_lo;
+    sh.nmodes = a.mode_hi - a.mode_lo;
+    sh.Z = a.zd + (size_t)p * 2 * M;
+    sh.D = sh.Z + M;
+    sh.Dm = share ? a.zd + (size_t)q.mirror * 2 * M + M : nullptr;
+    sh.out = a.out + (size_t)p * 4 * sh.nmodes;
+    sh.outm = share ? a.out + (size_t)q.mirror * 4 * sh.nmodes : nullptr;
+    near_finish<NB>(sh, M, tw, reinterpret_cast<longlong2*>(seq), zs, cv,
+                    [&](longlong2* x, int) { return fx_quantise(x, S1, lane); });
 }
 
 // ---------------------------------------------------------------------------
@@ -1102,19 +1063,15 @@ struct RhsArgs {
     double2* b2;
 };
 
+template <int NB>
 __global__ void rhs_kernel(RhsArgs a) {
     extern __shared__ double2 sm[];
     const int l = blockIdx.x, r = blockIdx.y, M = a.M, K = M / 2;
-    double2* tw = sm;                    // M: e^{-2 pi i e / M}
-    double2* hs = tw + M;                // K: even-DFT weights
-    double2* s1 = hs + K;                // K + 1 samples -> spectrum
+    int4* tw = reinterpret_cast<int4*>(sm);   // 3M/4: e^{-2 pi i e / M}
+    double2* s1 = sm + 3 * M / 4;        // K + 1 samples -> spectrum
     double2* s2 = s1 + (K + 1);
-    double2* scr = s2 + (K + 1);         // 2 warps x 2K
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-        const double2 t = a.T.twid[i];
-        tw[i] = t;
-        if (i < K) hs[i] = c2(0.5 + t.y, 0.5 - t.y);
-    }
+    __shared__ int exs[2];
+    for (int i = threadIdx.x; i < 3 * M / 4; i += blockDim.x) tw[i] = a.T.twid_fx[2 * i];
     const double* pr = a.rhs_par + kRhsPar * r;
     double sp = pr[0], cp = pr[1];
     double2 R = c2(pr[2], pr[3]), ks = c2(pr[4], pr[5]);
@@ -1140,8 +1097,9 @@ __global__ void rhs_kernel(RhsArgs a) {
     // warp), then the incidence azimuth theta_inc rotates mode n by e^{-i n theta_inc}
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < 2) {
-        double2* y = scr + warp * 2 * K;
-        warp_even_dft(warp == 0 ? s1 : s2, y, y + K, K, tw, hs, 1, lane);
+        double2* x = warp == 0 ? s1 : s2;
+        const int ex = fx_even_dft<NB>(reinterpret_cast<longlong2*>(x), fx_quantise(x, K + 1, lane), K, tw, 1, lane);
+        if (lane == 0) exs[warp] = ex;
     }
     __syncthreads();
     const double scale = 2.0 * kPi / M, az = pr[6];
@@ -1151,8 +1109,8 @@ __global__ void rhs_kernel(RhsArgs a) {
         sincos(n * az, &sr, &cr);
         const double2 rot = c2(-scale * cr, scale * sr);      // -(2 pi/M) e^{-i n theta_inc}
         size_t o = ((size_t)t * a.N + l) * a.nrhs + r;
-        a.b1[o] = cmul(s1[n], rot);
-        a.b2[o] = cmul(s2[n], rot);
+        a.b1[o] = cmul(fx_to_double2(reinterpret_cast<const longlong2*>(s1)[n], exs[0]), rot);
+        a.b2[o] = cmul(fx_to_double2(reinterpret_cast<const longlong2*>(s2)[n], exs[1]), rot);
     }
 }
 
@@ -1207,13 +1165,7 @@ __global__ void outputs_kernel(int N, int nmodes, int nrhs, const double2* X, co
 // ---------------------------------------------------------------------------
 static int far_warps(int M) { return M <= 512 ? 8 : 4; }
 
-// shared memory of a far_kernel CTA with nw pairs: twiddles M, DFT weights
-// M/2, angle table S1, nw pair geometries (6 double2 each), nw buffers, nw flags
-static size_t far_smem(int M, int nw) {
-    const size_t S1 = M / 2 + 1;
-    return sizeof(double2) * ((size_t)M + M / 2 + S1 + 6 * (size_t)nw + (size_t)nw * (4 * S1 + M)) +
-           sizeof(double2) * (((size_t)nw + 3) / 4);
-}
+static size_t far_smem(int M, int nw) { return sizeof(double2) * far_elems(M, nw); }
 
 // Autotuned pairs per CTA of the far kernel, per (N, M, modes, output kind):
 // the first tunable launch of a shape runs every candidate that fits in
@@ -1237,15 +1189,17 @@ cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStre
     a.h = prob->H.h;
     a.A = fl.A;
     a.raw = fl.raw;
-    cudaError_t e = allow_max_smem(far_kernel);
+    cudaError_t e = with_half_class(M, [](auto nb) { return allow_max_smem(far_kernel<decltype(nb)::value>); });
     if (e != cudaSuccess) return e;
     auto run = [&](int nw) {
         g_far_pairs_per_cta = nw;
         const int tm = far_tile_m(nw), tl = nw / tm;
         dim3 grid((N + tl - 1) / tl, (N + tm - 1) / tm);
-        far_kernel<<<grid, 32 * nw, far_smem(M, nw), s>>>(a);
-        count_launch();
-        return cudaGetLastError();
+        return with_half_class(M, [&](auto nb) {
+            far_kernel<decltype(nb)::value><<<grid, 32 * nw, far_smem(M, nw), s>>>(a);
+            count_launch();
+            return cudaGetLastError();
+        });
     };
     // PMLBIE_FAR_PAIRS_PER_CTA=2|4|8|16 fixes the choice (reproducible profiling)
     static const int forced = [] {
@@ -1329,7 +1283,6 @@ cudaError_t launch_near(const pmlbie_problem* prob, int mode_lo, int mode_hi, do
     a.w2 = prob->P.k2;
     a.zd = zd;
     a.out = out;
-    a.only_subst = 0;
     const bool use_ff = ff && !prob->P.subst_off;
     a.pff = use_ff ? reinterpret_cast<float4*>(zd + (size_t)a.npairs * 2 * M) : nullptr;
     taylor_coeffs(a.L, a.pa, a.pb);
@@ -1352,10 +1305,20 @@ cudaError_t launch_near(const pmlbie_problem* prob, int mode_lo, int mode_hi, do
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (mid && (e = cudaEventRecord(mid, s)) != cudaSuccess) return e;
+    // the pairs without a PML point in float-float or FP64, then the others in FP64
     if (use_ff) {
-        // float-float for the pairs without a PML point, FP64 for the others
         if ((e = launch_near_modes_ff(prob, mode_lo, mode_hi, zd, a.pff, out, s)) != cudaSuccess) return e;
-        a.only_subst = 1;
+    } else {
+        const size_t smem = sizeof(double2) * near_elems(M);
+        e = with_full_class(M, [&](auto nb) {
+            constexpr int NB = decltype(nb)::value;
+            const cudaError_t er = allow_max_smem(near_modes_fx_kernel<NB>);
+            if (er != cudaSuccess) return er;
+            near_modes_fx_kernel<NB><<<a.npairs, near_threads(NB), smem, s>>>(a);
+            count_launch();
+            return cudaGetLastError();
+        });
+        if (e != cudaSuccess) return e;
     }
     if (mid_ff && (e = cudaEventRecord(mid_ff, s)) != cudaSuccess) return e;
     // tw2 (2M) + 8 x (M/2+1) + 4 x (M+1) + 2 scratch slots x 2M (+ M weights when they
@@ -1441,16 +1404,12 @@ cudaError_t launch_rhs(const pmlbie_problem* prob, int n_rhs, int mode_lo, int m
     a.b1 = b1;
     a.b2 = b2;
     dim3 grid(a.N, n_rhs);
-    // twiddles M, weights M/2, two spectra M/2+1, two warps' scratch 2 x M
-    const size_t K = a.M / 2;
-    size_t smem = sizeof(double2) * ((size_t)a.M + K + 2 * (K + 1) + 4 * K);
-    if (smem > 48 * 1024) {
-        cudaError_t e = allow_max_smem(rhs_kernel);
-        if (e != cudaSuccess) return e;
-    }
-    rhs_kernel<<<grid, 128, smem, s>>>(a);
-    count_launch();
-    return cudaGetLastError();
+    const size_t smem = sizeof(double2) * ((size_t)3 * a.M / 4 + 2 * (size_t)(a.M / 2 + 1));
+    return with_half_class(a.M, [&](auto nb) {
+        rhs_kernel<decltype(nb)::value><<<grid, 128, smem, s>>>(a);
+        count_launch();
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_block_rhs(const pmlbie_problem* prob, int n_rhs, int nm, const double2* A,
@@ -1496,11 +1455,13 @@ struct FieldArgs {
 };
 
 // S~ and K~ of one (physical point x = (rx, 0, zx), node m) pair at the M/2+1
-// distinct angles, then their modes by two even-sequence DFTs: buf[0..K] holds
-// M/(2 pi) S^_n and buf[S1..S1+K] M/(2 pi) K^_n, n = 0..K, with the double-layer
-// kernel along sg times the node's conormal.  One warp; buf holds 4 K + 2 doubles2.
-__device__ void point_node_modes(const DeviceTables& T, int M, double w, double sg, double rx, double zx, int m,
-                                 const double2* cs, const double2* tw, const double2* hs, double2* buf, int lane) {
+// distinct angles, then their modes by two even-sequence DFTs (fxdft.cuh): buf[0..K]
+// holds M/(2 pi) S^_n and buf[S1..S1+K] M/(2 pi) K^_n, n = 0..K, in fixed point with
+// the exponents exS, exK, the double-layer kernel along sg times the node's
+// conormal.  One warp; buf holds 2 S1 values.
+template <int NB>
+__device__ __forceinline__ void point_node_modes(const DeviceTables& T, int M, double w, double sg, double rx, double zx, int m,
+                                 const double2* cs, const int4* tw, double2* buf, int lane, int& exS, int& exK) {
     const int K = M / 2, S1 = K + 1;
     const double dr = rx - T.rho[m], dz = zx - T.z[m], dI = -T.I[m];   // the point is physical: I = 0
     const double2 drt = c2(dr, dI);
@@ -1522,43 +1483,43 @@ __device__ void point_node_modes(const DeviceTables& T, int M, double w, double 
         buf[S1 + j] = cmul(cmul(cscale(cmul(ND, iR3), -kInv4Pi), e), c2(1.0 + q.y, -q.x));
     }
     __syncwarp();
-    double2* y = buf + 2 * S1;
-    warp_even_dft(buf, y, y + K, K, tw, hs, 1, lane);
-    warp_even_dft(buf + S1, y, y + K, K, tw, hs, 1, lane);
+    longlong2* f = reinterpret_cast<longlong2*>(buf);
+    exS = fx_even_dft<NB>(f, fx_quantise(buf, S1, lane), K, tw, 1, lane);
+    exK = fx_even_dft<NB>(f + S1, fx_quantise(buf + S1, S1, lane), K, tw, 1, lane);
 }
 
-// Shared tables of the point kernels: twiddles (M), half-sum weights (K), cos (K + 1).
-__device__ void point_tables(const DeviceTables& T, int M, double2* tw, double2* hs, double2* cs) {
-    const int K = M / 2;
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-        const double2 t = T.twid[i];
-        tw[i] = t;
-        if (i < K) hs[i] = c2(0.5 + t.y, 0.5 - t.y);
-    }
-    for (int i = threadIdx.x; i <= K; i += blockDim.x) cs[i] = T.cos_tab[i];
+// Shared tables of the point kernels: twiddles (3M/4), cos (K + 1).
+__device__ void point_tables(const DeviceTables& T, int M, int4* tw, double2* cs) {
+    for (int i = threadIdx.x; i < 3 * M / 4; i += blockDim.x) tw[i] = T.twid_fx[2 * i];
+    for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) cs[i] = T.cos_tab[i];
     __syncthreads();
 }
+static size_t point_smem(int M, int nw) {
+    return sizeof(double2) * ((size_t)3 * M / 4 + (M / 2 + 1) + (size_t)nw * 2 * (M / 2 + 1));
+}
 
+template <int NB>
 __global__ void field_kernel(FieldArgs a) {
     extern __shared__ double2 smem[];
     const int M = a.M, K = M / 2, S1 = K + 1;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double2* tw = smem;                      // M
-    double2* hs = tw + M;                    // K
-    double2* cs = hs + K;                    // K + 1
-    double2* buf = cs + S1 + warp * (2 * S1 + 2 * K);
-    point_tables(a.T, M, tw, hs, cs);
+    int4* tw = reinterpret_cast<int4*>(smem);
+    double2* cs = smem + 3 * M / 4;
+    double2* buf = cs + S1 + warp * 2 * S1;
+    point_tables(a.T, M, tw, cs);
     const int p = blockIdx.y, m = blockIdx.x * nw + warp;
     if (m >= a.N) return;
     const int reg = a.preg[p];
     const double sg = reg == 0 ? 1.0 : -1.0;
-    point_node_modes(a.T, M, reg == 0 ? a.w1 : a.w2, sg, a.prho[p], a.pz[p], m, cs, tw, hs, buf, lane);
+    int exS, exK;
+    point_node_modes<NB>(a.T, M, reg == 0 ? a.w1 : a.w2, sg, a.prho[p], a.pz[p], m, cs, tw, buf, lane, exS, exK);
+    const longlong2* f = reinterpret_cast<const longlong2*>(buf);
     const double scale = 2.0 * kPi / M;
     const double fs = 0.5 * sg * scale * a.h * a.T.Wphi[m], fk = -0.5 * scale * a.h * a.T.Wu[m];
     double2* o = a.coef + ((size_t)p * a.N + m) * a.nmodes * 2;
     for (int t = lane; t < a.nmodes; t += 32) {
-        o[2 * t] = cscale(buf[a.mode_lo + t], fs);
-        o[2 * t + 1] = cscale(buf[S1 + a.mode_lo + t], fk);
+        o[2 * t] = cscale(fx_to_double2(f[a.mode_lo + t], exS), fs);
+        o[2 * t + 1] = cscale(fx_to_double2(f[S1 + a.mode_lo + t], exK), fk);
     }
 }
 
@@ -1567,20 +1528,22 @@ __global__ void field_kernel(FieldArgs a) {
 //   b1_n(m) = -e^{-i n phi_s} S^a_n(x_s, r_m),  b2_n(m) = -e^{-i n phi_s} |r'_m| K^a_n(x_s, r_m)
 // (the modes of -G~_1(r~_m, x_s) and -|r'| d_nu_c G~_1 over the node azimuth),
 // laid out [mode - mode_lo][node][rhs].  One warp per (node, source).
+template <int NB>
 __global__ void point_rhs_kernel(DeviceTables T, int N, int M, int nrhs, int mode_lo, int nmodes, double w1,
                                  const double* rpar, const double* speed, double2* b1, double2* b2) {
     extern __shared__ double2 smem[];
     const int K = M / 2, S1 = K + 1;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double2* tw = smem;
-    double2* hs = tw + M;
-    double2* cs = hs + K;
-    double2* buf = cs + S1 + warp * (2 * S1 + 2 * K);
-    point_tables(T, M, tw, hs, cs);
+    int4* tw = reinterpret_cast<int4*>(smem);
+    double2* cs = smem + 3 * M / 4;
+    double2* buf = cs + S1 + warp * 2 * S1;
+    point_tables(T, M, tw, cs);
     const int r = blockIdx.y, m = blockIdx.x * nw + warp;
     if (m >= N) return;
     const double* pr = rpar + (size_t)kRhsPar * r;
-    point_node_modes(T, M, w1, 1.0, pr[0], pr[1], m, cs, tw, hs, buf, lane);
+    int exS, exK;
+    point_node_modes<NB>(T, M, w1, 1.0, pr[0], pr[1], m, cs, tw, buf, lane, exS, exK);
+    const longlong2* f = reinterpret_cast<const longlong2*>(buf);
     const double scale = 2.0 * kPi / M, az = pr[6], sp = speed[m];
     for (int t = lane; t < nmodes; t += 32) {
         const int n = mode_lo + t;
@@ -1588,8 +1551,8 @@ __global__ void point_rhs_kernel(DeviceTables T, int N, int M, int nrhs, int mod
         sincos(n * az, &sr, &cr);
         const double2 rot = c2(-scale * cr, scale * sr);      // -(2 pi/M) e^{-i n phi_s}
         const size_t o = ((size_t)t * N + m) * nrhs + r;
-        b1[o] = cmul(buf[n], rot);
-        b2[o] = cscale(cmul(buf[S1 + n], rot), sp);
+        b1[o] = cmul(fx_to_double2(f[n], exS), rot);
+        b2[o] = cscale(cmul(fx_to_double2(f[S1 + n], exK), rot), sp);
     }
 }
 
@@ -1634,13 +1597,16 @@ cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prh
     a.pz = pz;
     a.preg = preg;
     a.coef = coef;
-    const int nw = 4, K = a.M / 2;
-    const size_t smem = sizeof(double2) * ((size_t)a.M + K + (K + 1) + (size_t)nw * (2 * (K + 1) + 2 * K));
-    if (smem > 48 * 1024) {
-        cudaError_t e = allow_max_smem(field_kernel);
+    const int nw = 4;
+    const size_t smem = point_smem(a.M, nw);
+    const cudaError_t ef = with_half_class(a.M, [&](auto nb) {
+        constexpr int NB = decltype(nb)::value;
+        cudaError_t e = smem > 48 * 1024 ? allow_max_smem(field_kernel<NB>) : cudaSuccess;
         if (e != cudaSuccess) return e;
-    }
-    field_kernel<<<dim3((a.N + nw - 1) / nw, npts), 32 * nw, smem, s>>>(a);
+        field_kernel<NB><<<dim3((a.N + nw - 1) / nw, npts), 32 * nw, smem, s>>>(a);
+        return cudaGetLastError();
+    });
+    if (ef != cudaSuccess) return ef;
     const size_t tot = (size_t)a.nmodes * npts * nrhs;
     field_contract_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(a.N, npts, a.nmodes, nrhs, preg, coef, u1,
                                                                         phi1, u2, phi2, out);
@@ -1651,17 +1617,17 @@ cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prh
 cudaError_t launch_point_rhs(const pmlbie_problem* prob, int n_rhs, int mode_lo, int mode_hi,
                              const double* rhs_par_dev, const double* speed, double2* b1, double2* b2,
                              cudaStream_t s) {
-    const int N = prob->P.N, M = prob->P.M, K = M / 2, nw = 4;
-    const size_t smem = sizeof(double2) * ((size_t)M + K + (K + 1) + (size_t)nw * (2 * (K + 1) + 2 * K));
-    if (smem > 48 * 1024) {
-        cudaError_t e = allow_max_smem(point_rhs_kernel);
+    const int N = prob->P.N, M = prob->P.M, nw = 4;
+    const size_t smem = point_smem(M, nw);
+    return with_half_class(M, [&](auto nb) {
+        constexpr int NB = decltype(nb)::value;
+        cudaError_t e = smem > 48 * 1024 ? allow_max_smem(point_rhs_kernel<NB>) : cudaSuccess;
         if (e != cudaSuccess) return e;
-    }
-    point_rhs_kernel<<<dim3((N + nw - 1) / nw, n_rhs), 32 * nw, smem, s>>>(prob->D, N, M, n_rhs, mode_lo,
-                                                                           mode_hi - mode_lo, prob->P.k1,
-                                                                           rhs_par_dev, speed, b1, b2);
-    count_launch();
-    return cudaGetLastError();
+        point_rhs_kernel<NB><<<dim3((N + nw - 1) / nw, n_rhs), 32 * nw, smem, s>>>(
+            prob->D, N, M, n_rhs, mode_lo, mode_hi - mode_lo, prob->P.k1, rhs_par_dev, speed, b1, b2);
+        count_launch();
+        return cudaGetLastError();
+    });
 }
 
 namespace {
