@@ -209,6 +209,7 @@ struct Workspace {
     int2* ptab = nullptr;           // the FP32 LU's row-interchange mapping per step
     int *piv = nullptr, *info = nullptr, *active = nullptr, *nanflag = nullptr;
     double *rn = nullptr, *bn = nullptr, *xn = nullptr, *an = nullptr, *rpar = nullptr;
+    size_t near_bytes = 0;          // zd and nout together
     size_t bytes = 0;
 };
 
@@ -247,8 +248,10 @@ Workspace plan(const pmlbie_problem* prob, int precision, int nrhs, int nmodes, 
         w.ptab = (int2*)take(sizeof(int2) * lu_ptab_elems((int)n2, (int)nm));
         w.R = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
     }
+    const size_t near0 = off;
     w.zd = (double2*)take(near_zd_bytes(std::max<size_t>(np, 1), M, true));
     w.nout = (double2*)take(sizeof(double2) * std::max<size_t>(np, 1) * 4 * nm);
+    w.near_bytes = off - near0;
     w.b1 = (double2*)take(sizeof(double2) * nm * N * nrhs);
     w.b2 = (double2*)take(sizeof(double2) * nm * N * nrhs);
     w.B = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
@@ -591,9 +594,9 @@ __global__ void wait_probe_kernel(long long iters, int* expired) {
 thread_local int g_lu_graph_replays = 0;
 
 static cudaError_t lu_direct(int precision, int n, int batch, void* A, int* piv, int* info, unsigned char* img,
-                             int2* ptab, const LuSide* side, cudaStream_t s, cudaEvent_t* upd_ev = nullptr) {
+                             int2* ptab, const LuSide* side, cudaStream_t s, cudaEvent_t* upd_ev, size_t img_bytes) {
     return precision == PMLBIE_FP64
-               ? batched_lu<double2>(n, batch, (double2*)A, piv, info, s, nullptr, nullptr, nullptr, upd_ev)
+               ? batched_lu<double2>(n, batch, (double2*)A, piv, info, s, img, nullptr, nullptr, upd_ev, img_bytes)
                : batched_lu<float2>(n, batch, (float2*)A, piv, info, s, img, ptab, side, upd_ev);
 }
 
@@ -612,7 +615,7 @@ static cudaError_t ensure_update_events(pmlbie_dev_extra* ex, int n) {
 }
 
 static int batched_lu_graphed(pmlbie_problem* prob, int precision, int n, int batch, void* A, int* piv, int* info,
-                              unsigned char* img, int2* ptab, cudaStream_t s) {
+                              unsigned char* img, int2* ptab, cudaStream_t s, size_t img_bytes = 0) {
     pmlbie_dev_extra* ex = extra_of(prob);
     LuGraph& g = ex->lu;
     PMLBIE_CUDA_TRY(ensure_update_events(ex, n));
@@ -622,7 +625,8 @@ static int batched_lu_graphed(pmlbie_problem* prob, int precision, int n, int ba
         PMLBIE_CUDA_TRY(cudaEventCreateWithFlags(&ex->lu_side.join, cudaEventDisableTiming));
     }
     if (g.unavailable) {
-        PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data()));
+        PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data(),
+                                  img_bytes));
         return PMLBIE_OK;
     }
     LuKey key;
@@ -640,7 +644,8 @@ static int batched_lu_graphed(pmlbie_problem* prob, int precision, int n, int ba
         if (!(g.has_pending && g.pending == key)) {
             g.pending = key;
             g.has_pending = true;
-            PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data()));
+            PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data(),
+                                  img_bytes));
             return PMLBIE_OK;
         }
         if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -652,7 +657,8 @@ static int batched_lu_graphed(pmlbie_problem* prob, int precision, int n, int ba
         cudaError_t e = cudaStreamBeginCapture(ex->capture, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             const cudaError_t el =
-                lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, ex->capture, ex->upd_ev.data());
+                lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, ex->capture, ex->upd_ev.data(),
+                          img_bytes);
             e = cudaStreamEndCapture(ex->capture, &graph);
             if (el != cudaSuccess) e = el;
         }
@@ -665,7 +671,8 @@ static int batched_lu_graphed(pmlbie_problem* prob, int precision, int n, int ba
             if (g.exec) cudaGraphExecDestroy(g.exec);
             g = LuGraph();
             g.unavailable = true;
-            PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data()));
+            PMLBIE_CUDA_TRY(lu_direct(precision, n, batch, A, piv, info, img, ptab, &ex->lu_side, s, ex->upd_ev.data(),
+                                  img_bytes));
             return PMLBIE_OK;
         }
         g.launches = captured;
@@ -734,7 +741,12 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
     bool unconverged = false;
     std::vector<double> mres(nm, 0.0), mbwd(nm, 0.0);
     if (precision == PMLBIE_FP64) {
-        if ((rc = batched_lu_graphed(prob, PMLBIE_FP64, n2, nm, w.A, w.piv, w.info, nullptr, nullptr, s))) return rc;
+        // the close-pair scratch is free after the assembly: the digit images of the
+        // updates live in it (about 20 corrections per node and more, 32 M bytes of
+        // Laplace modes each: more than one mode's images, 3 KB per row of the system)
+        if ((rc = batched_lu_graphed(prob, PMLBIE_FP64, n2, nm, w.A, w.piv, w.info, (unsigned char*)w.zd, nullptr, s,
+                                     w.near_bytes)))
+            return rc;
         PMLBIE_CUDA_TRY(cudaEventRecord(ev[2], s));
         PMLBIE_CUDA_TRY(cudaMemcpyAsync(w.X, w.B, xbytes, cudaMemcpyDeviceToDevice, s));
         PMLBIE_CUDA_TRY((batched_lu_solve<double2, double2>(n2, nm, n_rhs, w.A, w.piv, w.X, s)));

@@ -277,8 +277,8 @@ int peak_probe(int kind, double* out_tflops, cudaStream_t s);
 // (its update launch, with its operand-image launch when that is on s; for its
 // timing; recorded as external events, so that they become event-record nodes
 // when the factorisation is captured in a graph)
-// img: for complex64, lu_image_bytes(n, batch) bytes of device scratch (16-byte
-// aligned) holding one step's split operand images; unused for complex128
+// img: device scratch (16-byte aligned) of one step's split operand images, for
+// complex64 lu_image_bytes(n, batch) bytes, for complex128 img_bytes
 // ptab: for complex64, lu_ptab_elems(n, batch) entries receiving each step's
 // row-interchange mapping: the interchanges are applied to the columns right of
 // each panel only (L keeps the row order of its step), piv keeps LAPACK's
@@ -293,7 +293,11 @@ struct LuSide {
 };
 template <typename T>
 cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t s, unsigned char* img,
-                       int2* ptab, const LuSide* side = nullptr, cudaEvent_t* upd_ev = nullptr);
+                       int2* ptab, const LuSide* side = nullptr, cudaEvent_t* upd_ev = nullptr,
+                       size_t img_bytes = 0);
+// complex128: digit-image scratch of one mode; img then holds img_bytes >= this, and
+// the modes are updated in groups of as many as fit
+size_t lu_image64_bytes(int n);
 size_t lu_ptab_elems(int n, int batch);
 // scratch bytes of the complex64 factorisation's operand images (the first
 // step's 64-row blocks of L21 and 64-column blocks of U12, 96 KB per pair)

@@ -7,9 +7,9 @@
 // factorisation itself is textbook right-looking blocked LU: panel
 // factorisation (pivot search, row swap, scaling, rank-1 updates inside the
 // panel), row swaps + unit-lower triangular solve for the block row, and a
-// tiled GEMM update of the trailing matrix (complex128: FP64 CUDA cores;
-// complex64: tcgen05 tensor cores on split operand images formed once per
-// step, tc_update.cuh).  complex128 leaves LAPACK getrf's row order (every
+// GEMM update of the trailing matrix on the tcgen05 tensor cores from split
+// operand images formed once per step (complex64: TF32 hi / lo, tc_update.cuh;
+// complex128: exact bf16 digit slices, tc_update64.cuh).  complex128 leaves LAPACK getrf's row order (every
 // column swapped) and a row permutation in piv; complex64 swaps only the
 // columns right of each panel, so L's column blocks keep their step's row
 // order, and the solves apply each step's interchanges (the per-step slot
@@ -28,6 +28,7 @@
 
 #include "internal.h"
 #include "tc_update.cuh"
+#include "tc_update64.cuh"
 
 namespace pmlbie {
 
@@ -675,67 +676,6 @@ __global__ void __launch_bounds__(256) swap_trsm_kernel(int n, int k0, int kb, i
     }
 }
 
-// Trailing update A22 -= L21 U12 (K = kb <= 32).  Output tile TILE x TILE per
-// CTA of 256 threads (16 x 16), TILE/16 x TILE/16 outputs per thread, operands
-// staged in static shared memory (< 48 KB): TILE = 64 for complex64, 32 for
-// complex128.
-template <typename T> struct GemmTile { static constexpr int v = sizeof(T) == 8 ? 64 : 32; };
-
-template <typename T>
-__global__ void gemm_update_kernel(int n, int k0, int kb, T* A) {
-    constexpr int TL = GemmTile<T>::v, RPT = TL / 16;
-    __shared__ T sL[kNB][TL + 1];
-    __shared__ T sU[kNB][TL + 1];
-    const int b = blockIdx.z;
-    T* a = A + (size_t)b * n * n;
-    const int r0 = k0 + kb + blockIdx.x * TL, c0 = k0 + kb + blockIdx.y * TL;
-    if (r0 >= n || c0 >= n) return;
-    const int tid = threadIdx.x;
-    for (int idx = tid; idx < kb * TL; idx += blockDim.x) {
-        int kk = idx / TL, i = idx % TL;
-        int r = r0 + i;
-        sL[kk][i] = r < n ? a[(size_t)(k0 + kk) * n + r] : Cx<T>::mk(0, 0);
-    }
-    for (int idx = tid; idx < kb * TL; idx += blockDim.x) {
-        int j = idx / kb, kk = idx % kb;
-        int c = c0 + j;
-        sU[kk][j] = c < n ? a[(size_t)c * n + k0 + kk] : Cx<T>::mk(0, 0);
-    }
-    __syncthreads();
-    const int tr = tid % 16, tc = tid / 16;
-    T acc[RPT][RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i)
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) acc[i][j] = Cx<T>::mk(0, 0);
-    for (int kk = 0; kk < kb; ++kk) {
-        T l[RPT], u[RPT];
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) l[i] = sL[kk][tr + 16 * i];
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) u[j] = sU[kk][tc + 16 * j];
-#pragma unroll
-        for (int i = 0; i < RPT; ++i)
-#pragma unroll
-            for (int j = 0; j < RPT; ++j) {
-                acc[i][j].x += l[i].x * u[j].x - l[i].y * u[j].y;
-                acc[i][j].y += l[i].x * u[j].y + l[i].y * u[j].x;
-            }
-    }
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-        int c = c0 + tc + 16 * j;
-        if (c >= n) continue;
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-            int r = r0 + tr + 16 * i;
-            if (r >= n) continue;
-            T* e = a + (size_t)c * n + r;
-            *e = sub(*e, acc[i][j]);
-        }
-    }
-}
-
 // Solve LU x = b for every matrix and rhs: the row permutation (gathered
 // while loading), then blocked unit-lower forward and upper backward
 // substitution.  One CTA (512 threads) per (matrix, group of up to kSolveR
@@ -1209,6 +1149,8 @@ cudaError_t lu_prepare() {
                     (e = allow_max_smem(panel_reg_kernel<1, kNB, 256>)) == cudaSuccess &&
                     (e = allow_max_smem(panel_reg_kernel<1, kNB, kPanelThreads>)) == cudaSuccess)
                     e = allow_max_smem(panel_reg_kernel<2, kNB / 2, kPanelThreads>);
+            } else {
+                e = allow_max_smem(tcu::update64_kernel);
             }
         }
         err = e;
@@ -1271,9 +1213,17 @@ size_t lu_image_bytes(int n, int batch) {
     return (size_t)batch * nblk * (tcu::kAImg + tcu::kBImg);
 }
 
+// complex128: per mode the first step's digit images and 2 n exponents
+size_t lu_image64_bytes(int n) {
+    if (n <= kNB) return 0;
+    const int rem = n - kNB;
+    return (size_t)tcu::row_blocks64(rem) * tcu::kAImg64 + (size_t)tcu::col_blocks64(rem) * tcu::kBImg64 +
+           sizeof(int) * 2 * (size_t)n;
+}
+
 template <typename T>
 cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t s, unsigned char* img,
-                       int2* ptab, const LuSide* side, cudaEvent_t* upd_ev) {
+                       int2* ptab, const LuSide* side, cudaEvent_t* upd_ev, size_t img_bytes) {
     cudaError_t pe = lu_prepare<T>();
     if (pe != cudaSuccess) return pe;
     if constexpr (sizeof(T) == 8) {
@@ -1285,15 +1235,19 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
     // persistent update
     CUtensorMap tmA;
     int sms = 0;
-    if constexpr (sizeof(T) == 8) {
-        if (n > kNB) {
-            if (!img || (reinterpret_cast<uintptr_t>(img) & 15)) return cudaErrorInvalidValue;
-            cudaError_t e = trailing_tensor_map(&tmA, reinterpret_cast<float2*>(A), n, batch);
-            int dev = 0;
-            if (e == cudaSuccess) e = cudaGetDevice(&dev);
-            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return e;
+    int group = 0;       // complex128: modes whose digit images fit in img at once
+    if (n > kNB) {
+        if (!img || (reinterpret_cast<uintptr_t>(img) & 15)) return cudaErrorInvalidValue;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if constexpr (sizeof(T) == 8) {
+            if (e == cudaSuccess) e = trailing_tensor_map(&tmA, reinterpret_cast<float2*>(A), n, batch);
+        } else {
+            group = (int)std::min<size_t>(batch, img_bytes / lu_image64_bytes(n));
+            if (group < 1) return cudaErrorInvalidValue;
         }
+        if (e != cudaSuccess) return e;
     }
     for (int k0 = 0; k0 < n; k0 += kNB) {
         int kb = std::min(kNB, n - k0);
@@ -1366,12 +1320,21 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
                 const int grid = (int)std::min<long long>(units, sms);
                 tcu::update_kernel<<<grid, tcu::kPipeThreads, tcu::kPipeSmem, s>>>(tmA, k0, kb, nblk, batch, img,
                                                                                    bimg, info);
+                count_launch();
             } else {
-                constexpr int TL = GemmTile<T>::v;
-                dim3 g2((rem + TL - 1) / TL, (rem + TL - 1) / TL, batch);
-                gemm_update_kernel<T><<<g2, 256, 0, s>>>(n, k0, kb, A);
+                // complex128: digit images and update, as many modes at a time as the
+                // scratch holds images of (the exponents behind the images)
+                const int nra = tcu::row_blocks64(rem), nca = tcu::col_blocks64(rem);
+                int* expo = reinterpret_cast<int*>(img + (size_t)group * (lu_image64_bytes(n) - sizeof(int) * 2 * (size_t)n));
+                for (int b0 = 0; b0 < batch; b0 += group) {
+                    const int g = std::min(group, batch - b0);
+                    double2* Ab = reinterpret_cast<double2*>(A) + (size_t)b0 * n * n;
+                    tcu::operand_image64_kernel<<<dim3(nra + nca, g), 256, 0, s>>>(n, k0, nra, Ab, img, nca, expo);
+                    tcu::update64_kernel<<<std::min(g * nra, sms), tcu::kUpd64Threads, tcu::kUpd64Smem, s>>>(
+                        n, k0, g, Ab, img, expo, info + b0);
+                    count_launch(2);
+                }
             }
-            count_launch();
             if (upd_ev && (ee = record_update_event(upd_ev[2 * (k0 / kNB) + 1], s)) != cudaSuccess) return ee;
         }
     }
@@ -1414,9 +1377,9 @@ cudaError_t batched_lu_solve(int n, int batch, int nrhs, const TF* LU, const int
 template cudaError_t lu_prepare<double2>();
 template cudaError_t lu_prepare<float2>();
 template cudaError_t batched_lu<double2>(int, int, double2*, int*, int*, cudaStream_t, unsigned char*, int2*,
-                                          const LuSide*, cudaEvent_t*);
+                                          const LuSide*, cudaEvent_t*, size_t);
 template cudaError_t batched_lu<float2>(int, int, float2*, int*, int*, cudaStream_t, unsigned char*, int2*,
-                                         const LuSide*, cudaEvent_t*);
+                                         const LuSide*, cudaEvent_t*, size_t);
 template cudaError_t batched_lu_solve<double2, double2>(int, int, int, const double2*, const int*, double2*,
                                                         cudaStream_t, const int*, const double2*, const int2*);
 template cudaError_t batched_lu_solve<float2, float2>(int, int, int, const float2*, const int*, float2*,
