@@ -339,9 +339,8 @@ def run_ours(args, rank, world):
     epp = entries_per_problem(w)
     value = job_value(world, epp, ms)
     pk = peaks()
-    stages = {"far_kernel_ff": last.ms_far, "near_laplace_kernel": last.ms_near_laplace,
-              "near_modes_kernel_ff": last.ms_near_ff,
-              "near_modes_kernel_fp64_pml": last.ms_near - last.ms_near_laplace - last.ms_near_ff,
+    stages = {"far_kernel": last.ms_far, "near_laplace_kernel": last.ms_near_laplace,
+              "near_modes_kernel": last.ms_near - last.ms_near_laplace,
               "assemble": last.ms_assemble, "lu_fp32": last.ms_lu, "solve_refine": last.ms_solve}
     clocks = clk.summary()
     roof = near_roofline(w, last, pk, clocks, ncounts, pipes)
@@ -351,7 +350,7 @@ def run_ours(args, rank, world):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": max(args.warmup, 3), "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "float-float (FP32 pairs) sampling/FFT, FP64 PML close pairs and Laplace modes, c64 LU, c128 refinement",
+        "dtype": "FP64 / 64-bit fixed-point sampling and DFTs, FP64 Laplace modes, c64 LU, c128 refinement",
         "data": "synthetic",
         "config": {"workload": "two-layer bump, N=%d M=%d (%d modes), k1=%gpi k2=%gpi, PML a1=2.5 T=1 S=3, "
                                "1 plane wave at 30 deg, mixed precision" % (w["N"], w["M"], w["M"] // 2,
@@ -364,7 +363,7 @@ def run_ours(args, rank, world):
         "far_pairs": last.far_pairs, "far_pairs_sampled": last.far_pairs_sampled,
         "far_pairs_per_cta": last.far_pairs_per_cta,
         "stages_ms": {k: round(v, 4) for k, v in stages.items()},
-        "stages_note": ("far_kernel_ff runs beside the close-pair kernels (near_*, on a high-priority stream): "
+        "stages_note": ("far_kernel runs beside the close-pair kernels (near_*, on a high-priority stream): "
                         "their times overlap; the others are sequential"),
         "mode_chunks": chunks,
         "refine_iters": last.refine_iters, "refine_residual": last.residual,
@@ -727,47 +726,39 @@ def profile_traffic(path, src_name, units):
     return float(vals["dram_bytes_per_unit"]) * units
 
 
-def fp64_peak(pk, clk, pipes):
-    """Measured FP64 FMA TFLOP/s (pmlbie_selftest_peak), else derived."""
-    if pipes and pipes.get("fp64_fma_tflops"):
-        return pipes["fp64_fma_tflops"], "measured: FP64 FMA probe on this GPU (pmlbie_selftest_peak)"
-    mhz = clk.get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
-    return 152 * 2 * 2 * mhz * 1e6 / 1e12, "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x %.0f MHz" % mhz
-
-
 def near_roofline(w, rep, pk, clk, counts, pipes=None):
-    """Roofline of the close-pair modes kernel for the pairs with a PML point
-    (near_modes_kernel<0>, FP64 in both paths, the longest single kernel of
-    the mixed step; one launch per mode chunk): FP64-ALU bound.  achieved =
-    the algorithmic FP64 flops of those pairs (near_flops_per_launch) / the
-    kernel's event time; peak = the measured FP64 FMA rate."""
+    """Roofline of the close-pair modes kernel (all close pairs, one launch per
+    mode chunk), the HBM view: algorithmic bytes = per pair the 2 M Laplace
+    modes read and the 4 kernels' modes written.  The kernel is bounded by
+    the barriers and the integer issue of its fixed-point transforms, so this
+    fraction is low by construction; `flops_per_launch` counts the FP64 work
+    that its samples, transforms and products stand for."""
     M = w["M"]
-    peak, note = fp64_peak(pk, clk, pipes)
     launches = max(1, rep.chunks)
-    npml = counts[1]
+    packed, npml, plain = counts[:3]
     couples = counts[3] if len(counts) > 3 else 0
-    flops = near_flops_per_launch(M, rep.chunk_modes, 0, npml, 0, couples)
-    ms1 = (rep.ms_near - rep.ms_near_laplace - rep.ms_near_ff) / launches
-    ach = flops / (ms1 / 1e3) / 1e12
-    traffic = profile_traffic("near_modes_kernel_pml_n256_m128.md", "kernels.cu", npml)
-    return {"kernel": "near_modes_kernel<0> (close pairs with a PML point: Sec. 4.3 substitution split, even DFTs, "
-                      "FFT convolution with the exact Laplace modes, FP64)",
-            "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-            "traffic": traffic, "flops_per_launch": flops, "ms_per_launch": ms1, "launches_per_step": launches,
-            "pairs": npml, "pml_couples": couples,
-            "algorithmic_bytes": float(npml) * (2 * M + 4 * rep.chunk_modes) * 16,
-            "peak_note": note,
-            "traffic_note": ("ncu dram read+write per PML pair (profiles/near_modes_kernel_pml_n256_m128.md) x pairs"
-                             if traffic else "null: no ncu capture of the current kernels.cu")}
+    n = packed + npml + plain
+    ms1 = (rep.ms_near - rep.ms_near_laplace) / launches
+    nbytes = float(n) * (2 * M + 4 * rep.chunk_modes) * 16
+    hbm = pk.get("hbm_gbs", 6794.1)
+    ach = nbytes / (ms1 / 1e3) / 1e9
+    return {"kernel": "near_modes_kernel (close pairs: split samples, even DFTs in block fixed point, convolution with "
+                      "the exact Laplace modes)",
+            "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": None,
+            "flops_per_launch": near_flops_per_launch(M, rep.chunk_modes, packed, npml, plain, couples),
+            "ms_per_launch": ms1, "launches_per_step": launches, "pairs": n, "pml_couples": couples,
+            "algorithmic_bytes": nbytes, "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)",
+            "time_note": "span in the step, where it runs beside the far-pair kernel",
+            "traffic_note": "null: no ncu capture of the current kernels.cu"}
 
 
 def roofline(w, rep, pk, clk, pipes=None):
-    """Roofline of the far-pair kernel of the mixed path (far_kernel_ff:
-    float-float sampling, transforms and block scatter), the HBM view of
+    """Roofline of the far-pair kernel (sampling, fixed-point transforms and
+    block scatter), the HBM view of
     SURVEY-style stage a3: algorithmic bytes = the 4 N^2 (M/2) complex128
     entries it writes per launch, against the measured HBM copy bandwidth.
-    The kernel is bounded by instruction issue on its FP32 / integer pipes
-    (ncu summary in profiles/), so this fraction is low by construction."""
+    The kernel is bounded by its FP64 sampling and the integer issue of its
+    transforms, so this fraction is low by construction."""
     M = w["M"]
     launches = max(1, rep.chunks)
     # the kernel alone (its autotuning launch): in the solve it runs beside the
@@ -777,18 +768,16 @@ def roofline(w, rep, pk, clk, pipes=None):
     wbytes = 4.0 * w["N"] ** 2 * rep.chunk_modes * 16
     hbm = pk.get("hbm_gbs", 6794.1)
     ach = wbytes / (ms1 / 1e3) / 1e9
-    traffic = profile_traffic("far_kernel_ff_n256_m128.md", "kernels_ff.cu", 4.0 * w["N"] ** 2 * rep.chunk_modes)
-    return {"kernel": "far_kernel_ff (S~, K~ sampling of both media per unordered pair + 4 even DFTs + block scatter "
-                      "of both orientations, float-float)",
+    traffic = None
+    return {"kernel": "far_kernel (S~, K~ sampling of both media per unordered pair + 4 even DFTs in block fixed point "
+                      "+ block scatter of both orientations)",
             "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": traffic,
             "ms_per_launch": ms1, "launches_per_step": launches, "algorithmic_bytes": wbytes,
             "time_note": ("the kernel alone: its autotuning launch of the chosen CTA size (CUDA events); in the "
                           "step it runs beside the close-pair kernels" if alone > 0 else
                           "span of the launch in the step (runs beside the close-pair kernels)"),
             "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)",
-            "traffic_note": ("ncu dram read+write per entry written (profiles/far_kernel_ff_n256_m128.md) x "
-                             "4 N^2 (M/2) entries"
-                             if traffic else "null: no ncu capture of the current kernels_ff.cu")}
+            "traffic_note": "null: no ncu capture of the current kernels.cu"}
 
 
 def lu_update_roofline(w, rep, pk):
@@ -855,7 +844,7 @@ def stage_rooflines(w, rep, pk, pipes=None):
                             "TF32 peak measured by the tcgen05 probe (pmlbie_selftest_peak), HBM measured copy"},
         "block_writes": {"bytes": wr, "ms": far_ms, "gbs": wr / s_far / 1e9,
                          "frac_hbm": wr / s_far / 1e9 / hbm,
-                         "note": "fused into the far kernel, bounded by its FP32 / integer instruction issue"},
+                         "note": "fused into the far kernel, bounded by its FP64 sampling and integer instruction issue"},
     }
 
 

@@ -122,14 +122,14 @@ typedef struct {
                                      sampling and one set of transforms serves both (l, m) and
                                      (m, l) (S~ is symmetric, K~ differs by its normal factor) */
     int      far_pairs_sampled_physical;  /* of those, pairs of two physical nodes           */
-    double   ms_near_ff;          /* mixed: device time of the float-float close-pair modes kernel
-                                     (pairs without a PML point; part of ms_near) (ms) */
+    double   ms_near_ff;          /* mixed: device time of the close-pair modes kernel (all close
+                                     pairs; ms_near - ms_near_laplace) (ms)            */
     double   ms_lu_update;        /* device time of the LU's trailing updates, summed (part of
                                      ms_lu; an event pair around each step's operand-image and
                                      tensor-core update launches) (ms) */
     int      lu_update_launches;  /* trailing updates (steps with a trailing matrix) of those
                                      factorisations, each timed by one event pair             */
-    double   ms_far_alone;        /* mixed: device time of the float-float far-pair kernel run
+    double   ms_far_alone;        /* mixed: device time of the far-pair kernel run
                                      alone (its autotuning launch of the chosen CTA size, on the
                                      first solve of this shape; 0 when not tuned) (ms)          */
 } pmlbie_report;
@@ -242,16 +242,11 @@ size_t pmlbie_workspace_bytes(const pmlbie_problem* prob, int precision, int n_r
 int  pmlbie_modal_kernels(pmlbie_problem* prob, int mode_lo, int mode_hi, void* dev_out,
                           void* stream);
 
-/* pmlbie_modal_kernels in the arithmetic of a solve's precision: PMLBIE_FP64
- * as pmlbie_modal_kernels; PMLBIE_MIXED as the mixed solve builds its
- * matrices: the far pairs' samples, transforms and scatter, and the close
- * pairs' split samples, transforms and convolution, in float-float (pairs
- * of FP32 numbers, ~48-bit significands, on the FP32 pipe; relative rounding
- * ~1e-14 of a pair's samples, growing with |q| = omega |dr| as |q| 2^-47),
- * with the exact modal Laplace kernels of the split (Sec. 4.1, the
- * near-singular part) in FP64.  Problems whose phases |q| reach the
- * float-float sin / cos range (~780), and the diagnostic exact split
- * (subst_off), take the FP64 kernels in both precisions.
+/* pmlbie_modal_kernels as a solve of the given precision builds them.  Both
+ * precisions take the same kernels: phases, sines, exponentials and the even
+ * DFTs in 64-bit fixed point (57 bits and more of the largest sample of a
+ * pair), the rest and the exact modal Laplace kernels of the split (Sec. 4.1,
+ * the near-singular part) in FP64.
  * Errors as pmlbie_modal_kernels; EINVAL for another precision. */
 int  pmlbie_modal_kernels_ex(pmlbie_problem* prob, int precision, int mode_lo, int mode_hi, void* dev_out,
                              void* stream);
@@ -259,7 +254,7 @@ int  pmlbie_modal_kernels_ex(pmlbie_problem* prob, int precision, int mode_lo, i
 /* Split modal kernels of every close pair (Sec. 4.1 kernel splitting; Sec. 4.3
  * substitution on PML pairs), in the close-pair list's order (pmlbie_near_pairs:
  * grid pairs, then Alpert correction pairs -- the values the assembly adds
- * with the Lagrange stencils), in the arithmetic of `precision` as
+ * with the Lagrange stencils), for `precision` as
  * pmlbie_modal_kernels_ex.  Output: dev_out, caller-owned device buffer of
  * (n_grid_near + n_corr) * 4 * (mode_hi - mode_lo) complex128 laid out
  * [pair][kernel][mode], kernel as in pmlbie_modal_kernels; no quadrature
@@ -296,14 +291,13 @@ int  pmlbie_modal_kernels_noalloc(pmlbie_problem* prob, int mode_lo, int mode_hi
  * Outputs (caller-owned device buffers, complex128, [mode][node][rhs], M/2
  * modes): u1 = u^{s,1}_n, phi1 = |r'| d_nu_c u^{s,1}_n, u2, phi2 (the same for
  * the lower medium, d_nu with the same nu).  Any output may be NULL.
- * Mixed precision: modal kernels in float-float arithmetic on the FP32 pipe
- * (as pmlbie_modal_kernels_ex with PMLBIE_MIXED) stored as complex128
+ * Mixed precision: modal kernels as for PMLBIE_FP64, stored as complex128
  * matrices, complex64 LU (tensor-core trailing updates), iterative
  * refinement with FP64 residuals of those matrices until, for
  * every mode and right-hand side, the relative residual is <= 1e-13, or the
- * normwise backward error |B - A x| / (|A|_F |x| + |B|) is <= 1e-16, or it is
- * <= 1e-14 and no longer decreasing (the FP64 floor); modes
- * whose refinement stalls (condition number x FP32 LU error near 1 or above)
+ * normwise backward error |B - A x| / (|A|_F |x| + |B|) is <= 1e-16, or it has
+ * stopped decreasing (the FP64 floor) at <= 4e-16 in refinement or <= 1e-14 in
+ * GMRES; modes whose refinement stalls above that (condition number x FP32 LU error near 1 or above)
  * are restarted and solved by flexible GMRES in FP64 preconditioned by the
  * same LU.  Errors: EINVAL, ENOMEM, ECUDA, ESINGULAR, ENOCONVERGE (mixed: a
  * mode missed both tolerances after the iteration caps; outputs still

@@ -113,14 +113,14 @@ int ensure_device(pmlbie_problem* prob) {
         (rc = upload(D.corr_w, H.corr_w)))
         return rc;
     const int M = prob->P.M;
-    std::vector<double2> cs(M / 2 + 1), tw2(2 * M);
-    for (int e = 0; e < 2 * M; ++e)
-        tw2[e] = make_double2(std::cos(kPi * e / M), -std::sin(kPi * e / M));
+    std::vector<double2> cs(M / 2 + 1);
     for (int j = 0; j <= M / 2; ++j) {
         double s = std::sin(kPi * j / M);
         cs[j] = make_double2(s * s, std::cos(2.0 * kPi * j / M));
     }
-    if ((rc = upload(D.cos_tab, cs)) || (rc = upload(D.twid2, tw2)) || (rc = upload(D.twid_fx, fx_twiddles(M)))) return rc;
+    if ((rc = upload(D.cos_tab, cs)) || (rc = upload(D.twid_fx, fx_twiddles(M))) ||
+        (rc = upload(D.trig_fx, fx_trig_table())) || (rc = upload(D.exp_fx, fx_exp_table())))
+        return rc;
     {
         const int nr = rec_table_len(M);
         std::vector<double2> up(nr), dn(nr);
@@ -131,24 +131,8 @@ int ensure_device(pmlbie_problem* prob) {
         }
         if ((rc = upload(D.rec_up, up)) || (rc = upload(D.rec_dn, dn))) return rc;
     }
-    {
-        std::vector<float4> ftw, ftw2, fcs, ftrig;
-        std::vector<float2> fexp, fwu(H.Wu.size()), fwp(H.Wphi.size());
-        ff_tables(M, ftw, ftw2, fcs, fexp, ftrig);
-        auto f2 = [](double x) {
-            const float hi = (float)x;
-            return make_float2(hi, (float)(x - (double)hi));
-        };
-        const double c4 = 0.5 / M;
-        for (size_t m = 0; m < fwu.size(); ++m) {
-            fwu[m] = f2(H.h * H.Wu[m] * c4);
-            fwp[m] = f2(H.h * H.Wphi[m] * c4);
-        }
-        if ((rc = upload(D.twid_ff, ftw)) || (rc = upload(D.twid2_ff, ftw2)) || (rc = upload(D.cos_ff, fcs)) ||
-            (rc = upload(D.exp_ff, fexp)) || (rc = upload(D.trig_ff, ftrig)) || (rc = upload(D.wuc_ff, fwu)) ||
-            (rc = upload(D.wpc_ff, fwp)))
-            return rc;
-    }
+    D.ph[0] = fx_phase(prob->P.k1);
+    D.ph[1] = fx_phase(prob->P.k2);
     if ((rc = upload(ex->nu_r, H.nu_r)) || (rc = upload(ex->nu_z, H.nu_z)) || (rc = upload(ex->speed, H.speed)))
         return rc;
     ex->ready = true;
@@ -158,9 +142,8 @@ int ensure_device(pmlbie_problem* prob) {
 void free_device(pmlbie_problem* prob) {
     DeviceTables& D = prob->D;
     void* ptrs[] = {D.rho, D.z, D.I, D.Wu, D.Wphi, D.rho_t, D.nuc_r, D.nuc_z, D.bk, D.off, D.cls, D.near, D.near_lead,
-                    D.corr_target, D.corr_m, D.corr_coef, D.Da, D.Db, D.cos_tab, D.twid2, D.twid_fx,
-                    D.corr_start, D.corr_cmin, D.corr_w, D.rec_up, D.rec_dn, D.twid_ff, D.twid2_ff, D.cos_ff, D.exp_ff, D.trig_ff, D.wuc_ff,
-                    D.wpc_ff};
+                    D.corr_target, D.corr_m, D.corr_coef, D.Da, D.Db, D.cos_tab, D.twid_fx, D.trig_fx, D.exp_fx,
+                    D.corr_start, D.corr_cmin, D.corr_w, D.rec_up, D.rec_dn};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     pmlbie_dev_extra* ex = extra_of(prob);
@@ -223,6 +206,11 @@ constexpr int kGmresCycles = 10;     // FGMRES restarts at most
 constexpr double kTolRel = 1e-13;
 constexpr double kTolBwd = 1e-16;
 constexpr double kTolFloor = 1e-14;
+// a refinement that no longer halves its backward error is at the FP64 floor only below
+// kTolFloorIr: above it the FP32 factors contract too slowly (a factor near 1 a step
+// looks the same), and FGMRES takes the mode over, which stops on kTolFloor when a cycle
+// gains less than 10 %
+constexpr double kTolFloorIr = 4e-16;
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -249,7 +237,7 @@ Workspace plan(const pmlbie_problem* prob, int precision, int nrhs, int nmodes, 
         w.R = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
     }
     const size_t near0 = off;
-    w.zd = (double2*)take(near_zd_bytes(std::max<size_t>(np, 1), M, true));
+    w.zd = (double2*)take(near_zd_bytes(std::max<size_t>(np, 1), M));
     w.nout = (double2*)take(sizeof(double2) * std::max<size_t>(np, 1) * 4 * nm);
     w.near_bytes = off - near0;
     w.b1 = (double2*)take(sizeof(double2) * nm * N * nrhs);
@@ -297,18 +285,13 @@ void fresnel(double w1, double w2, double phi, double* out6) {
     out6[5] = ks.imag();
 }
 
-// modal kernels + assembly into w.A for modes [lo, hi).  The far kernel and
-// the close-pair chain (Laplace modes, float-float close pairs, FP64 PML close
-// pairs) are independent until the assembly and load different pipes (the
-// mixed path's far kernel the FP32 / integer issue, the PML pairs the FP64
-// pipe): the chain runs on a high-priority stream forked from s, so that its
-// CTAs are dispatched first and the far kernel's fill the SMs it leaves
-// (mostly during the latency-bound Laplace-mode kernel); the assembly waits
-// for both.  ev[0] = fork, ev[1] = far kernel done (on s), ev[4] / ev[5] =
-// Laplace modes / float-float close pairs done and ev[2] = chain done (on the
-// chain's stream), ev[6] = join, ev[3] = assembly done.
-// (the mixed path samples the far pairs in float-float arithmetic when the
-// problem's phases fit its range, else in FP64)
+// modal kernels + assembly into w.A for modes [lo, hi), the same for both precisions.
+// The far kernel and the close-pair chain (Laplace modes, then the close pairs' modes)
+// are independent until the assembly: the chain runs on a high-priority stream forked
+// from s, so that its CTAs are dispatched first and the far kernel's fill the SMs it
+// leaves (mostly during the latency-bound Laplace-mode kernel); the assembly waits for
+// both.  ev[0] = fork, ev[1] = far kernel done (on s), ev[4] = Laplace modes done and
+// ev[2] = chain done (on the chain's stream), ev[6] = join, ev[3] = assembly done.
 int build_system(pmlbie_problem* prob, int precision, Workspace& w, int lo, int hi, cudaStream_t s,
                  cudaEvent_t* ev) {
     FarLaunch fl{lo, hi, w.A, nullptr, true};
@@ -320,15 +303,14 @@ int build_system(pmlbie_problem* prob, int precision, Workspace& w, int lo, int 
         PMLBIE_CUDA_TRY(cudaEventCreateWithFlags(&ex->fork, cudaEventDisableTiming));
         PMLBIE_CUDA_TRY(cudaEventCreateWithFlags(&ex->join, cudaEventDisableTiming));
     }
-    const bool ff = precision == PMLBIE_MIXED && far_ff_supported(prob);
     cudaStream_t sn = ex->near_stream;
     PMLBIE_CUDA_TRY(cudaEventRecord(ev[0], s));
     PMLBIE_CUDA_TRY(cudaEventRecord(ex->fork, s));
     PMLBIE_CUDA_TRY(cudaStreamWaitEvent(sn, ex->fork, 0));
     // the far kernel first: its CTAs take the SMs the Laplace-mode kernel leaves idle
-    PMLBIE_CUDA_TRY(ff ? launch_far_ff(prob, fl, s) : launch_far(prob, fl, s));
+    PMLBIE_CUDA_TRY(launch_far(prob, fl, s));
     PMLBIE_CUDA_TRY(cudaEventRecord(ev[1], s));
-    PMLBIE_CUDA_TRY(launch_near(prob, lo, hi, w.zd, w.nout, sn, ev[4], ff, ev[5]));
+    PMLBIE_CUDA_TRY(launch_near(prob, lo, hi, w.zd, w.nout, sn, ev[4]));
     PMLBIE_CUDA_TRY(cudaEventRecord(ev[2], sn));
     PMLBIE_CUDA_TRY(cudaEventRecord(ex->join, sn));
     PMLBIE_CUDA_TRY(cudaStreamWaitEvent(s, ex->join, 0));
@@ -508,9 +490,8 @@ int pmlbie_close_pair_kernels(pmlbie_problem* prob, int precision, int mode_lo, 
     cudaStream_t s = (cudaStream_t)stream;
     const size_t np = std::max<size_t>(prob->H.near.size(), 1);
     double2* zd = nullptr;
-    PMLBIE_CUDA_TRY(cudaMalloc(&zd, near_zd_bytes(np, prob->P.M, true)));
-    cudaError_t e = launch_near(prob, mode_lo, mode_hi, zd, (double2*)dev_out, s, nullptr,
-                                precision == PMLBIE_MIXED && far_ff_supported(prob));
+    PMLBIE_CUDA_TRY(cudaMalloc(&zd, near_zd_bytes(np, prob->P.M)));
+    cudaError_t e = launch_near(prob, mode_lo, mode_hi, zd, (double2*)dev_out, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(zd);
     if (e != cudaSuccess) return fail(PMLBIE_ECUDA, std::string("close-pair kernels: ") + cudaGetErrorString(e));
@@ -529,16 +510,15 @@ int pmlbie_modal_kernels_ex(pmlbie_problem* prob, int precision, int mode_lo, in
     const size_t np = std::max<size_t>(prob->H.near.size(), 1);
     const int M = prob->P.M;
     double2 *zd = nullptr, *nout = nullptr;
-    PMLBIE_CUDA_TRY(cudaMalloc(&zd, near_zd_bytes(np, M, true)));
+    PMLBIE_CUDA_TRY(cudaMalloc(&zd, near_zd_bytes(np, M)));
     if (cudaMalloc(&nout, sizeof(double2) * np * 4 * (mode_hi - mode_lo)) != cudaSuccess) {
         cudaFree(zd);
         return fail(PMLBIE_ENOMEM, "scratch allocation failed");
     }
     FarLaunch fl{mode_lo, mode_hi, nullptr, (double2*)dev_out, true};
-    cudaError_t e = precision == PMLBIE_MIXED && far_ff_supported(prob) ? launch_far_ff(prob, fl, s)
-                                                                        : launch_far(prob, fl, s);
+    cudaError_t e = launch_far(prob, fl, s);
     if (e == cudaSuccess)
-        e = launch_near(prob, mode_lo, mode_hi, zd, nout, s, nullptr, precision == PMLBIE_MIXED && far_ff_supported(prob));
+        e = launch_near(prob, mode_lo, mode_hi, zd, nout, s);
     if (e == cudaSuccess) e = launch_near_to_raw(prob, mode_lo, mode_hi, nout, (double2*)dev_out, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(zd);
@@ -794,7 +774,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
                     mres[mo] = worst;
                     mbwd[mo] = wbwd;
                     const bool stalled = iters >= 2 && !(wbwd < 0.5 * prev[mo]);
-                    if (ok || (stalled && wbwd <= kTolFloor)) {
+                    if (ok || (stalled && wbwd <= kTolFloorIr)) {
                         act[mo] = 0;     // done, or at the FP64 floor
                     } else if (stalled) {
                         act[mo] = 0;     // contraction too slow or divergent: FGMRES
@@ -880,9 +860,6 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
     cudaEventElapsedTime(&f[1], sev[0], sev[2]);
     cudaEventElapsedTime(&f[2], sev[6], sev[3]);
     cudaEventElapsedTime(&fl, sev[0], sev[4]);
-    float fff = 0.f;
-    cudaEventElapsedTime(&fff, sev[4], sev[5]);
-    st.ms_near_ff += fff;
     for (int k = 0; k < ex->upd_pairs; ++k) {
         float tu = 0.f;
         if (cudaEventElapsedTime(&tu, ex->upd_ev[2 * k], ex->upd_ev[2 * k + 1]) == cudaSuccess) {
@@ -898,6 +875,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
     st.ms_near += f[1];
     st.ms_assemble += f[2];
     st.ms_near_laplace += fl;
+    if (precision == PMLBIE_MIXED) st.ms_near_ff += f[1] - fl;
     st.iters = std::max(st.iters, iters);
     st.resid = std::max(st.resid, resid);
     st.bwd = std::max(st.bwd, bwd);
@@ -1107,8 +1085,7 @@ int pmlbie_solve_ex(pmlbie_problem* prob, const pmlbie_solve_opts* o, void* dev_
         rep->backward_error = st.bwd;
         rep->lu_graph_replays = g_lu_graph_replays;
         rep->far_pairs_per_cta = g_far_pairs_per_cta;
-        rep->ms_far_alone =
-            precision == PMLBIE_MIXED && far_ff_supported(prob) ? far_ff_alone_ms(prob, chunk, false) : 0.0;
+        rep->ms_far_alone = precision == PMLBIE_MIXED ? far_alone_ms(prob, chunk, false) : 0.0;
     }
     if (precision == PMLBIE_MIXED && st.unconverged)
         return fail(PMLBIE_ENOCONVERGE, "refinement missed its tolerance: residual " + std::to_string(st.resid) +

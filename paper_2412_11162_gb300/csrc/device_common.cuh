@@ -1,5 +1,5 @@
-// Device helpers shared by the FP64 kernels (kernels.cu) and the
-// float-float kernels of the mixed path (kernels_ff.cu): complex128
+// Device helpers shared by the modal kernels (kernels.cu) and the
+// float-float self-test (kernels_ff.cu): complex128
 // arithmetic and the geometry of a grid node pair.
 #pragma once
 

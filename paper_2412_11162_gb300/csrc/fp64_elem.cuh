@@ -1,6 +1,5 @@
-// FP64 elementary functions of the sampling loops and the Taylor-polynomial
-// evaluation of the Sec. 4.3 substitution, shared by the FP64 kernels
-// (kernels.cu) and the mixed path's kernels (kernels_ff.cu).
+// FP64 elementary functions of the sampling loops (diagnostic exact split,
+// self-test).
 #pragma once
 
 #include "device_common.cuh"
@@ -114,29 +113,6 @@ __device__ __forceinline__ double2 fcexpi(double2 q) {
     fsincos(q.x, &s, &c);
     const double m = fexp(-q.y);
     return c2(m * c, m * s);
-}
-
-// Principal square root R of z (z not 0) and 1/R = conj(R)/|z|, from two
-// reciprocal square roots.  Cancellation-free on both half planes.
-__device__ __forceinline__ void fcsqrt_rcp(double2 z, double2& R, double2& iR) {
-    const double m2 = fma(z.x, z.x, z.y * z.y);
-    const double ir = frsqrt(m2);                  // 1/|z|
-    const double r = m2 * ir;                      // |z|
-    const double u = 0.5 * (r + fabs(z.x));
-    const double it = frsqrt(u);
-    const double t = u * it;                       // sqrt((|z| + |Re z|)/2)
-    const double s = 0.5 * z.y * it;               // Im z / (2 t)
-    R = z.x >= 0.0 ? c2(t, s) : c2(fabs(s), copysign(t, z.y));
-    iR = c2(R.x * ir, -R.y * ir);
-}
-
-// sum_{k = k0}^{L} c_k q^{k - k0} by Horner, L <= 7 (unrolled: static indices)
-__device__ __forceinline__ double2 cpoly_from(const double2 (&c)[8], int k0, int L, double2 q) {
-    double2 r = c2(0.0, 0.0);
-#pragma unroll
-    for (int k = 7; k >= 0; --k)
-        if (k >= k0 && k <= L) r = cadd(cmul(r, q), c[k]);
-    return r;
 }
 
 }  // namespace

@@ -282,7 +282,7 @@ __device__ __forceinline__ int fx_fft(longlong2* x, int K, int T, const int4* tw
 // sc: the quantised sequence's scale; sum |y| <= 2 sum |x|.  Returns the exponent of
 // the result, |X| <= 2^60 (1 + 1/K).  tw[e tws] = e^{-2 pi i e / L}.
 template <int NB>
-__device__ __noinline__ int fx_even_dft(longlong2* x, FxScale sc, int K, const int4* tw, int tws, int lane) {
+__device__ __forceinline__ int fx_even_dft(longlong2* x, FxScale sc, int K, const int4* tw, int tws, int lane) {
     const int H = K / 2;
     longlong2 hi = fx2(0, 0);
     int2 lo = make_int2(0, 0);

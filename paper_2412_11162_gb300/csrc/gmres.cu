@@ -350,8 +350,8 @@ int gmres_refine(int n, int batch, int nrhs, const double2* A, const float2* LU3
                 hist[t].clear();
             }
             // after a cycle: also done at the FP64 floor (backward error below
-            // tol_floor that the last cycle did not halve)
-            const bool floor = cyc > 0 && wbwd <= tol_floor && wbwd >= 0.5 * mode_bwd[b];
+            // tol_floor that the last cycle did not lower by 10 %)
+            const bool floor = cyc > 0 && wbwd <= tol_floor && wbwd >= 0.9 * mode_bwd[b];
             mode_res[b] = worst;
             mode_bwd[b] = wbwd;
             if (ok || floor) act[b] = 0;

@@ -435,6 +435,43 @@ std::vector<int4> fx_twiddles(int M) {
     return tw;
 }
 
+std::vector<int4> fx_trig_table() {
+    std::vector<int4> t = fx_twiddles(512);      // e^{-2 pi i j / 1024}
+    t.resize(kTrigFx);
+    for (int4& v : t) {
+        const int64_t s = -(((int64_t)v.z << 32) + v.w);
+        const int l = (int)(uint32_t)(uint64_t)s;
+        v.z = (int)((s - l) >> 32);
+        v.w = l;
+    }
+    return t;
+}
+
+std::vector<int2> fx_exp_table() {
+    std::vector<int2> t(kExpFx);
+    const Dd ln2{0.6931471805599453, 2.3190468138462996e-17};
+    for (int j = 0; j < kExpFx; ++j) {
+        const Dd x = dd_div(dd_mul(ln2, Dd{(double)j, 0.0}), 256.0);
+        Dd e{1.0, 0.0}, term = e;
+        for (int k = 1; k <= 26; ++k) {
+            term = dd_div(dd_mul(term, x), k);
+            e = dd_add(e, term);
+        }
+        const int64_t q = dd_q62(Dd{0.5 * e.h, 0.5 * e.l});      // Q61
+        const int l = (int)(uint32_t)(uint64_t)q;
+        t[j] = make_int2((int)((q - l) >> 32), l);
+    }
+    return t;
+}
+
+FxPhase fx_phase(double w) {
+    const Dd p = dd_mul(Dd{w, 0.0}, Dd{0.15915494309189535, -9.839338337591243e-18});
+    FxPhase f;
+    std::frexp(p.h, &f.e);                       // p.h in [2^(e-1), 2^e)
+    f.W = (unsigned long long)std::ldexp(p.h, 64 - f.e) + (unsigned long long)(int64_t)std::floor(std::ldexp(p.l, 64 - f.e) + 0.5);
+    return f;
+}
+
 // ---------------------------------------------------------------------------
 // Alpert's log-singular end correction (j nodes, skip a): nodes x_k in (0, a)
 // and weights w_k with  sum_k w_k x_k^p = -zeta(-p, a)  and

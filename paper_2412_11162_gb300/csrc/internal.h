@@ -81,6 +81,14 @@ struct HostTables {
     std::vector<double> Da, Db;
 };
 
+// w / 2 pi = W 2^(e - 64) (fxtrig.cuh)
+struct FxPhase {
+    unsigned long long W = 0;
+    int e = 0;
+};
+// table lengths of fxtrig.cuh: angles 2 pi j / 1024 of the first quadrant, 2^(j/256)
+constexpr int kTrigFx = 257, kExpFx = 256;
+
 struct DeviceTables {
     double *rho = nullptr, *z = nullptr, *I = nullptr, *Wu = nullptr, *Wphi = nullptr;
     double2 *rho_t = nullptr, *nuc_r = nullptr, *nuc_z = nullptr;
@@ -97,24 +105,15 @@ struct DeviceTables {
     int* corr_w = nullptr;
     double *Da = nullptr, *Db = nullptr;
     double2* cos_tab = nullptr;   // (sin^2(psi_j/2), cos psi_j), j = 0..M/2
-    double2* twid2 = nullptr;     // e^{-2 pi i e / (2M)}, e = 0..2M-1
     int4* twid_fx = nullptr;      // e^{-2 pi i e / (2M)}, e = 0..3M/2-1, Q62 balanced digits (fxdft.cuh)
-    // float-float copies for the mixed path's kernels (kernels_ff.cu): the
-    // length-M and length-2M twiddles and the angle table above as (re.hi, re.lo, im.hi, im.lo), the exp
-    // and sin / cos tables of ffloat.cuh, and per node h W_u / (2M) and
-    // h W_phi / (2M) (column weight times the trapezoid factor of the modes)
+    int4* trig_fx = nullptr;      // fxtrig.cuh: cos, sin of 2 pi j / 1024; 2^(j/256); the media's phases
+    int2* exp_fx = nullptr;
+    FxPhase ph[2];
     // coefficients of the Legendre-Q three-term recurrence of the close-pair
     // Laplace modes, m = 0 .. kRecLen(M): upward (4m/(2m+1), (2m-1)/(2m+1)),
     // downward (4m/(2m-1), (2m+1)/(2m-1)) (entry 0 unused)
     double2* rec_up = nullptr;
     double2* rec_dn = nullptr;
-    float4* twid_ff = nullptr;
-    float4* twid2_ff = nullptr;
-    float4* cos_ff = nullptr;
-    float2* exp_ff = nullptr;
-    float4* trig_ff = nullptr;
-    float2* wuc_ff = nullptr;
-    float2* wpc_ff = nullptr;
 };
 
 }  // namespace pmlbie
@@ -161,6 +160,10 @@ int build_tables(pmlbie_problem* prob);
 // e^{-2 pi i e / (2M)}, e = 0..3M/2-1, as Q62 integers in balanced 32-bit digits
 // (re.high, re.low, im.high, im.low), correctly rounded to about one unit
 std::vector<int4> fx_twiddles(int M);
+// tables of fxtrig.cuh
+std::vector<int4> fx_trig_table();
+std::vector<int2> fx_exp_table();
+FxPhase fx_phase(double w);
 void alpert_log_rule(int j, int a, std::vector<double>& x, std::vector<double>& w);
 
 // kernels (kernels.cu)
@@ -174,45 +177,20 @@ struct FarLaunch {
     bool tune = false;
 };
 cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStream_t s);
-// device time (ms) of the float-float far kernel's chosen configuration in its
-// autotuning launch for this (N, M, modes, output) shape, run alone; 0 if not tuned
-float far_ff_alone_ms(const pmlbie_problem* prob, int modes, bool raw);
-// float-float far kernel of the mixed path (kernels_ff.cu); usable when
-// far_ff_supported (every |q| of the problem inside its sin / cos range)
-cudaError_t launch_far_ff(const pmlbie_problem* prob, const FarLaunch& fl, cudaStream_t s);
-bool far_ff_supported(const pmlbie_problem* prob);
-// host float-float tables of a problem with M azimuthal samples
-void ff_tables(int M, std::vector<float4>& twid, std::vector<float4>& twid2, std::vector<float4>& cosv,
-               std::vector<float2>& expv, std::vector<float4>& trig);
+// device time (ms) of the far kernel's chosen configuration in its autotuning
+// launch for this (N, M, modes, output) shape, run alone; 0 if not tuned
+float far_alone_ms(const pmlbie_problem* prob, int modes, bool raw);
+// host tables of the float-float self-test: angles, exponential, trigonometric
+void ff_tables(std::vector<float2>& expv, std::vector<float4>& trig);
 bool ff_elementary_known(int fn);
 cudaError_t launch_ff_elementary(int fn, const double* x, double* out, size_t n, cudaStream_t s);
 // pairs per CTA of this thread's last far-kernel launch (the tuned choice)
 extern thread_local int g_far_pairs_per_cta;
-// Per close pair, the float-float kernel's quantities (units of L = 2^eL):
-// d~^2 / L^2, rho~ rho~' / L^2, the normal factor's two terms / L, omega_r L,
-// 1 / (omega_r L), then eL and the all-real flag -- written by the Laplace-
-// mode kernel (FP64, one pair per thread) into the float4 area that follows
-// the Laplace modes in the zd scratch (kNearFF float4 per pair).
-constexpr int kNearFF = 7;
-// zd scratch of launch_near: Laplace modes [p][2][M], then, for ff, the
-// per-pair float-float quantities
-inline size_t near_zd_bytes(size_t np, int M, bool ff) {
-    return sizeof(double2) * np * 2 * (size_t)M + (ff ? sizeof(float4) * kNearFF * np : 0);
-}
-// mid (optional): event recorded between the Laplace-mode and the modes kernels;
-// ff: the modes kernel in float-float (mixed path; not with subst_off), zd
-// sized by near_zd_bytes(.., true)
-// mid_ff (optional): event recorded after the float-float modes kernel (right
-// after mid when there is none)
+// zd scratch of launch_near: Laplace modes [p][2][M]
+inline size_t near_zd_bytes(size_t np, int M) { return sizeof(double2) * np * 2 * (size_t)M; }
+// mid (optional): event recorded between the Laplace-mode and the modes kernels
 cudaError_t launch_near(const pmlbie_problem* prob, int mode_lo, int mode_hi, double2* zd_scratch,
-                        double2* out, cudaStream_t s, cudaEvent_t mid = nullptr, bool ff = false,
-                        cudaEvent_t mid_ff = nullptr);
-// the float-float close-pair modes kernel alone (kernels_ff.cu), after the
-// Laplace modes are in zd
-cudaError_t launch_near_modes_ff(const pmlbie_problem* prob, int mode_lo, int mode_hi, const double2* zd,
-                                 const float4* pff, double2* out, cudaStream_t s);
-// Taylor coefficients of cH1 (pa) and cH3 (pb) of degree L <= 7 (Sec. 4.3)
-void taylor_coeffs(int L, double2* pa, double2* pb);
+                        double2* out, cudaStream_t s, cudaEvent_t mid = nullptr);
 cudaError_t launch_near_to_raw(const pmlbie_problem* prob, int mode_lo, int mode_hi,
                                const double2* near_out, double2* raw, cudaStream_t s);
 cudaError_t launch_assemble(const pmlbie_problem* prob, int mode_lo, int mode_hi,

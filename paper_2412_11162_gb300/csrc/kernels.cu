@@ -1,6 +1,8 @@
 // CUDA kernels of the PML-BIE modal solver (sm_103a): modal kernels of far and
 // close node pairs, Alpert assembly of the per-mode block systems, and the
-// right-hand sides.  FP64 (complex128) arithmetic throughout.
+// right-hand sides.  Complex128 results of both precisions: phases, exponentials and
+// transforms in 64-bit fixed point on the integer pipe (fxtrig.cuh, fxdft.cuh), the
+// rest in FP64.
 //
 // Wang & Lu, arXiv 2412.11162:
 //   Sec. 3.1 / 4.3  G~ = e^{i w |dr|}/(4 pi |dr|), |dr|^2 = d^2 + 4 rho~ rho~' sin^2(psi/2)
@@ -20,8 +22,8 @@
 #include "internal.h"
 #include "device_common.cuh"
 #include "fp64_elem.cuh"
-#include "ffloat.cuh"
 #include "modal_fx.cuh"
+#include "fxtrig.cuh"
 
 namespace pmlbie {
 
@@ -33,128 +35,6 @@ namespace {
 // index the low modes' convolutions use); above it Miller's downward
 // recurrence (M + 20 / Re(eta) steps) is used.
 constexpr double kUpward = kRecUpward;
-
-// ---------------------------------------------------------------------------
-// FP64 transforms of the close pairs with a PML point (near_modes_kernel): the
-// Sec. 4.3 split cancels by up to 1e12 there, so that any change of rounding moves
-// the solutions of ill-conditioned modes; every other transform is fixed point
-// (fxdft.cuh).
-//
-// Warp-cooperative Stockham FFT (forward, e^{-2 pi i k n / M}) in shared
-// memory, radices 4, 2, 3 (M = 2^a 3^b).  x, y: two buffers of M elements;
-// returns the buffer holding the result.  tw[e] = e^{-2 pi i e / M}.
-// ---------------------------------------------------------------------------
-__device__ double2* warp_fft(double2* x, double2* y, int M, const double2* tw, int lane, int tws = 1) {
-    // tw[e * tws] = e^{-2 pi i e / M}.  lgNs = log2(Ns) while Ns is a power of
-    // two (radix-4 and radix-2 stages come first), else -1: integer division
-    // by a run-time value expands into conversions, which this GPU issues to
-    // its FP64 pipe.  r k step < M (r < R, k < Ns, step = M / (Ns R)).
-    int rem = M, Ns = 1, lgNs = 0;
-    while (rem > 1) {
-        int R = (rem & 3) == 0 ? 4 : ((rem & 1) == 0 ? 2 : 3);
-        int MR = M / R, step = M / (Ns * R);
-        for (int j = lane; j < MR; j += 32) {
-            const int jq = lgNs >= 0 ? (j >> lgNs) : j / Ns;
-            const int k = j - jq * Ns;
-            double2 v[4];
-            for (int r = 0; r < R; ++r) v[r] = x[j + r * MR];
-            if (Ns > 1)   // the first stage's twiddles are all 1
-                for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[r * k * step * tws]);
-            if (R == 2) {
-                double2 a = v[0], b = v[1];
-                v[0] = cadd(a, b);
-                v[1] = csub(a, b);
-            } else if (R == 4) {
-                double2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-                double2 t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
-                v[0] = cadd(t0, t2);
-                v[2] = csub(t0, t2);
-                v[1] = c2(t1.x + t3.y, t1.y - t3.x);   // t1 - i t3
-                v[3] = c2(t1.x - t3.y, t1.y + t3.x);   // t1 + i t3
-            } else {
-                const double s3 = 0.86602540378443864676;   // sin(2 pi / 3)
-                double2 a = v[0], b = v[1], c = v[2];
-                double2 bc = cadd(b, c), bmc = csub(b, c);
-                v[0] = cadd(a, bc);
-                double2 m = c2(a.x - 0.5 * bc.x, a.y - 0.5 * bc.y);
-                // w = e^{-2 pi i/3}: a + w b + w^2 c = m - i s3 (b - c)
-                v[1] = c2(m.x + s3 * bmc.y, m.y - s3 * bmc.x);
-                v[2] = c2(m.x - s3 * bmc.y, m.y + s3 * bmc.x);
-            }
-            int idxD = jq * Ns * R + k;
-            for (int r = 0; r < R; ++r) y[idxD + r * Ns] = v[r];
-        }
-        __syncwarp();
-        double2* t = x;
-        x = y;
-        y = t;
-        Ns *= R;
-        lgNs = (lgNs >= 0 && R != 3) ? lgNs + (R == 4 ? 2 : 1) : -1;
-        rem /= R;
-    }
-    return x;
-}
-
-// DFT of an even sequence x_0..x_{L-1} (x_k = x_{L-k}, L = 2K, K even) from
-// its K+1 distinct values, in place: xh[0..K] -> X_0..X_K.  Real and imaginary
-// parts are two real-even (DCT-I) transforms; each is reduced to a K-point
-// transform of y_j = x_j (1/2 - sin(pi j/K)) + x_{K-j} (1/2 + sin(pi j/K)) --
-// the two are packed into one complex K-point FFT -- after which the even
-// outputs are the real parts and the odd outputs follow from the imaginary
-// parts by a running sum started at X_1 = 2 sum_{j<K} x_j cos(pi j/K) - x_0 - x_K.
-// y, scr: warp scratch of K elements; twL[e * tws] = e^{-2 pi i e / L};
-// hs[e * tws] = (1/2 + Im twL[e * tws], 1/2 - Im twL[e * tws]) (NULL: computed).
-__device__ void warp_even_dft(double2* xh, double2* y, double2* scr, int K, const double2* twL,
-                              const double2* hs, int tws, int lane) {
-    double2 part = c2(0.0, 0.0);
-    for (int j = lane; j < K; j += 32) {
-        const double2 a = xh[j], b = xh[K - j];
-        const double2 t = twL[j * tws];     // (cos(pi j/K), -sin(pi j/K))
-        const double2 h = hs ? hs[j * tws] : c2(0.5 + t.y, 0.5 - t.y);
-        y[j] = c2(fma(a.x, h.x, b.x * h.y), fma(a.y, h.x, b.y * h.y));
-        const double ct = t.x;
-        part = c2(fma(a.x, ct, part.x), fma(a.y, ct, part.y));
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        part.x += __shfl_xor_sync(0xffffffff, part.x, o);
-        part.y += __shfl_xor_sync(0xffffffff, part.y, o);
-    }
-    const double2 x0 = xh[0], xK = xh[K];
-    const double2 X1 = c2(2.0 * part.x - (x0.x + xK.x), 2.0 * part.y - (x0.y + xK.y));
-    __syncwarp();
-    double2* Z = warp_fft(y, scr, K, twL, lane, 2 * tws);
-    double2* I = (Z == y) ? scr : y;         // imaginary parts for the running sum
-    const int H = K / 2;
-    for (int kk = lane; kk <= H; kk += 32) {
-        const double2 zk = Z[kk], zc = Z[kk == 0 ? 0 : K - kk];
-        // with Ya = (z_k + conj z_{K-k})/2, Yb = (z_k - conj z_{K-k})/(2i):
-        // X_{2k} = 2 (Re Ya + i Re Yb); I_k = 2 (Im Ya + i Im Yb)
-        xh[2 * kk] = c2(zk.x + zc.x, zk.y + zc.y);
-        I[kk] = c2(zk.y - zc.y, zc.x - zk.x);
-    }
-    __syncwarp();
-    // odd outputs: X_{2k+1} = X_1 - sum_{m=1}^{k} I_m, k = 0..H-1 (a warp scan)
-    const int per = (H + 31) / 32;
-    const int b0 = lane * per;
-    double2 run = c2(0.0, 0.0);
-    for (int q = 0; q < per; ++q) {
-        int kk = b0 + q;
-        if (kk >= 1 && kk < H) run = cadd(run, I[kk]);
-    }
-    double2 incl = run;
-    for (int o = 1; o < 32; o <<= 1) {
-        double2 v = c2(__shfl_up_sync(0xffffffff, incl.x, o), __shfl_up_sync(0xffffffff, incl.y, o));
-        if (lane >= o) incl = cadd(incl, v);
-    }
-    double2 acc = csub(X1, csub(incl, run));   // X_1 minus the exclusive prefix of this lane's chunk
-    for (int q = 0; q < per; ++q) {
-        int kk = b0 + q;
-        if (kk >= H) break;
-        if (kk >= 1) acc = csub(acc, I[kk]);
-        xh[2 * kk + 1] = acc;
-    }
-    __syncwarp();
-}
 
 // ---------------------------------------------------------------------------
 // Far pairs.  The kernel samples the ordered pairs (l, m) and (m, l) together:
@@ -176,10 +56,14 @@ __host__ __device__ __forceinline__ size_t far_elems(int M, int nw) {
     return (size_t)3 * M / 4 + (M / 2 + 1) + (size_t)nw * (12 + 4 * (size_t)(M / 2 + 1)) + (5 * (size_t)nw + 3) / 4;
 }
 
-// The samples are FP64; the transforms run on the integer pipe in block fixed
-// point (fxdft.cuh), and the scatter's normal factors carry the column weights.
+// The FP64 pipe (2 lanes a clock and SM) bounds every sampling that works in doubles,
+// so the phases, sines and exponentials (fxtrig.cuh) and the transforms (fxdft.cuh)
+// run on the integer pipe, and FP64 keeps the geometry and the joining products; the
+// scatter's normal factors carry the column weights.  N = 384, M = 256 alone: 1.30 ms,
+// FP64 pipe 49 % busy.  The mixed path takes it too: all modal kernels at N = 512, M = 128
+// 15.2 ms with float-float samples and transforms, 11.7 ms with these.
 template <int NB>
-__global__ void __launch_bounds__(512, NB == 1 ? 2 : 1) far_kernel(FarArgs a) {
+__global__ void __launch_bounds__(256, NB == 1 ? 3 : 2) far_kernel(FarArgs a) {
     extern __shared__ double2 smem[];
     const int M = a.M, N = a.N, K = M / 2, S1 = K + 1;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -195,6 +79,7 @@ __global__ void __launch_bounds__(512, NB == 1 ? 2 : 1) far_kernel(FarArgs a) {
     int* exs = act + nw;                        // per pair: the sequences' exponents
     for (int i = threadIdx.x; i < 3 * M / 4; i += blockDim.x) tw[i] = a.T.twid_fx[2 * i];
     for (int i = threadIdx.x; i <= K; i += blockDim.x) cs[i] = a.T.cos_tab[i];
+    const FxTab TB = fx_tables(a.T);
     // all pairs by the lanes of warp 0: an FP64 instruction occupies its pipe for a
     // whole warp whatever the active lanes
     if (warp == 0 && lane < nw) {
@@ -228,13 +113,13 @@ __global__ void __launch_bounds__(512, NB == 1 ? 2 : 1) far_kernel(FarArgs a) {
         if (g.d2.y == 0.0 && g.rr.y == 0.0) {
             // both nodes physical: real distance, e^{iq} = cos q + i sin q
             const double D2 = fma(4.0 * sc.x, g.rr.x, g.d2.x);
-            const double iR = frsqrt(D2), R = D2 * iR;
+            const double iR = fx_rsqrt(D2), R = D2 * iR;
             const double gk = -(iR * iR * iR), f = iR;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 const double q = (r == 0 ? a.w1 : a.w2) * R, gr = r == 0 ? gk : -gk;
-                double sn, cn;
-                fsincos(q, &sn, &cn);
+                const longlong2 e = fx_cis(fx_turns(R, a.T.ph[r]), TB);
+                const double cn = fx_to_double(e.x, -62), sn = fx_to_double(e.y, -62);
                 buf[(2 * r) * S1 + j] = c2(f * cn, f * sn);
                 buf[(2 * r + 1) * S1 + j] = c2(gr * fma(q, sn, cn), gr * fma(-q, cn, sn));   // e (1 - i q)
             }
@@ -242,14 +127,14 @@ __global__ void __launch_bounds__(512, NB == 1 ? 2 : 1) far_kernel(FarArgs a) {
         }
         const double2 D2 = cadd(g.d2, cscale(g.rr, 4.0 * sc.x));
         double2 R, iR;
-        fcsqrt_rcp(D2, R, iR);
+        fx_csqrt_rcp(D2, R, iR);
         const double2 gk = cscale(cmul(iR, cmul(iR, iR)), -1.0);
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const double w = r == 0 ? a.w1 : a.w2;
             const double2 gr = r == 0 ? gk : c2(-gk.x, -gk.y);
             const double2 q = cscale(R, w);
-            const double2 e = fcexpi(q);
+            const double2 e = fx_expi(R, q.y, a.T.ph[r], TB);
             buf[(2 * r) * S1 + j] = cmul(e, iR);
             buf[(2 * r + 1) * S1 + j] = cmul(cmul(gr, e), c2(1.0 + q.y, -q.x));   // (1 - i q)
         }
@@ -289,11 +174,7 @@ struct NearArgs {
     double w1, w2;
     double2* zd;     // [p][2][M]
     double2* out;    // [p][4][nmodes]
-    double2 pa[8], pb[8];   // Taylor coefficients of cH1 (pa) and cH3 (pb)
-    int hs_tab;             // keep the even-DFT weight table in shared memory
-    float4* pff;            // per-pair float-float quantities (kNearFF float4), or null
-    int share_mirror;       // 1: a pair with a PML point and its mirror are computed by one
-                            // CTA (shared memory permitting)
+    double pa[8], pb[8];    // tails of cH1 (pa) and cH3 (pb), taylor_tails
     const int* lead;        // pairs whose Laplace modes a thread computes (HostTables::near_lead)
     int nlead;
 };
@@ -414,35 +295,9 @@ __device__ void laplace_modes_real(const NearPair& q, const NearPair* qm, int M,
 // criterion; of a grid pair and its mirror, which share chi and hence c_m,
 // the lower index, which computes the modes of both), the list grouped by
 // arithmetic class and recurrence length so that a warp's lanes do the same
-// work.  With a.pff, thread t also writes pair t's float-float quantities.
-// Float-float quantities of close pair q for the mixed path's modes kernel
-// (units of L = 2^eL, L^2 ~ |d~^2| + 4 |rho~ rho~'|), one thread per pair.
-__device__ void near_pair_ff(const NearPair& q, double w1, double w2, float4* out) {
-    using namespace ffm;
-    const double lsq = fabs(q.d2.x) + fabs(q.d2.y) + 4.0 * (fabs(q.rr.x) + fabs(q.rr.y));
-    const int e = ilogb(lsq) / 2;
-    auto c4 = [&](double2 z, int sh) {
-        const ff re = from_double(ldexp(z.x, sh)), im = from_double(ldexp(z.y, sh));
-        return make_float4(re.hi, re.lo, im.hi, im.lo);
-    };
-    auto r4 = [&](double x, double y) {
-        const ff u = from_double(x), v = from_double(y);
-        return make_float4(u.hi, u.lo, v.hi, v.lo);
-    };
-    out[0] = c4(q.d2, -2 * e);
-    out[1] = c4(q.rr, -2 * e);
-    // N_D(psi) / L = [nu'_r (rho~' - rho~) - nu'_z dz] / L + (2 nu'_r rho~ / L) sin^2(psi/2)
-    out[2] = c4(cadd(cmul(q.nuc_r, q.drt), cscale(q.nuc_z, -q.dz)), -e);
-    out[3] = c4(cscale(cmul(q.nuc_r, q.rho_t), 2.0), -e);
-    out[4] = r4(ldexp(w1, e), ldexp(w2, e));
-    out[5] = r4(ldexp(1.0 / w1, -e), ldexp(1.0 / w2, -e));
-    const bool phys = near_physical(q);
-    out[6] = make_float4(__int_as_float(e), __int_as_float(phys ? 1 : 0), 0.0f, 0.0f);
-}
-
+// work.
 __global__ void near_laplace_kernel(NearArgs a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a.pff && t < a.npairs) near_pair_ff(a.np[t], a.w1, a.w2, a.pff + (size_t)t * kNearFF);
     if (t >= a.nlead) return;
     const int p = a.lead[t];
     NearPair q = a.np[p];
@@ -579,60 +434,84 @@ __global__ void __launch_bounds__(128) near_laplace_out_kernel(NearArgs a) {
     }
 }
 
-// Close pairs with a PML point, stage 2 (one CTA of 4 warps per pair), FP64
-// throughout (above): samples of the smooth factors f1, f3 and remainders r1, r3
-// (both regions; the Taylor substitution of Sec. 4.3), their FFTs, and the convolution
+// Close pairs, stage 2 (one CTA per pair): FP64 samples of the smooth
+// factors f1, f3 and remainders r1, r3 (both regions; for PML pairs the
+// Taylor substitution of Sec. 4.3, otherwise H1 = cos q, H3 = cos q + q sin q),
+// their DFTs in block fixed point (fxdft.cuh), and the convolution
 //   S^_n = (1/2pi) sum_{|k| < M/2} Z^_{|n-k|} F1_k + R1_n   (K^_n with D^, F3, R3).
 // Correction pairs that are far by the criterion use the plain FFT.
+// Physical pairs (no point in the PML) have real Z^, D^, f1, f3 and purely
+// imaginary r1, r3, so the two regions are packed as real and imaginary parts
+// of one sequence: 4 sample transforms and 4 convolution transforms instead
+// of 8 and 8.
 // kExact: the diagnostic exact split on PML pairs (compiled into its own
 // variant so that the default one keeps its register budget)
-// Mirror sharing (a.share_mirror): a grid pair (l, m) of the general path and
-// its mirror (m, l) have the same d~^2, rho~ rho~' and hence the same R(psi),
-// samples of the smooth factors f1, f3 and of the single-layer remainder r1,
-// and the same Z^; only the double-layer remainder r3 (its normal factor N_D
-// is the source's) and D^ differ.  The CTA of the lower index computes both:
-// the mirror's r3 samples and their two transforms, its D^ transform, and per
-// region one more product and inverse transform (5 transforms instead of 18);
-// the mirror's S^ equal the pair's.  The mirror's CTA returns at once.
-template <bool kExact>
-__global__ void near_modes_kernel(NearArgs a) {
+// Mirror sharing: a grid pair (l, m) and its mirror (m, l) have the same d~^2,
+// rho~ rho~' and hence the same R(psi), samples of the smooth factors f1, f3 and of
+// the single-layer remainder r1, and the same Z^; only the double-layer remainder
+// r3 (its normal factor N_D is the source's) and D^ differ.  The CTA of the lower
+// index computes both; the mirror's S^ equal the pair's, and its CTA returns at once.
+//
+// Samples, transforms and phases as in the far kernel.  Modal kernels at N = 1024,
+// M = 512 through this kernel: 49.1 ms; with float-float physical pairs and FP64 PML
+// pairs 84.6 ms.  Bounded by the barriers between the phases of one pair and by issue
+// (IPC 1.1 at M = 256); two CTAs of 256 threads hold M = 512's shared memory.
+//
+// Threads of a modes CTA and its shared memory (double2): three quarters of the
+// length-2M twiddles, 8 sample sequences and 2 of the mirror (M/2 + 1), three
+// Laplace-mode sequences and four convolution sequences (M + 1)
+__host__ __device__ constexpr int near_threads(int NB) { return NB <= 2 ? 128 : 256; }
+static size_t near_elems(int M) { return (size_t)3 * M / 2 + 10 * (size_t)(M / 2 + 1) + 7 * (size_t)(M + 1); }
+
+// sum_{j <= n} c_j x^j, x = xr + i xi, |x|^2 = xs, real c_j, n <= 6: the recurrence b_j = c_j
+// + 2 Re x b_{j+1} - |x|^2 b_{j+2} (two operations per degree, where Horner's rule in
+// complex arithmetic takes five)
+__device__ __forceinline__ double2 real_poly(const double (&c)[8], int n, double xr, double xi, double xs) {
+    const double r = 2.0 * xr;
+    double b1 = 0.0, b2 = 0.0;
+#pragma unroll
+    for (int j = 6; j >= 1; --j)
+        if (j <= n) {
+            const double b = fma(r, b1, fma(-xs, b2, c[j]));
+            b2 = b1;
+            b1 = b;
+        }
+    return c2(fma(xr, b1, fma(-xs, b2, c[0])), xi * b1);
+}
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
+    return c2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+
+template <bool kExact, int NB>
+__global__ void __launch_bounds__(near_threads(NB), NB <= 2 ? 4 : NB <= 4 ? 2 : 1) near_modes_kernel(NearArgs a) {
     extern __shared__ double2 smem[];
-    const int M = a.M, K = M / 2, S1 = K + 1, L2 = 2 * M, S2 = M + 1, p = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double2* tw2 = smem;                // 2M: e^{-2 pi i e / (2M)}
-    double2* hs = a.hs_tab ? tw2 + L2 : nullptr;   // M even-DFT weights (if they fit)
-    double2* seq = tw2 + L2 + (a.hs_tab ? M : 0);  // 8 sequences of K+1 (samples, then spectra)
-    double2* cv = seq + 8 * S1;         // 4 sequences of M+1 (convolution)
-    // two scratch slots of 2M: warps w and w + 2 share slot w & 1 (length-2M
-    // transforms of warps 0-1 and 2-3 never overlap; length-M ones take half)
-    double2* slot = cv + 4 * S2 + (warp & 1) * 2 * M;
-    double2* wyK = slot + (warp >> 1) * M;         // y, scr of a length-M transform (K = M/2)
-    // mirror sharing: D^ and K convolution of the mirror (2 x (M+1)), its r3
-    // samples / spectra of both regions (2 x (K+1)), a third 2M scratch slot
-    double2* zDm = cv + 4 * S2 + 4 * M;
-    double2* cKm = zDm + S2;
-    double2* seqm = cKm + S2;
-    double2* slot2 = seqm + 2 * S1;
-    for (int i = threadIdx.x; i < L2; i += blockDim.x) {
-        const double2 t = a.T.twid2[i];
-        tw2[i] = t;
-        if (hs && i < M) hs[i] = c2(0.5 + t.y, 0.5 - t.y);
-    }
-    NearPair q = a.np[p];
-    const bool plain = (q.flags & kFlagFar) != 0;
-    const bool subst = (q.flags & kFlagSubst) != 0;
-    // the other pairs: near_modes_fx_kernel or the float-float kernel
-    if (!subst && (plain || near_physical(q))) return;
-    // mirror sharing (both pairs on the general path, same substitution flag)
+    const int M = a.M, K = M / 2, S1 = K + 1, S2 = M + 1, p = blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    int4* tw = reinterpret_cast<int4*>(smem);   // 3M/2: e^{-2 pi i e / (2M)}
+    double2* seq = smem + 3 * M / 2;    // 10 sequences of K+1 (samples, then spectra)
+    double2* zs = seq + 10 * S1;        // Z^, D^, the mirror's D^
+    double2* cv = zs + 3 * S2;          // per region S and K convolution
+    const NearPair& gp = a.np[p];
+    const bool plain = (gp.flags & kFlagFar) != 0;
+    const bool subst = (gp.flags & kFlagSubst) != 0;
+    NearPair q = gp;
+    // both points physical: every pair quantity is real (the two regions pack
+    // into one transform); a PML pair without the substitution (diagnostic
+    // exact split) takes the general path
+    const bool phys = near_physical(q);
+    const bool packed = !plain && !subst && phys;
+    // mirror sharing (both pairs on the same path)
     bool share = false;
     NearPair qm;
-    if (a.share_mirror && !plain && q.mirror >= 0) {
+    if (!plain && q.mirror >= 0) {
         qm = a.np[q.mirror];
-        const bool mphys = near_physical(qm);
         const bool msubst = (qm.flags & kFlagSubst) != 0;
-        share = (qm.flags & kFlagFar) == 0 && msubst == subst && !(mphys && !msubst);
+        share = (qm.flags & kFlagFar) == 0 && msubst == subst && near_physical(qm) == phys;
         if (share && q.mirror < p) return;    // computed by the mirror's CTA
     }
+    for (int i = threadIdx.x; i < 3 * M / 2; i += blockDim.x) tw[i] = a.T.twid_fx[i];
+    const FxTab TB = fx_tables(a.T);
+    double2* seqm = seq + (packed ? 4 : 8) * S1;   // the mirror's r3
     // sampling; N_D(psi) = [nu'_r (rho~' - rho~) - nu'_z dz] + 2 nu'_r rho~ sin^2(psi/2)
     const double2 nd0 = cadd(cmul(q.nuc_r, q.drt), cscale(q.nuc_z, -q.dz));
     const double2 nds = cscale(cmul(q.nuc_r, q.rho_t), 2.0);
@@ -647,15 +526,44 @@ __global__ void near_modes_kernel(NearArgs a) {
         const double2 sc = a.T.cos_tab[j];
         const double2 D2 = cadd(q.d2, cscale(q.rr, 4.0 * sc.x));
         double2 R, iR;
-        fcsqrt_rcp(D2, R, iR);
+        fx_csqrt_rcp(D2, R, iR);
         const double2 ND = cadd(nd0, cscale(nds, sc.x));
         const double2 NDm = cadd(nd0m, cscale(ndsm, sc.x));
+        if (packed) {
+            // real q = w R; H1 = cos q, i Z H2 = (i w / 4 pi) sin(q)/q, H3 = cos q + q sin q,
+            // i D H4 = -(i w^3 / 4 pi) N_D (sin q - q cos q)/q^3 (region b: -N_D)
+            double f1[2], r1[2], f3[2], r3[2], r3m[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const double w = r == 0 ? a.w1 : a.w2;
+                const double qr = w * R.x, iq = iR.x / w;
+                const longlong2 t = fx_cis(fx_turns(R.x, a.T.ph[r]), TB);
+                const double cs = fx_to_double(t.x, -62), sn = fx_to_double(t.y, -62);
+                const double q2 = qr * qr;
+                const double sinc = fabs(qr) < 1e-3 ? 1.0 - q2 / 6.0 + q2 * q2 / 120.0 : sn * iq;
+                const double h4 = fabs(qr) < 1e-2
+                                      ? 1.0 / 3.0 - q2 / 30.0 + q2 * q2 / 840.0 - q2 * q2 * q2 / 45360.0
+                                      : (sn - qr * cs) * (iq * iq * iq);
+                f1[r] = cs;
+                r1[r] = w * kInv4Pi * sinc;
+                f3[r] = fma(qr, sn, cs);
+                const double h4w = (r == 0 ? -1.0 : 1.0) * w * w * w * kInv4Pi * h4;
+                r3[r] = h4w * ND.x;
+                r3m[r] = h4w * NDm.x;
+            }
+            seq[0 * S1 + j] = c2(f1[0], f1[1]);
+            seq[1 * S1 + j] = c2(r1[0], r1[1]);
+            seq[2 * S1 + j] = c2(f3[0], f3[1]);
+            seq[3 * S1 + j] = c2(r3[0], r3[1]);
+            if (share) seqm[j] = c2(r3m[0], r3m[1]);
+            continue;
+        }
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const double w = r == 0 ? a.w1 : a.w2;
             const double sg = r == 0 ? 1.0 : -1.0;     // region b normal -nu
             const double2 qq = cscale(R, w);
-            const double2 e = fcexpi(qq);
+            const double2 e = fx_expi(R, qq.y, a.T.ph[r], TB);
             double2 v0, v1, v2, v3, v3m = c2(0.0, 0.0);
             if (plain) {
                 const double2 iR3 = cmul(iR, cmul(iR, iR));
@@ -689,198 +597,26 @@ __global__ void near_modes_kernel(NearArgs a) {
                 if (share) v3m = cscale(cmul(c2(0.0, 1.0), cmul(NDm, h4)), -w * w * w * kInv4Pi * sg);
             } else {
                 // cH1 = e^{iq} sum a_k q^k, Z (e^{iq} - cH1) = -(w / 4 pi) e^{iq} sum_{k>=1} a_k q^{k-1};
-                // cH3 likewise; D (e^{iq}(1 - iq) - cH3) = (w^3 / 4 pi) N_D e^{iq} sum_{k>=3} b_k q^{k-3}
-                // (L >= 3; coefficients beyond L are zero) the full sums from the tails:
-                // P_a = a_0 + q P_a1, P_b = b_0 + q (b_1 + q (b_2 + q P_b3))
-                const double2 pa1 = cpoly_from(a.pa, 1, L, qq);
-                const double2 pb3 = cpoly_from(a.pb, 3, L, qq);
-                const double2 pa0 = cadd(a.pa[0], cmul(qq, pa1));
-                const double2 pb0 =
-                    cadd(a.pb[0], cmul(qq, cadd(a.pb[1], cmul(qq, cadd(a.pb[2], cmul(qq, pb3))))));
-                v0 = cmul(e, pa0);
-                v1 = cscale(cmul(e, pa1), -w * kInv4Pi);
-                v2 = cmul(e, pb0);
-                v3 = cscale(cmul(cmul(ND, e), pb3), w * w * w * kInv4Pi * sg);
-                if (share) v3m = cscale(cmul(cmul(NDm, e), pb3), w * w * w * kInv4Pi * sg);
+                // cH3 likewise; D (e^{iq}(1 - iq) - cH3) = (w^3 / 4 pi) N_D e^{iq} sum_{k>=3} b_k q^{k-3}.
+                // With x = -2iq both tails have real coefficients (taylor_tails): sum_{k>=1}
+                // a_k q^{k-1} = -i g1(x), sum_{k>=3} b_k q^{k-3} = i g3(x), and a_0 = b_0 = 1, b_1 =
+                // -i, b_2 = 0.  t1 and t3, the tails times e^{iq}, enter the smooth factor and the
+                // remainder alike, so that their rounding cancels in the split's two terms.
+                const double xr = 2.0 * qq.y, xi = -2.0 * qq.x, xs = fma(xr, xr, xi * xi);
+                const double2 g1 = real_poly(a.pa, L - 1, xr, xi, xs), g3 = real_poly(a.pb, L - 3, xr, xi, xs);
+                const double2 t1 = cmul(e, c2(g1.y, -g1.x)), t3 = cmul(e, c2(-g3.y, g3.x));
+                v0 = cfma(qq, t1, e);
+                v1 = cscale(t1, -w * kInv4Pi);
+                v2 = cfma(cmul(qq, cmul(qq, qq)), t3, cmul(e, c2(1.0 + qq.y, -qq.x)));
+                const double2 t3w = cscale(t3, w * w * w * kInv4Pi * sg);
+                v3 = cmul(ND, t3w);
+                if (share) v3m = cmul(NDm, t3w);
             }
             seq[(4 * r + 0) * S1 + j] = v0;
             seq[(4 * r + 1) * S1 + j] = v1;
             seq[(4 * r + 2) * S1 + j] = v2;
             seq[(4 * r + 3) * S1 + j] = v3;
             if (share) seqm[r * S1 + j] = v3m;
-        }
-    }
-    __syncthreads();
-    // even-sequence DFTs of length M: plain pairs 0, 2, 4, 6, the others all 8
-    for (int s = warp; s < (share ? 10 : 8); s += 4) {
-        if (plain && (s & 1)) continue;
-        warp_even_dft(s < 8 ? seq + s * S1 : seqm + (s - 8) * S1, wyK, wyK + K, K, tw2, hs, 2, lane);
-    }
-    __syncthreads();
-    const double scale = 2.0 * kPi / M;
-    const int nmodes = a.mode_hi - a.mode_lo;
-    double2* out = a.out + (size_t)p * 4 * nmodes;
-    const double2* Z = a.zd + (size_t)p * 2 * M;
-    const double2* Dd = Z + M;
-    if (plain) {
-        for (int t = threadIdx.x; t < nmodes; t += blockDim.x) {
-            int n = a.mode_lo + t;
-            out[0 * (size_t)nmodes + t] = cscale(seq[0 * S1 + n], scale);
-            out[1 * (size_t)nmodes + t] = cscale(seq[2 * S1 + n], scale);
-            out[2 * (size_t)nmodes + t] = cscale(seq[4 * S1 + n], scale);
-            out[3 * (size_t)nmodes + t] = cscale(seq[6 * S1 + n], scale);
-        }
-        return;
-    }
-    // convolution (1/2pi) sum_{|k| < M/2} X^_{|n-k|} C_k as a circular convolution
-    // of length 2M (exact for n < M/2) of the even sequences zZ[m] = Z^_{|m|}
-    // (|m| <= M-2), zD[m] = D^_{|m|}, c[k] = C_{|k|} (|k| <= M/2-1); all are even,
-    // so every transform is an even-sequence DFT of M+1 values, and the inverse
-    // of an even sequence is its forward transform divided by 2M.
-    double2* zZ = cv;
-    double2* zD = cv + S2;
-    double2* cS = cv + 2 * S2;
-    double2* cK = cv + 3 * S2;
-    const double2* Ddm = share ? a.zd + (size_t)q.mirror * 2 * M + M : nullptr;
-    double2* outm = share ? a.out + (size_t)q.mirror * 4 * nmodes : nullptr;
-    for (int i = threadIdx.x; i <= M; i += blockDim.x) {
-        bool inz = i <= M - 2;
-        zZ[i] = inz ? Z[i] : c2(0.0, 0.0);
-        zD[i] = inz ? Dd[i] : c2(0.0, 0.0);
-        if (share) zDm[i] = inz ? Ddm[i] : c2(0.0, 0.0);
-    }
-    __syncthreads();
-    if (warp < 2) warp_even_dft(warp == 0 ? zZ : zD, slot, slot + M, M, tw2, hs, 1, lane);
-    if (share && warp == 2) warp_even_dft(zDm, slot2, slot2 + M, M, tw2, hs, 1, lane);
-    const double c = 1.0 / (2.0 * kPi * L2);
-    for (int r = 0; r < 2; ++r) {
-        for (int i = threadIdx.x; i <= M; i += blockDim.x) {
-            bool in = i <= K - 1;
-            double2 vS = c2(0.0, 0.0), vK = c2(0.0, 0.0);
-            if (in) {
-                vS = cscale(seq[(4 * r + 0) * S1 + i], scale);
-                vK = cscale(seq[(4 * r + 2) * S1 + i], scale);
-            }
-            cS[i] = vS;
-            cK[i] = vK;
-        }
-        __syncthreads();
-        if (warp >= 2) warp_even_dft(warp == 2 ? cS : cK, slot, slot + M, M, tw2, hs, 1, lane);
-        __syncthreads();
-        const double sgn = r == 0 ? 1.0 : -1.0;      // region b: D^ -> -D^
-        for (int i = threadIdx.x; i <= M; i += blockDim.x) {
-            cS[i] = cmul(zZ[i], cS[i]);
-            if (share) cKm[i] = cscale(cmul(zDm[i], cK[i]), sgn);
-            cK[i] = cscale(cmul(zD[i], cK[i]), sgn);
-        }
-        __syncthreads();
-        if (warp >= 2) warp_even_dft(warp == 2 ? cS : cK, slot, slot + M, M, tw2, hs, 1, lane);
-        if (share && warp == 1) warp_even_dft(cKm, slot2, slot2 + M, M, tw2, hs, 1, lane);
-        __syncthreads();
-        for (int t = threadIdx.x; t < nmodes; t += blockDim.x) {
-            int n = a.mode_lo + t;
-            const double2 sv = cadd(cscale(cS[n], c), cscale(seq[(4 * r + 1) * S1 + n], scale));
-            out[(2 * r + 0) * (size_t)nmodes + t] = sv;
-            out[(2 * r + 1) * (size_t)nmodes + t] = cadd(cscale(cK[n], c), cscale(seq[(4 * r + 3) * S1 + n], scale));
-            if (share) {
-                outm[(2 * r + 0) * (size_t)nmodes + t] = sv;
-                outm[(2 * r + 1) * (size_t)nmodes + t] = cadd(cscale(cKm[n], c), cscale(seqm[r * S1 + n], scale));
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// Close pairs without a PML point (and correction pairs far by the criterion),
-// stage 2, FP64 samples: physical pairs have real Z^, D^, f1, f3 and purely
-// imaginary r1, r3 (H1 = cos q, H3 = cos q + q sin q), so the two regions are packed
-// as real and imaginary parts of one sequence; the transforms and the convolution
-// run in block fixed point (near_finish).  The FP64 path; the mixed path takes the
-// same pairs with float-float samples.  Mirror sharing as above.
-//
-// Threads of a CTA and its shared memory (double2): three quarters of the length-2M
-// twiddles, 7 sample sequences (M/2 + 1; packed pairs use 5), three Laplace-mode and
-// two convolution sequences (M + 1)
-__host__ __device__ constexpr int near_threads(int NB) { return NB <= 2 ? 128 : 256; }
-static size_t near_elems(int M) { return (size_t)3 * M / 2 + 7 * (size_t)(M / 2 + 1) + 5 * (size_t)(M + 1); }
-
-template <int NB>
-__global__ void __launch_bounds__(near_threads(NB), NB <= 2 ? 4 : NB <= 4 ? 2 : 1) near_modes_fx_kernel(NearArgs a) {
-    extern __shared__ double2 smem[];
-    const int M = a.M, K = M / 2, S1 = K + 1, S2 = M + 1, p = blockIdx.x;
-    const int lane = threadIdx.x & 31;
-    int4* tw = reinterpret_cast<int4*>(smem);   // 3M/2: e^{-2 pi i e / (2M)}
-    double2* seq = smem + 3 * M / 2;    // 7 sequences of K+1 (samples, then spectra)
-    double2* zs = seq + 7 * S1;         // Z^, D^, the mirror's D^
-    double2* cv = zs + 3 * S2;          // S and K convolution
-    const NearPair q = a.np[p];
-    const bool plain = (q.flags & kFlagFar) != 0;
-    if ((q.flags & kFlagSubst) || !(plain || near_physical(q))) return;   // near_modes_kernel's
-    const bool packed = !plain;
-    bool share = false;
-    NearPair qm;
-    if (packed && q.mirror >= 0) {
-        qm = a.np[q.mirror];
-        share = (qm.flags & (kFlagFar | kFlagSubst)) == 0 && near_physical(qm);
-        if (share && q.mirror < p) return;    // computed by the mirror's CTA
-    }
-    for (int i = threadIdx.x; i < 3 * M / 2; i += blockDim.x) tw[i] = a.T.twid_fx[i];
-    double2* seqm = seq + 4 * S1;       // the mirror's r3
-    // sampling; N_D(psi) = [nu'_r (rho~' - rho~) - nu'_z dz] + 2 nu'_r rho~ sin^2(psi/2)
-    const double2 nd0 = cadd(cmul(q.nuc_r, q.drt), cscale(q.nuc_z, -q.dz));
-    const double2 nds = cscale(cmul(q.nuc_r, q.rho_t), 2.0);
-    double2 nd0m = c2(0.0, 0.0), ndsm = nd0m;
-    if (share) {
-        nd0m = cadd(cmul(qm.nuc_r, qm.drt), cscale(qm.nuc_z, -qm.dz));
-        ndsm = cscale(cmul(qm.nuc_r, qm.rho_t), 2.0);
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j <= K; j += blockDim.x) {
-        const double2 sc = a.T.cos_tab[j];
-        const double2 D2 = cadd(q.d2, cscale(q.rr, 4.0 * sc.x));
-        double2 R, iR;
-        fcsqrt_rcp(D2, R, iR);
-        const double2 ND = cadd(nd0, cscale(nds, sc.x));
-        const double2 NDm = cadd(nd0m, cscale(ndsm, sc.x));
-        if (packed) {
-            // real q = w R; H1 = cos q, i Z H2 = (i w / 4 pi) sin(q)/q, H3 = cos q + q sin q,
-            // i D H4 = -(i w^3 / 4 pi) N_D (sin q - q cos q)/q^3 (region b: -N_D)
-            double f1[2], r1[2], f3[2], r3[2], r3m[2];
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const double w = r == 0 ? a.w1 : a.w2;
-                const double qr = w * R.x, iq = iR.x / w;
-                double sn, cs;
-                fsincos(qr, &sn, &cs);
-                const double q2 = qr * qr;
-                const double sinc = fabs(qr) < 1e-3 ? 1.0 - q2 / 6.0 + q2 * q2 / 120.0 : sn * iq;
-                const double h4 = fabs(qr) < 1e-2
-                                      ? 1.0 / 3.0 - q2 / 30.0 + q2 * q2 / 840.0 - q2 * q2 * q2 / 45360.0
-                                      : (sn - qr * cs) * (iq * iq * iq);
-                f1[r] = cs;
-                r1[r] = w * kInv4Pi * sinc;
-                f3[r] = fma(qr, sn, cs);
-                const double h4w = (r == 0 ? -1.0 : 1.0) * w * w * w * kInv4Pi * h4;
-                r3[r] = h4w * ND.x;
-                r3m[r] = h4w * NDm.x;
-            }
-            seq[0 * S1 + j] = c2(f1[0], f1[1]);
-            seq[1 * S1 + j] = c2(r1[0], r1[1]);
-            seq[2 * S1 + j] = c2(f3[0], f3[1]);
-            seq[3 * S1 + j] = c2(r3[0], r3[1]);
-            if (share) seqm[j] = c2(r3m[0], r3m[1]);
-            continue;
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const double w = r == 0 ? a.w1 : a.w2;
-            const double sg = r == 0 ? 1.0 : -1.0;     // region b normal -nu
-            const double2 qq = cscale(R, w);
-            const double2 e = fcexpi(qq);
-            const double2 iR3 = cmul(iR, cmul(iR, iR));
-            const double2 Dk = cscale(cmul(ND, iR3), -kInv4Pi * sg);
-            seq[(4 * r + 0) * S1 + j] = cscale(cmul(e, iR), kInv4Pi);
-            seq[(4 * r + 2) * S1 + j] = cmul(cmul(Dk, e), c2(1.0 + qq.y, -qq.x));
         }
     }
     __syncthreads();
@@ -1174,7 +910,15 @@ static size_t far_smem(int M, int nw) { return sizeof(double2) * far_elems(M, nw
 // repeated runs leave the same output).
 static std::mutex g_far_tune_mu;
 static std::map<std::tuple<int, int, int, int>, int> g_far_tuned;
+// device time of the chosen configuration in its tuning launch (alone on the GPU)
+static std::map<std::tuple<int, int, int, int>, float> g_far_tuned_ms;
 thread_local int g_far_pairs_per_cta = 0;
+
+float far_alone_ms(const pmlbie_problem* prob, int modes, bool raw) {
+    std::lock_guard<std::mutex> lk(g_far_tune_mu);
+    auto it = g_far_tuned_ms.find(std::make_tuple(prob->P.N, prob->P.M, modes, raw ? 1 : 0));
+    return it == g_far_tuned_ms.end() ? 0.f : it->second;
+}
 
 cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStream_t s) {
     const int N = prob->P.N, M = prob->P.M;
@@ -1201,11 +945,11 @@ cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStre
             return cudaGetLastError();
         });
     };
-    // PMLBIE_FAR_PAIRS_PER_CTA=2|4|8|16 fixes the choice (reproducible profiling)
+    // PMLBIE_FAR_PAIRS_PER_CTA=2|4|8 fixes the choice (reproducible profiling)
     static const int forced = [] {
         const char* v = std::getenv("PMLBIE_FAR_PAIRS_PER_CTA");
         const int f = v ? std::atoi(v) : 0;
-        return (f == 2 || f == 4 || f == 8 || f == 16) ? f : 0;
+        return (f == 2 || f == 4 || f == 8) ? f : 0;
     }();
     if (forced && far_smem(M, forced) <= 227 * 1024) return run(forced);
     const auto key = std::make_tuple(N, M, fl.mode_hi - fl.mode_lo, fl.raw ? 1 : 0);
@@ -1228,7 +972,7 @@ cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStre
     }
     int best = far_warps(M);
     float tbest = 1e30f;
-    for (int c : {2, 4, 8, 16}) {
+    for (int c : {2, 4, 8}) {
         if (far_smem(M, c) > (size_t)optin) continue;
         float ms = 0.f;
         if ((e = cudaEventRecord(e0, s)) != cudaSuccess || (e = run(c)) != cudaSuccess ||
@@ -1242,33 +986,27 @@ cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStre
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_far_tune_mu);
     g_far_tuned[key] = best;
+    g_far_tuned_ms[key] = tbest;
     g_far_pairs_per_cta = best;
     return cudaSuccess;
 }
 
-void taylor_coeffs(int L, double2* pa, double2* pb) {
-    // P1 = Taylor_L[(1 + e^{-2iq})/2], P3 = Taylor_L[(1 + e^{-2iq})/2 - iq (1 - e^{-2iq})/2]
-    cd e[9];
-    double f = 1.0;
-    for (int k = 0; k <= L; ++k) {
-        if (k > 0) f *= k;
-        e[k] = std::pow(cd(0.0, -2.0), k) / f;
-    }
-    for (int k = 0; k < 8; ++k) {
-        pa[k] = make_double2(0, 0);
-        pb[k] = make_double2(0, 0);
-    }
-    for (int k = 0; k <= L; ++k) {
-        cd ak = ((k == 0 ? 1.0 : 0.0) + e[k]) / 2.0;
-        cd bk = ak;
-        if (k >= 1) bk += cd(0.0, -1.0) * ((k == 1 ? 1.0 : 0.0) - e[k - 1]) / 2.0;
-        pa[k] = make_double2(ak.real(), ak.imag());
-        pb[k] = make_double2(bk.real(), bk.imag());
+// Coefficients in x = -2iq of the tails of the Sec. 4.3 polynomials of degree L.
+// P1 = Taylor_L[(1 + e^{-2iq})/2] has a_k = (-2i)^k / (2 k!) (k >= 1), so sum_{k>=1} a_k
+// q^{k-1} = -i sum_j x^j / (j+1)!; P3 = Taylor_L[(1 + e^{-2iq})/2 - iq (1 - e^{-2iq})/2]
+// has b_k = (-2i)^k (1 - k/2) / (2 k!) (k >= 2), so sum_{k>=3} b_k q^{k-3} = i sum_j x^j
+// 8 (1 - (j+3)/2) / (2 (j+3)!).
+static void taylor_tails(int L, double* p1, double* p3) {
+    double f[16] = {1.0};
+    for (int k = 1; k < 16; ++k) f[k] = f[k - 1] * k;
+    for (int j = 0; j < 8; ++j) {
+        p1[j] = j <= L - 1 ? 1.0 / f[j + 1] : 0.0;
+        p3[j] = j <= L - 3 ? 4.0 * (1.0 - 0.5 * (j + 3)) / f[j + 3] : 0.0;
     }
 }
 
 cudaError_t launch_near(const pmlbie_problem* prob, int mode_lo, int mode_hi, double2* zd,
-                        double2* out, cudaStream_t s, cudaEvent_t mid, bool ff, cudaEvent_t mid_ff) {
+                        double2* out, cudaStream_t s, cudaEvent_t mid) {
     const int M = prob->P.M;
     NearArgs a;
     a.T = prob->D;
@@ -1283,62 +1021,31 @@ cudaError_t launch_near(const pmlbie_problem* prob, int mode_lo, int mode_hi, do
     a.w2 = prob->P.k2;
     a.zd = zd;
     a.out = out;
-    const bool use_ff = ff && !prob->P.subst_off;
-    a.pff = use_ff ? reinterpret_cast<float4*>(zd + (size_t)a.npairs * 2 * M) : nullptr;
-    taylor_coeffs(a.L, a.pa, a.pb);
-    if (a.npairs == 0) {
-        cudaError_t e0 = mid ? cudaEventRecord(mid, s) : cudaSuccess;
-        if (e0 == cudaSuccess && mid_ff) e0 = cudaEventRecord(mid_ff, s);
-        return e0;
-    }
+    taylor_tails(a.L, a.pa, a.pb);
+    if (a.npairs == 0) return mid ? cudaEventRecord(mid, s) : cudaSuccess;
     a.lead = prob->D.near_lead;
     a.nlead = (int)prob->H.near_lead.size();
-    const int nthr = std::max(a.nlead, a.pff ? a.npairs : 0);
-    if (nthr > 0) {
-        near_laplace_kernel<<<(nthr + 127) / 128, 128, 0, s>>>(a);
-        count_launch();
-    }
     if (a.nlead > 0) {
+        near_laplace_kernel<<<(a.nlead + 127) / 128, 128, 0, s>>>(a);
         near_laplace_out_kernel<<<a.nlead, 128, sizeof(double2) * ((size_t)M + kLapRec), s>>>(a);
-        count_launch();
+        count_launch(2);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (mid && (e = cudaEventRecord(mid, s)) != cudaSuccess) return e;
-    // the pairs without a PML point in float-float or FP64, then the others in FP64
-    if (use_ff) {
-        if ((e = launch_near_modes_ff(prob, mode_lo, mode_hi, zd, a.pff, out, s)) != cudaSuccess) return e;
-    } else {
-        const size_t smem = sizeof(double2) * near_elems(M);
-        e = with_full_class(M, [&](auto nb) {
-            constexpr int NB = decltype(nb)::value;
-            const cudaError_t er = allow_max_smem(near_modes_fx_kernel<NB>);
-            if (er != cudaSuccess) return er;
-            near_modes_fx_kernel<NB><<<a.npairs, near_threads(NB), smem, s>>>(a);
-            count_launch();
-            return cudaGetLastError();
-        });
-        if (e != cudaSuccess) return e;
-    }
-    if (mid_ff && (e = cudaEventRecord(mid_ff, s)) != cudaSuccess) return e;
-    // tw2 (2M) + 8 x (M/2+1) + 4 x (M+1) + 2 scratch slots x 2M (+ M weights when they
-    // fit), + for mirror sharing 2 x (M+1) + 2 x (M/2+1) + a third slot of 2M (when
-    // it fits too)
-    size_t smem = sizeof(double2) * ((size_t)2 * M + 8 * (M / 2 + 1) + 4 * (M + 1) + 4 * (size_t)M);
-    const size_t share_bytes = sizeof(double2) * ((size_t)2 * (M + 1) + 2 * (M / 2 + 1) + 2 * (size_t)M);
-    a.hs_tab = smem + sizeof(double2) * M <= 227 * 1024 ? 1 : 0;
-    if (a.hs_tab) smem += sizeof(double2) * M;
-    a.share_mirror = smem + share_bytes <= 227 * 1024 ? 1 : 0;
-    if (a.share_mirror) smem += share_bytes;
-    if (prob->P.subst_off) {
-        if ((e = allow_max_smem(near_modes_kernel<true>)) != cudaSuccess) return e;
-        near_modes_kernel<true><<<a.npairs, 128, smem, s>>>(a);
-    } else {
-        if ((e = allow_max_smem(near_modes_kernel<false>)) != cudaSuccess) return e;
-        near_modes_kernel<false><<<a.npairs, 128, smem, s>>>(a);
-    }
-    count_launch();
-    return cudaGetLastError();
+    const size_t smem = sizeof(double2) * near_elems(M);
+    const bool exact = prob->P.subst_off != 0;
+    return with_full_class(M, [&](auto nb) {
+        constexpr int NB = decltype(nb)::value;
+        cudaError_t er = exact ? allow_max_smem(near_modes_kernel<true, NB>) : allow_max_smem(near_modes_kernel<false, NB>);
+        if (er != cudaSuccess) return er;
+        if (exact)
+            near_modes_kernel<true, NB><<<a.npairs, near_threads(NB), smem, s>>>(a);
+        else
+            near_modes_kernel<false, NB><<<a.npairs, near_threads(NB), smem, s>>>(a);
+        count_launch();
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_near_to_raw(const pmlbie_problem* prob, int mode_lo, int mode_hi,
@@ -1461,7 +1168,8 @@ struct FieldArgs {
 // conormal.  One warp; buf holds 2 S1 values.
 template <int NB>
 __device__ __forceinline__ void point_node_modes(const DeviceTables& T, int M, double w, double sg, double rx, double zx, int m,
-                                 const double2* cs, const int4* tw, double2* buf, int lane, int& exS, int& exK) {
+                                 const double2* cs, const int4* tw, FxPhase ph, double2* buf, int lane,
+                                                 int& exS, int& exK) {
     const int K = M / 2, S1 = K + 1;
     const double dr = rx - T.rho[m], dz = zx - T.z[m], dI = -T.I[m];   // the point is physical: I = 0
     const double2 drt = c2(dr, dI);
@@ -1470,15 +1178,16 @@ __device__ __forceinline__ void point_node_modes(const DeviceTables& T, int M, d
     const double2 ncr = cscale(T.nuc_r[m], sg), ncz = cscale(T.nuc_z[m], sg);
     const double2 nd0 = cadd(cmul(ncr, c2(-dr, -dI)), cscale(ncz, -dz));
     const double2 nds = cscale(ncr, 2.0 * rx);
+    const FxTab TB = fx_tables(T);
     for (int j = lane; j <= K; j += 32) {
         const double2 sc = cs[j];
         const double2 D2 = cadd(d2, cscale(rr, 4.0 * sc.x));
         double2 R, iR;
-        fcsqrt_rcp(D2, R, iR);
+        fx_csqrt_rcp(D2, R, iR);
         const double2 iR3 = cmul(iR, cmul(iR, iR));
         const double2 ND = cadd(nd0, cscale(nds, sc.x));
         const double2 q = cscale(R, w);
-        const double2 e = fcexpi(q);
+        const double2 e = fx_expi(R, q.y, ph, TB);
         buf[j] = cscale(cmul(e, iR), kInv4Pi);
         buf[S1 + j] = cmul(cmul(cscale(cmul(ND, iR3), -kInv4Pi), e), c2(1.0 + q.y, -q.x));
     }
@@ -1512,7 +1221,8 @@ __global__ void field_kernel(FieldArgs a) {
     const int reg = a.preg[p];
     const double sg = reg == 0 ? 1.0 : -1.0;
     int exS, exK;
-    point_node_modes<NB>(a.T, M, reg == 0 ? a.w1 : a.w2, sg, a.prho[p], a.pz[p], m, cs, tw, buf, lane, exS, exK);
+    point_node_modes<NB>(a.T, M, reg == 0 ? a.w1 : a.w2, sg, a.prho[p], a.pz[p], m, cs, tw, a.T.ph[reg],
+                         buf, lane, exS, exK);
     const longlong2* f = reinterpret_cast<const longlong2*>(buf);
     const double scale = 2.0 * kPi / M;
     const double fs = 0.5 * sg * scale * a.h * a.T.Wphi[m], fk = -0.5 * scale * a.h * a.T.Wu[m];
@@ -1542,7 +1252,7 @@ __global__ void point_rhs_kernel(DeviceTables T, int N, int M, int nrhs, int mod
     if (m >= N) return;
     const double* pr = rpar + (size_t)kRhsPar * r;
     int exS, exK;
-    point_node_modes<NB>(T, M, w1, 1.0, pr[0], pr[1], m, cs, tw, buf, lane, exS, exK);
+    point_node_modes<NB>(T, M, w1, 1.0, pr[0], pr[1], m, cs, tw, T.ph[0], buf, lane, exS, exK);
     const longlong2* f = reinterpret_cast<const longlong2*>(buf);
     const double scale = 2.0 * kPi / M, az = pr[6], sp = speed[m];
     for (int t = lane; t < nmodes; t += 32) {

@@ -85,7 +85,7 @@ struct FarArgs {
 };
 
 // targets x sources of a CTA with nw pairs
-__host__ __device__ __forceinline__ int far_tile_m(int nw) { return nw >= 16 ? 4 : 2; }
+__host__ __device__ __forceinline__ int far_tile_m(int nw) { return 2; }
 
 // Pair of lane `lane` (< nw) of a far CTA: target l = l0 + lane % TL, source m =
 // m0 + lane / TL.  Returns its flags (bit 0: (l, m) is far; bit 1: (m, l) is far;
@@ -201,66 +201,76 @@ __device__ __forceinline__ void near_finish(const NearShape& p, int M, const int
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     const double scale = 6.28318530717958647692 / M;
     const int mirror0 = p.packed ? 4 : 8;          // the mirror's r3
-    // One warp per task, the longest first: a smooth factor's transform of length M
-    // followed by its modes' transform of length 2M; the Laplace modes' transforms;
-    // the remainders' transforms.
+    // One warp per task, the longest first.  Phase 0: a smooth factor's transform of
+    // length M followed by its modes' transform of length 2M; the Laplace modes'
+    // transforms; the remainders' transforms.  Phase 1: the products' transforms.  (One
+    // loop, so that each transform's code is in the kernel once.)
     const int nc = p.plain ? 0 : p.packed ? 2 : 4, nz = p.plain ? 0 : p.share ? 3 : 2;
     const int nr = p.plain ? 4 : nc + (p.share ? nc / 2 : 0);
-    for (int t = warp; t < nc + nz + nr; t += nwarp) {
-        if (t >= nc && t < nc + nz) {
-            const double2* src = t == nc ? p.Z : t == nc + 1 ? p.D : p.Dm;
-            double2* z = zs + (t - nc) * S2;
-            for (int i = lane; i <= M; i += 32) z[i] = i <= M - 2 ? src[i] : c2(0.0, 0.0);
-            __syncwarp();
-            const int ex = fx_even_dft<NB>(reinterpret_cast<longlong2*>(z), fx_quantise(z, S2, lane), M, tw, 1, lane);
-            if (lane == 0) exz[t - nc] = ex;
-            continue;
+    for (int phase = 0; phase < 2; ++phase) {
+        const int ntask = phase == 0 ? nc + nz + nr : nc + (p.share ? nc / 2 : 0);
+        for (int t = warp; t < ntask; t += nwarp) {
+            double2* y = nullptr;         // sequence of length 2M to transform, its scale and exponent's place
+            int* ey = nullptr;
+            FxScale sc;
+            if (phase == 0 && (t < nc || t >= nc + nz)) {
+                // f1 / f3 (t < nc), r1 / r3 of the same pairs, the mirror's r3; plain: 0, 2, 4, 6
+                const int u = t - nc - nz;
+                const int s = t < nc ? 2 * t : p.plain ? 2 * u : u < nc ? 2 * u + 1 : mirror0 + (u - nc);
+                longlong2* x = seq + s * S1;
+                const int ex = fx_even_dft<NBH>(x, quantise(x, s), K, tw, 2, lane);
+                if (lane == 0) exq[s] = ex;
+                if (t < nc) {
+                    // packed: F1a + i F1b and F3a - i F3b (region b's -D^ as the conjugate)
+                    y = cv + t * S2;
+                    ey = exc + t;
+                    sc = fx_requantise(x, reinterpret_cast<longlong2*>(y), K, S2, ex, p.packed && t == 1, lane);
+                }
+            } else {
+                if (phase == 0) {
+                    const double2* src = t == nc ? p.Z : t == nc + 1 ? p.D : p.Dm;
+                    y = zs + (t - nc) * S2;
+                    ey = exz + (t - nc);
+                    for (int i = lane; i <= M; i += 32) y[i] = i <= M - 2 ? src[i] : c2(0.0, 0.0);
+                    __syncwarp();
+                } else {
+                    y = t < nc ? cv + t * S2 : zs + (t - nc) * S2;
+                    ey = exo + t;
+                }
+                sc = fx_quantise(y, S2, lane);
+            }
+            if (y) {
+                const int ex = fx_even_dft<NB>(reinterpret_cast<longlong2*>(y), sc, M, tw, 1, lane);
+                if (lane == 0) *ey = ex;
+            }
         }
-        // sequence: f1 / f3 (t < nc), r1 / r3 of the same pairs, the mirror's r3; plain: 0, 2, 4, 6
-        const int u = t - nc - nz;
-        const int s = t < nc ? 2 * t : p.plain ? 2 * u : u < nc ? 2 * u + 1 : mirror0 + (u - nc);
-        longlong2* x = seq + s * S1;
-        const int ex = fx_even_dft<NBH>(x, quantise(x, s), K, tw, 2, lane);
-        if (lane == 0) exq[s] = ex;
-        if (t < nc) {
-            // packed: F1a + i F1b and F3a - i F3b (region b's -D^ as the conjugate)
-            longlong2* c = reinterpret_cast<longlong2*>(cv) + t * S2;
-            const FxScale sc = fx_requantise(x, c, K, S2, ex, p.packed && t == 1, lane);
-            const int ec = fx_even_dft<NB>(c, sc, M, tw, 1, lane);
-            if (lane == 0) exc[t] = ec;
+        __syncthreads();
+        if (phase == 1) break;
+        if (p.plain) {
+            for (int t = threadIdx.x; t < 4 * p.nmodes; t += blockDim.x) {
+                const int k = t / p.nmodes, n = p.mode_lo + (t - k * p.nmodes);
+                p.out[t] = cscale(fx_to_double2(seq[2 * k * S1 + n], exq[2 * k]), scale);
+            }
+            return;
         }
-    }
-    __syncthreads();
-    if (p.plain) {
-        for (int t = threadIdx.x; t < 4 * p.nmodes; t += blockDim.x) {
-            const int k = t / p.nmodes, n = p.mode_lo + (t - k * p.nmodes);
-            p.out[t] = cscale(fx_to_double2(seq[2 * k * S1 + n], exq[2 * k]), scale);
+        // products in FP64 (their range is the product of two sequences' ranges);
+        // region b's D^ is -D^ (unpacked)
+        for (int i = threadIdx.x; i <= M; i += blockDim.x) {
+            const longlong2* zi = reinterpret_cast<const longlong2*>(zs) + i;
+            const longlong2* ci = reinterpret_cast<const longlong2*>(cv) + i;
+            const double2 z = fx_to_double2(zi[0], exz[0]), d = fx_to_double2(zi[S2], exz[1]);
+            const double2 dm = p.share ? fx_to_double2(zi[2 * S2], exz[2]) : c2(0.0, 0.0);
+            for (int r = 0; r < nc / 2; ++r) {
+                const double2 cS = fx_to_double2(ci[2 * r * S2], exc[2 * r]);
+                double2 cK = fx_to_double2(ci[(2 * r + 1) * S2], exc[2 * r + 1]);
+                if (r == 1) cK = c2(-cK.x, -cK.y);
+                cv[2 * r * S2 + i] = cmul(z, cS);
+                cv[(2 * r + 1) * S2 + i] = cmul(d, cK);
+                if (p.share) zs[r * S2 + i] = cmul(dm, cK);
+            }
         }
-        return;
+        __syncthreads();
     }
-    // products in FP64 (their range is the product of two sequences' ranges);
-    // region b's D^ is -D^ (unpacked)
-    for (int i = threadIdx.x; i <= M; i += blockDim.x) {
-        const longlong2* zi = reinterpret_cast<const longlong2*>(zs) + i;
-        const longlong2* ci = reinterpret_cast<const longlong2*>(cv) + i;
-        const double2 z = fx_to_double2(zi[0], exz[0]), d = fx_to_double2(zi[S2], exz[1]);
-        const double2 dm = p.share ? fx_to_double2(zi[2 * S2], exz[2]) : c2(0.0, 0.0);
-        for (int r = 0; r < nc / 2; ++r) {
-            const double2 cS = fx_to_double2(ci[2 * r * S2], exc[2 * r]);
-            double2 cK = fx_to_double2(ci[(2 * r + 1) * S2], exc[2 * r + 1]);
-            if (r == 1) cK = c2(-cK.x, -cK.y);
-            cv[2 * r * S2 + i] = cmul(z, cS);
-            cv[(2 * r + 1) * S2 + i] = cmul(d, cK);
-            if (p.share) zs[r * S2 + i] = cmul(dm, cK);
-        }
-    }
-    __syncthreads();
-    for (int t = warp; t < nc + (p.share ? nc / 2 : 0); t += nwarp) {
-        double2* x = t < nc ? cv + t * S2 : zs + (t - nc) * S2;
-        const int ex = fx_even_dft<NB>(reinterpret_cast<longlong2*>(x), fx_quantise(x, S2, lane), M, tw, 1, lane);
-        if (lane == 0) exo[t] = ex;
-    }
-    __syncthreads();
     // (1 / 2 pi) (1 / 2M) of the convolution and 2 pi / M of the modes
     const double c = 0.5 / ((double)M * M);
     const longlong2* cq = reinterpret_cast<const longlong2*>(cv);
