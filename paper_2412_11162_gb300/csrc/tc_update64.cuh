@@ -145,8 +145,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
-__device__ __forceinline__ int acc_int(uint32_t bits) {      // an integer below 2^23 held as a float
-    return __float_as_int(__uint_as_float(bits) + 12582912.0f) - 0x4b400000;
+// An integer held as a float, without the FP64 pipe's conversions.  Weight q sums 64 (q + 1)
+// digit products of at most 2^14: up to 2^22 for q < 4, where one magic number decodes
+// both signs, up to 2^23 beyond (kWide), where the sign is taken out first.
+template <bool kWide>
+__device__ __forceinline__ int acc_int(uint32_t bits) {
+    const float v = __uint_as_float(bits);
+    if (!kWide) return __float_as_int(v + 12582912.0f) - 0x4b400000;
+    const int m = __float_as_int(fabsf(v) + 8388608.0f) - 0x4b000000, sg = (int)bits >> 31;
+    return (m ^ sg) - sg;
 }
 
 struct Upd64Bars {
@@ -309,7 +316,8 @@ __global__ void __launch_bounds__(kUpd64Threads, 1) update64_kernel(int n, int k
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
-                        const int w = (acc_int(x[c]) << 8) + acc_int(y[c]);
+                        const int w = p < 2 ? (acc_int<false>(x[c]) << 8) + acc_int<false>(y[c])
+                                            : (acc_int<true>(x[c]) << 8) + acc_int<true>(y[c]);
                         // unit 2^-56 of the product's scale: weights 44 - 8 q
                         if (p == 0)
                             acc[c] = (i64)w;
