@@ -212,6 +212,9 @@ constexpr double kTolFloor = 1e-14;
 // gains less than 10 %
 constexpr double kTolFloorIr = 4e-16;
 
+// order of the complex64 factors of an n x n system: whole 32-row blocks
+int padded_order(int n) { return (n + 31) / 32 * 32; }
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // nmodes: modes per chunk (every per-mode buffer holds one chunk)
@@ -226,14 +229,15 @@ Workspace plan(const pmlbie_problem* prob, int precision, int nrhs, int nmodes, 
         return p;
     };
     w.A = (double2*)take(sizeof(double2) * nm * n2 * n2);
+    const size_t np2 = padded_order((int)n2);     // the complex64 factors' order
     if (precision == PMLBIE_MIXED) {
-        w.A32 = (float2*)take(sizeof(float2) * nm * n2 * n2);
+        w.A32 = (float2*)take(sizeof(float2) * nm * np2 * np2);
         w.w32 = (float2*)take(sizeof(float2) * nm * n2 * nrhs);
         // inverted 32 x 32 diagonal blocks of the factors (n2 / 32 of L and of U
         // per mode: 1/16 of the factor's bytes) for the correction solves
-        if (n2 % 32 == 0) w.dinv = (float2*)take(sizeof(float2) * nm * diag_inv_elems((int)n2));
-        w.img = (unsigned char*)take(lu_image_bytes((int)n2, (int)nm));
-        w.ptab = (int2*)take(sizeof(int2) * lu_ptab_elems((int)n2, (int)nm));
+        w.dinv = (float2*)take(sizeof(float2) * nm * diag_inv_elems((int)np2));
+        w.img = (unsigned char*)take(lu_image_bytes((int)np2, (int)nm));
+        w.ptab = (int2*)take(sizeof(int2) * lu_ptab_elems((int)np2, (int)nm));
         w.R = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
     }
     const size_t near0 = off;
@@ -244,7 +248,7 @@ Workspace plan(const pmlbie_problem* prob, int precision, int nrhs, int nmodes, 
     w.b2 = (double2*)take(sizeof(double2) * nm * N * nrhs);
     w.B = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
     w.X = (double2*)take(sizeof(double2) * nm * n2 * nrhs);
-    w.piv = (int*)take(sizeof(int) * nm * n2);
+    w.piv = (int*)take(sizeof(int) * nm * np2);
     w.info = (int*)take(sizeof(int) * nm);
     w.nanflag = (int*)take(sizeof(int));
     w.active = (int*)take(sizeof(int) * nm);
@@ -680,7 +684,7 @@ struct SolveStats {
 // into u1.. (already offset to the chunk).  Synchronises the stream at the end.
 static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool point, int lo, int hi, Workspace& w,
                        double2* u1, double2* phi1, double2* u2, double2* phi2, cudaStream_t s, SolveStats& st) {
-    const int N = prob->P.N, nm = hi - lo, n2 = 2 * N;
+    const int N = prob->P.N, nm = hi - lo, n2 = 2 * N, np2 = padded_order(n2);
     cudaEvent_t ev[4], sev[7];
     for (auto& e : ev) PMLBIE_CUDA_TRY(cudaEventCreate(&e));
     for (auto& e : sev) PMLBIE_CUDA_TRY(cudaEventCreate(&e));
@@ -729,12 +733,12 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
             return rc;
         PMLBIE_CUDA_TRY(cudaEventRecord(ev[2], s));
         PMLBIE_CUDA_TRY(cudaMemcpyAsync(w.X, w.B, xbytes, cudaMemcpyDeviceToDevice, s));
-        PMLBIE_CUDA_TRY((batched_lu_solve<double2, double2>(n2, nm, n_rhs, w.A, w.piv, w.X, s)));
+        PMLBIE_CUDA_TRY((batched_lu_solve<double2, double2>(n2, n2, nm, n_rhs, w.A, w.piv, w.X, s)));
     } else {
-        PMLBIE_CUDA_TRY(convert_fro2_c128(n2, nm, w.A, w.A32, w.an, slu));
-        if ((rc = batched_lu_graphed(prob, PMLBIE_MIXED, n2, nm, w.A32, w.piv, w.info, w.img, w.ptab, slu)))
+        PMLBIE_CUDA_TRY(convert_fro2_c128(n2, np2, nm, w.A, w.A32, w.an, slu));
+        if ((rc = batched_lu_graphed(prob, PMLBIE_MIXED, np2, nm, w.A32, w.piv, w.info, w.img, w.ptab, slu)))
             return rc;
-        if (w.dinv) PMLBIE_CUDA_TRY(batched_diag_inv(n2, nm, w.A32, w.dinv, slu));
+        PMLBIE_CUDA_TRY(batched_diag_inv(np2, nm, w.A32, w.dinv, slu));
         PMLBIE_CUDA_TRY(cudaEventRecord(ev[2], slu));
         PMLBIE_CUDA_TRY(cudaEventRecord(ex->join, slu));
         PMLBIE_CUDA_TRY(cudaStreamWaitEvent(s, ex->join, 0));
@@ -793,7 +797,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
                 }
                 PMLBIE_CUDA_TRY(cudaMemcpyAsync(w.active, act.data(), sizeof(int) * nm, cudaMemcpyHostToDevice, s));
             }
-            PMLBIE_CUDA_TRY(refine_step(n2, nm, n_rhs, w.A32, w.piv, w.R, w.w32, w.X, s, w.active, w.dinv, w.ptab));
+            PMLBIE_CUDA_TRY(refine_step(n2, np2, nm, n_rhs, w.A32, w.piv, w.R, w.w32, w.X, s, w.active, w.dinv, w.ptab));
         }
         const int nslow = (int)std::count(slow.begin(), slow.end(), 1);
         if (nslow > 0) {
@@ -820,11 +824,10 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
             std::vector<double> gan(an.begin() + g0, an.begin() + g1), gres(mres.begin() + g0, mres.begin() + g1),
                 gbwd(mbwd.begin() + g0, mbwd.begin() + g1);
             const size_t mat = (size_t)n2 * n2, vec = (size_t)n2 * n_rhs;
-            rc = gmres_refine(n2, gn, n_rhs, w.A + g0 * mat, w.A32 + g0 * mat, w.piv + (size_t)g0 * n2,
+            rc = gmres_refine(n2, np2, gn, n_rhs, w.A + g0 * mat, w.A32 + (size_t)g0 * np2 * np2, w.piv + (size_t)g0 * np2,
                               w.B + g0 * vec, w.X + g0 * vec, gslow, w.active, gm, kGmresM, kGmresCycles, kTolRel,
                               kTolBwd, kTolFloor, gan, s, git, gres, gbwd,
-                              w.dinv ? w.dinv + (size_t)g0 * diag_inv_elems(n2) : nullptr,
-                              w.ptab + (size_t)g0 * lu_ptab_elems(n2, 1));
+                              w.dinv + (size_t)g0 * diag_inv_elems(np2), w.ptab + (size_t)g0 * lu_ptab_elems(np2, 1));
             cudaStreamSynchronize(s);
             cudaFree(gm);
             if (rc) return rc;

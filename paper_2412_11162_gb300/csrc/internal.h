@@ -290,8 +290,8 @@ cudaError_t lu_prepare();
 // used when n is a multiple of 32
 template <typename T, typename TF>
 // ptab: the complex64 factorisation's interchange mapping (batched_lu); then
-// piv is not read
-cudaError_t batched_lu_solve(int n, int batch, int nrhs, const TF* LU, const int* piv, T* B,
+// piv is not read.  The right-hand sides have nv <= n rows (padded factors)
+cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, const int* piv, T* B,
                              cudaStream_t s, const int* active = nullptr, const TF* dinv = nullptr,
                              const int2* ptab = nullptr);
 // inverses of the 32 x 32 diagonal blocks of L (unit lower) and U of every
@@ -299,16 +299,16 @@ cudaError_t batched_lu_solve(int n, int batch, int nrhs, const TF* LU, const int
 cudaError_t batched_diag_inv(int n, int batch, const float2* LU, float2* dinv, cudaStream_t s);
 inline size_t diag_inv_elems(int n) { return (size_t)n * 64; }   // per matrix
 cudaError_t convert_to_c64(int64_t count, const double2* src, float2* dst, cudaStream_t s);
-// complex64 copies of batch n x n complex128 matrices and their squared
-// Frobenius norms (out[b] = |A_b|_F^2) in one pass over A
-cudaError_t convert_fro2_c128(int n, int batch, const double2* A, float2* A32, double* out, cudaStream_t s);
+// complex64 copies of batch n x n complex128 matrices, padded to np x np by an
+// identity, and their squared Frobenius norms (out[b] = |A_b|_F^2) in one pass over A
+cudaError_t convert_fro2_c128(int n, int np, int batch, const double2* A, float2* A32, double* out, cudaStream_t s);
 // Flexible GMRES (FP64, right-preconditioned by the FP32 LU) for the modes with
 // act[b] = 1; X holds the start and receives the solution; act is cleared for
 // converged modes (relative residual <= tol or normwise backward error
 // |r| / (|A|_F |x| + |b|) <= tol_bw; an2 = |A_b|_F^2), mode_res / mode_bwd
 // receive their final relative residuals and backward errors.
 size_t gmres_scratch_bytes(int n, int batch, int nrhs, int m);
-int gmres_refine(int n, int batch, int nrhs, const double2* A, const float2* LU32, const int* piv,
+int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const float2* LU32, const int* piv,
                  const double2* B, double2* X, std::vector<int>& act, int* active_dev, void* scratch, int m,
                  int max_cycles, double tol, double tol_bw, double tol_floor, const std::vector<double>& an2,
                  cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
@@ -317,7 +317,7 @@ int gmres_refine(int n, int batch, int nrhs, const double2* A, const float2* LU3
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,
                           const double2* B, double2* R, double* rnorm, double* bnorm, double* xnorm,
                           cudaStream_t s, const int* active = nullptr);
-cudaError_t refine_step(int n, int batch, int nrhs, const float2* LU32, const int* piv,
+cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const int* piv,
                         const double2* R, float2* work32, double2* X, cudaStream_t s,
                         const int* active = nullptr, const float2* dinv = nullptr, const int2* ptab = nullptr);
 

@@ -760,8 +760,9 @@ __global__ void __launch_bounds__(256) swap_trsm_kernel(int n, int k0, int kb, i
 // diagonal blocks of L and U, diag_inv_kernel; n a multiple of 32) a
 // diagonal block is applied as a matrix-vector product by one warp per
 // right-hand side, 32 independent products instead of a 32-step dependent
-// substitution that the other warps wait for.  Matrices whose active flag is
-// 0 are skipped (converged modes).
+// substitution that the other warps wait for.  The right-hand sides have nv <= n rows
+// (a factor padded to whole 32-row blocks by an identity; the rows beyond nv are zero
+// and stay so).  Matrices whose active flag is 0 are skipped (converged modes).
 constexpr int kSolveR = 8;
 
 template <typename T> __device__ __forceinline__ T widen(float2 v) { return Cx<T>::mk(v.x, v.y); }
@@ -805,7 +806,7 @@ __device__ __forceinline__ void block_pair_update(const TF* col, int n, const T*
 }
 
 template <typename T, typename TF, int RM>
-__global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nrhs, int Rg, const TF* LU, const int* perm,
+__global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nv, int nrhs, int Rg, const TF* LU, const int* perm,
                                                        T* B, const int* active, const TF* dinv, const int2* ptab) {
     const int R = RM == 1 ? 1 : Rg;    // compile-time 1 in the single-wave variant
     const int b = blockIdx.x, r0 = blockIdx.y * R, nr = RM == 1 ? 1 : min(R, nrhs - r0);
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nrhs, int Rg, 
     T* sx = reinterpret_cast<T*>(smraw);                     // n x R entries, sx[i * R + q]
     const TF* a = LU + (size_t)b * n * n;
     const int* pm = perm + (size_t)b * n;
-    T* x = B + (size_t)b * n * nrhs;
+    T* x = B + (size_t)b * nv * nrhs;
     __shared__ __align__(16) TF sD[kNB * kNB];     // diagonal block, sD[col * kNB + row]
     constexpr int kDiagPer = (int)(kNB * kNB * sizeof(TF) / (512 * 16));   // 16-byte pieces per thread
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -825,7 +826,7 @@ __global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nrhs, int Rg, 
     const int2* pt = ptab ? ptab + (size_t)b * nblk * 2 * kNB : nullptr;
     for (int idx = tid; idx < n * nr; idx += blockDim.x) {
         const int i = idx / nr, q = idx - i * nr;
-        sx[i * R + q] = x[(size_t)(pt ? i : pm[i]) * nrhs + r0 + q];
+        sx[i * R + q] = i < nv ? x[(size_t)(pt ? i : pm[i]) * nrhs + r0 + q] : Cx<T>::mk(0, 0);
     }
     // the pair path: full blocks only, and with several right-hand sides only
     // for complex64 accumulators (register budget of 512 threads)
@@ -1013,7 +1014,7 @@ __global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nrhs, int Rg, 
         }
         __syncthreads();
     }
-    for (int idx = tid; idx < n * nr; idx += blockDim.x) {
+    for (int idx = tid; idx < nv * nr; idx += blockDim.x) {
         const int i = idx / nr, q = idx - i * nr;
         x[(size_t)i * nrhs + r0 + q] = sx[i * R + q];
     }
@@ -1140,21 +1141,38 @@ __device__ __forceinline__ float f32_of_halves(uint32_t lo, uint32_t hi) {
     return __uint_as_float(sg | bits);
 }
 
-// complex64 copy of every matrix and |A_b|_F^2 in the same pass over A:
-// grid (blocks per matrix, matrices), out zeroed beforehand.  The entries are
+// complex64 copy of every matrix, padded from n to np = 32 ceil(n / 32) rows and
+// columns with an identity (so that the factorisation and its solves see whole 32-row
+// blocks: with ragged n the solves of n = 482 took 1.1 ms of a 7.8 ms run, three times
+// those of n = 512), and |A_b|_F^2 in the same pass over A: grid (blocks of columns per
+// matrix, matrices), out zeroed beforehand.  The entries are
 // read as 32-bit words and converted with integer operations; the squares
 // accumulate in FP32 per thread (the norm enters only the backward-error test
 // of the refinement, where 1e-5 relative is ample) and in FP64 across warps.
-__global__ void c64_fro2_kernel(int64_t per, const double2* A, float2* A32, double* out) {
+__global__ void c64_fro2_kernel(int n, int np, const double2* A, float2* A32, double* out) {
     __shared__ double sh[8];
-    const uint4* a = reinterpret_cast<const uint4*>(A + (size_t)blockIdx.y * per);
-    float2* d = A32 + (size_t)blockIdx.y * per;
+    const uint4* a = reinterpret_cast<const uint4*>(A + (size_t)blockIdx.y * n * n);
+    float2* d = A32 + (size_t)blockIdx.y * np * np;
     float acc = 0.0f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < per; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 v = __ldcs(a + i);      // read once: streaming
-        const float2 f = make_float2(f32_of_halves(v.x, v.y), f32_of_halves(v.z, v.w));
-        d[i] = f;
-        acc = __fmaf_rn(f.x, f.x, __fmaf_rn(f.y, f.y, acc));
+    if (n == np) {
+        const int64_t per = (int64_t)n * n;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < per; i += (int64_t)gridDim.x * blockDim.x) {
+            const uint4 v = __ldcs(a + i);      // read once: streaming
+            const float2 f = make_float2(f32_of_halves(v.x, v.y), f32_of_halves(v.z, v.w));
+            d[i] = f;
+            acc = __fmaf_rn(f.x, f.x, __fmaf_rn(f.y, f.y, acc));
+        }
+    } else {
+        for (int c = blockIdx.x; c < np; c += gridDim.x)
+            for (int r = threadIdx.x; r < np; r += blockDim.x) {
+                float2 f = make_float2(r == c ? 1.0f : 0.0f, 0.0f);
+                if (r < n && c < n) {
+                    const uint4 v = __ldcs(a + (size_t)c * n + r);
+                    f = make_float2(f32_of_halves(v.x, v.y), f32_of_halves(v.z, v.w));
+                    acc = __fmaf_rn(f.x, f.x, __fmaf_rn(f.y, f.y, acc));
+                }
+                d[(size_t)c * np + r] = f;
+            }
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffff, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = (double)acc;
@@ -1414,7 +1432,7 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
 }
 
 template <typename T, typename TF>
-cudaError_t batched_lu_solve(int n, int batch, int nrhs, const TF* LU, const int* piv, T* B,
+cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, const int* piv, T* B,
                              cudaStream_t s, const int* active, const TF* dinv, const int2* ptab) {
     // right-hand sides per CTA: up to kSolveR, as many as fit in shared memory
     // (about 200 KB for the group)
@@ -1429,13 +1447,13 @@ cudaError_t batched_lu_solve(int n, int batch, int nrhs, const TF* LU, const int
             cudaError_t e = allow_max_smem(lu_solve_kernel<T, TF, 1>);
             if (e != cudaSuccess) return e;
         }
-        lu_solve_kernel<T, TF, 1><<<g, 512, sm, s>>>(n, nrhs, R, LU, piv, B, active, dinv, ptab);
+        lu_solve_kernel<T, TF, 1><<<g, 512, sm, s>>>(n, nv, nrhs, R, LU, piv, B, active, dinv, ptab);
     } else {
         if (big) {
             cudaError_t e = allow_max_smem(lu_solve_kernel<T, TF, kSolveR>);
             if (e != cudaSuccess) return e;
         }
-        lu_solve_kernel<T, TF, kSolveR><<<g, 512, sm, s>>>(n, nrhs, R, LU, piv, B, active, dinv, ptab);
+        lu_solve_kernel<T, TF, kSolveR><<<g, 512, sm, s>>>(n, nv, nrhs, R, LU, piv, B, active, dinv, ptab);
     }
     count_launch();
     return cudaGetLastError();
@@ -1447,11 +1465,11 @@ template cudaError_t batched_lu<double2>(int, int, double2*, int*, int*, cudaStr
                                           const LuSide*, cudaEvent_t*, size_t);
 template cudaError_t batched_lu<float2>(int, int, float2*, int*, int*, cudaStream_t, unsigned char*, int2*,
                                          const LuSide*, cudaEvent_t*, size_t);
-template cudaError_t batched_lu_solve<double2, double2>(int, int, int, const double2*, const int*, double2*,
+template cudaError_t batched_lu_solve<double2, double2>(int, int, int, int, const double2*, const int*, double2*,
                                                         cudaStream_t, const int*, const double2*, const int2*);
-template cudaError_t batched_lu_solve<float2, float2>(int, int, int, const float2*, const int*, float2*,
+template cudaError_t batched_lu_solve<float2, float2>(int, int, int, int, const float2*, const int*, float2*,
                                                       cudaStream_t, const int*, const float2*, const int2*);
-template cudaError_t batched_lu_solve<double2, float2>(int, int, int, const float2*, const int*, double2*,
+template cudaError_t batched_lu_solve<double2, float2>(int, int, int, int, const float2*, const int*, double2*,
                                                        cudaStream_t, const int*, const float2*, const int2*);
 
 cudaError_t convert_to_c64(int64_t count, const double2* src, float2* dst, cudaStream_t s) {
@@ -1473,14 +1491,14 @@ cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const do
     return cudaGetLastError();
 }
 
-cudaError_t convert_fro2_c128(int n, int batch, const double2* A, float2* A32, double* out, cudaStream_t s) {
+cudaError_t convert_fro2_c128(int n, int np, int batch, const double2* A, float2* A32, double* out, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double) * batch, s);
     if (e != cudaSuccess) return e;
     const int64_t per = (int64_t)n * n;
     // about 32 CTAs of 256 threads per SM over all matrices (enough loads in flight)
     const int64_t want = std::max<int64_t>(1, (152 * 32 + batch - 1) / batch);
     dim3 g((unsigned)std::min<int64_t>((per + 255) / 256, want), batch);
-    c64_fro2_kernel<<<g, 256, 0, s>>>(per, A, A32, out);
+    c64_fro2_kernel<<<g, 256, 0, s>>>(n, np, A, A32, out);
     count_launch();
     return cudaGetLastError();
 }
@@ -1493,13 +1511,13 @@ cudaError_t batched_diag_inv(int n, int batch, const float2* LU, float2* dinv, c
     return cudaGetLastError();
 }
 
-cudaError_t refine_step(int n, int batch, int nrhs, const float2* LU32, const int* piv,
+cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const int* piv,
                         const double2* R, float2* work32, double2* X, cudaStream_t s, const int* active,
                         const float2* dinv, const int2* ptab) {
     int64_t cnt = (int64_t)batch * n * nrhs;
     cudaError_t e = convert_to_c64(cnt, R, work32, s);
     if (e != cudaSuccess) return e;
-    e = batched_lu_solve<float2, float2>(n, batch, nrhs, LU32, piv, work32, s, active, dinv, ptab);
+    e = batched_lu_solve<float2, float2>(np, n, batch, nrhs, LU32, piv, work32, s, active, dinv, ptab);
     if (e != cudaSuccess) return e;
     add_correction_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(cnt, (int64_t)n * nrhs, work32, X, active);
     count_launch();
