@@ -700,7 +700,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
     int rc;
     PMLBIE_CUDA_TRY(cudaEventRecord(ev[0], s));
     if ((rc = build_system(prob, precision, w, lo, hi, s, sev))) return rc;
-    // mixed: the right-hand sides (the FP64 block product, FP64-pipe bound) are
+    // mixed: the right-hand sides are
     // formed on s beside the complex64 conversion and factorisation, which run
     // on the high-priority stream and read / write only the FP32 copy; they
     // join before the refinement.  FP64: the factorisation overwrites w.A, so

@@ -313,6 +313,14 @@ int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const flo
                  int max_cycles, double tol, double tol_bw, double tol_floor, const std::vector<double>& an2,
                  cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
                  const float2* dinv = nullptr, const int2* ptab = nullptr);
+// Y[b] rows row0 .. n - 1 += sign A[b] [x0; x1] (n even; x0, x1 per mode [n/2][nrhs], modes
+// xs apart; Y [b][n][nrhs]) on the tensor cores (tc_product64.cuh)
+// From two right-hand sides on: the product's time hardly depends on their number up to 8
+// (n = 1600, 128 modes, one: 1.87 ms against 1.58 ms of the FP64 kernel, whose time grows
+// with them; n = 768, 96 modes, eight: 0.41 ms against 2.19 ms).
+constexpr int kProductRhs = 2;
+cudaError_t add_product_c128(int n, int row0, int nrhs, int batch, const double2* A, const double2* x0, const double2* x1,
+                             size_t xs, double2* Y, double sign, const int* active, cudaStream_t s);
 // R = B - A X with |R|^2, |B|^2, |X|^2 per (matrix, rhs)
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,
                           const double2* B, double2* R, double* rnorm, double* bnorm, double* xnorm,

@@ -1124,6 +1124,8 @@ cudaError_t launch_block_rhs(const pmlbie_problem* prob, int n_rhs, int nm, cons
     const int N = prob->P.N;
     cudaError_t e = cudaMemsetAsync(B, 0, sizeof(double2) * (size_t)nm * 2 * N * n_rhs, s);
     if (e != cudaSuccess) return e;
+    if (n_rhs >= kProductRhs)
+        return add_product_c128(2 * N, N, n_rhs, nm, A, b1, b2, (size_t)N * n_rhs, B, 1.0, nullptr, s);
     dim3 g((unsigned)(((size_t)N * n_rhs + 255) / 256), (unsigned)((2 * N + kBrhsCols - 1) / kBrhsCols), nm);
     block_rhs_kernel<<<g, 256, 0, s>>>(N, n_rhs, A, b1, b2, B);
     count_launch();

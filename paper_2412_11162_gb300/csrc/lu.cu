@@ -29,6 +29,7 @@
 #include "internal.h"
 #include "tc_update.cuh"
 #include "tc_update64.cuh"
+#include "tc_product64.cuh"
 
 namespace pmlbie {
 
@@ -1479,13 +1480,46 @@ cudaError_t convert_to_c64(int64_t count, const double2* src, float2* dst, cudaS
     return cudaGetLastError();
 }
 
+cudaError_t add_product_c128(int n, int row0, int nrhs, int batch, const double2* A, const double2* x0, const double2* x1,
+                             size_t xs, double2* Y, double sign, const int* active, cudaStream_t s) {
+    cudaError_t e = allow_max_smem(tcu::product64_kernel);
+    if (e != cudaSuccess) return e;
+    tcu::ProductArgs a;
+    a.n = n;
+    a.row0 = row0;
+    a.nc = n / 2;
+    a.nrhs = nrhs;
+    a.groups = (nrhs + tcu::kProdRhs - 1) / tcu::kProdRhs;
+    a.A = A;
+    a.x0 = x0;
+    a.x1 = x1;
+    a.xs = xs;
+    a.Y = Y;
+    a.sign = sign;
+    a.active = active;
+    // column splits: four waves of two CTAs per SM when the rows and modes give fewer
+    const int gx = (n - row0 + tcu::kProdRows - 1) / tcu::kProdRows * a.groups;
+    const int chunks = 2 * ((a.nc + tcu::kProdCols - 1) / tcu::kProdCols);
+    const long long ctas = (long long)gx * batch;
+    const int splits = (int)std::max(1ll, std::min((long long)chunks, (4 * 2 * 152 + ctas - 1) / ctas));
+    tcu::product64_kernel<<<dim3(gx, splits, batch), tcu::kProdThreads, tcu::kProdSmem, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,
                           const double2* B, double2* R, double* rnorm, double* bnorm, double* xnorm,
                           cudaStream_t s, const int* active) {
     cudaError_t e = cudaMemcpyAsync(R, B, sizeof(double2) * (size_t)batch * n * nrhs, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
-    dim3 g((unsigned)(((size_t)n * nrhs + 255) / 256), (unsigned)((n + kResCols - 1) / kResCols), batch);
-    residual_kernel<<<g, 256, 0, s>>>(n, nrhs, A, X, R, active);
+    if (nrhs >= kProductRhs) {
+        const size_t half = (size_t)(n / 2) * nrhs;
+        e = add_product_c128(n, 0, nrhs, batch, A, X, X + half, 2 * half, R, -1.0, active, s);
+        if (e != cudaSuccess) return e;
+    } else {
+        dim3 g((unsigned)(((size_t)n * nrhs + 255) / 256), (unsigned)((n + kResCols - 1) / kResCols), batch);
+        residual_kernel<<<g, 256, 0, s>>>(n, nrhs, A, X, R, active);
+    }
     norms3_kernel<<<dim3(batch, nrhs), 256, 0, s>>>(n, nrhs, R, B, X, rnorm, bnorm, xnorm, active);
     count_launch(2);
     return cudaGetLastError();
