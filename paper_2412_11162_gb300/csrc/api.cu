@@ -1196,8 +1196,19 @@ int pmlbie_field(pmlbie_problem* prob, int n_pts, const double* rho, const doubl
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nm = (size_t)(mode_hi - mode_lo), N = prob->P.N;
     double *d_rho = nullptr, *d_z = nullptr;
-    int* d_reg = nullptr;
+    int* d_map = nullptr;
     double2* coef = nullptr;
+    // the points of the upper medium first (each medium's densities meet whole row blocks)
+    std::vector<int> order;
+    std::vector<double> orho, oz;
+    for (int g = 0; g < 2; ++g)
+        for (int p = 0; p < n_pts; ++p)
+            if (region[p] == g) {
+                order.push_back(p);
+                orho.push_back(rho[p]);
+                oz.push_back(z[p]);
+            }
+    const int nup = (int)std::count(region, region + n_pts, 0);
     struct Free {
         double** a;
         double** b;
@@ -1209,18 +1220,18 @@ int pmlbie_field(pmlbie_problem* prob, int n_pts, const double* rho, const doubl
             if (*c) cudaFree(*c);
             if (*d) cudaFree(*d);
         }
-    } fr{&d_rho, &d_z, &d_reg, &coef};
+    } fr{&d_rho, &d_z, &d_map, &coef};
     if (cudaMalloc(&d_rho, sizeof(double) * n_pts) != cudaSuccess ||
         cudaMalloc(&d_z, sizeof(double) * n_pts) != cudaSuccess ||
-        cudaMalloc(&d_reg, sizeof(int) * n_pts) != cudaSuccess ||
+        cudaMalloc(&d_map, sizeof(int) * n_pts) != cudaSuccess ||
         cudaMalloc(&coef, sizeof(double2) * 2 * nm * N * n_pts) != cudaSuccess) {
         cudaGetLastError();
         return fail(PMLBIE_ENOMEM, "field: scratch allocation failed");
     }
-    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_rho, rho, sizeof(double) * n_pts, cudaMemcpyHostToDevice, s));
-    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_z, z, sizeof(double) * n_pts, cudaMemcpyHostToDevice, s));
-    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_reg, region, sizeof(int) * n_pts, cudaMemcpyHostToDevice, s));
-    PMLBIE_CUDA_TRY(launch_field(prob, n_pts, d_rho, d_z, d_reg, mode_lo, mode_hi, n_rhs, (const double2*)dev_u1,
+    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_rho, orho.data(), sizeof(double) * n_pts, cudaMemcpyHostToDevice, s));
+    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_z, oz.data(), sizeof(double) * n_pts, cudaMemcpyHostToDevice, s));
+    PMLBIE_CUDA_TRY(cudaMemcpyAsync(d_map, order.data(), sizeof(int) * n_pts, cudaMemcpyHostToDevice, s));
+    PMLBIE_CUDA_TRY(launch_field(prob, n_pts, nup, d_rho, d_z, d_map, mode_lo, mode_hi, n_rhs, (const double2*)dev_u1,
                                  (const double2*)dev_phi1, (const double2*)dev_u2, (const double2*)dev_phi2, coef,
                                  (double2*)dev_out, s));
     PMLBIE_CUDA_TRY(cudaStreamSynchronize(s));

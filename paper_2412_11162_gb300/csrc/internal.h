@@ -228,8 +228,8 @@ cudaError_t launch_expand_waves(int N, int nmodes, int mode_lo, int n_src, int n
 // Scattered-field modes at observation points (rho, z, region 0 upper / 1 lower,
 // device arrays): coef scratch npts x N x (mode_hi - mode_lo) x 2 complex;
 // densities and out laid out [mode - mode_lo][node or point][rhs]
-cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prho, const double* pz,
-                         const int* preg, int mode_lo, int mode_hi, int nrhs, const double2* u1,
+cudaError_t launch_field(const pmlbie_problem* prob, int npts, int nup, const double* prho, const double* pz,
+                         const int* map, int mode_lo, int mode_hi, int nrhs, const double2* u1,
                          const double2* phi1, const double2* u2, const double2* phi2, double2* coef, double2* out,
                          cudaStream_t s);
 // nm: modes in the chunk (A, b1, b2, B, X hold nm modes)
@@ -313,14 +313,22 @@ int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const flo
                  int max_cycles, double tol, double tol_bw, double tol_floor, const std::vector<double>& an2,
                  cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
                  const float2* dinv = nullptr, const int2* ptab = nullptr);
-// Y[b] rows row0 .. n - 1 += sign A[b] [x0; x1] (n even; x0, x1 per mode [n/2][nrhs], modes
-// xs apart; Y [b][n][nrhs]) on the tensor cores (tc_product64.cuh)
-// From two right-hand sides on: the product's time hardly depends on their number up to 8
-// (n = 1600, 128 modes, one: 1.87 ms against 1.58 ms of the FP64 kernel, whose time grows
-// with them; n = 768, 96 modes, eight: 0.41 ms against 2.19 ms).
-constexpr int kProductRhs = 2;
-cudaError_t add_product_c128(int n, int row0, int nrhs, int batch, const double2* A, const double2* x0, const double2* x1,
-                             size_t xs, double2* Y, double sign, const int* active, cudaStream_t s);
+// Y[b] += sign A[b] [x0; x1] for the rows row0 .. rows - 1 of `batch` matrices A[b] of 2 nc
+// columns (column-major, leading dimension ld, as apart): columns 0 .. nc - 1 meet x0[b],
+// the others x1[b] ([nc][nrhs], xs apart); rows from `split` on take x0s, x1s instead.
+// Row i of the result goes to row map[i] (map null: i) of Y[b] ([.][nrhs], ys apart).
+struct ProductArgs {
+    int ld = 0, row0 = 0, split = 0, rows = 0, nc = 0, nrhs = 0;
+    const double2 *A = nullptr, *x0 = nullptr, *x1 = nullptr, *x0s = nullptr, *x1s = nullptr;
+    size_t as = 0, xs = 0, ys = 0;
+    double2* Y = nullptr;
+    double sign = 1.0;
+    const int *active = nullptr, *map = nullptr;
+};
+// From two right-hand sides on, the tensor cores (tc_product64.cuh): their time hardly
+// depends on the number up to 8 (n = 1600, 128 modes, one: 1.87 ms against 1.58 ms of the
+// FP64 kernel, whose time grows with them; n = 768, 96 modes, eight: 0.41 against 2.19 ms).
+cudaError_t add_product_c128(const ProductArgs& a, int batch, cudaStream_t s);
 // R = B - A X with |R|^2, |B|^2, |X|^2 per (matrix, rhs)
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,
                           const double2* B, double2* R, double* rnorm, double* bnorm, double* xnorm,

@@ -850,33 +850,6 @@ __global__ void rhs_kernel(RhsArgs a) {
     }
 }
 
-// B_n = [0; A_n[N:2N, 0:N] b1 + A_n[N:2N, N:2N] b2], B laid out [mode][2N][rhs]
-// and zeroed beforehand.  Grid (lower-half rows x rhs / 256, column chunks of
-// kBrhsCols, modes): each thread sums one chunk of its row and adds it with
-// atomics, so that every mode's half matrix is streamed by many SMs at once.
-constexpr int kBrhsCols = 32;
-__global__ void block_rhs_kernel(int N, int nrhs, const double2* A, const double2* b1, const double2* b2,
-                                 double2* B) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)N * nrhs) return;
-    const int r = (int)(idx % nrhs), row = N + (int)(idx / nrhs);
-    const int t = blockIdx.z;
-    const size_t n2 = 2 * (size_t)N;
-    const int c0 = blockIdx.y * kBrhsCols, c1 = min((int)n2, c0 + kBrhsCols);
-    const double2* An = A + (size_t)t * n2 * n2;
-    const double2* v1 = b1 + (size_t)t * N * nrhs;
-    const double2* v2 = b2 + (size_t)t * N * nrhs;
-    double2 acc = c2(0.0, 0.0);
-#pragma unroll 8
-    for (int c = c0; c < c1; ++c) {
-        const double2 v = c < N ? v1[(size_t)c * nrhs + r] : v2[(size_t)(c - N) * nrhs + r];
-        acc = cadd(acc, cmul(An[(size_t)c * n2 + row], v));
-    }
-    double* o = reinterpret_cast<double*>(B + ((size_t)t * n2 + row) * nrhs + r);
-    atomicAdd(o, acc.x);
-    atomicAdd(o + 1, acc.y);
-}
-
 __global__ void outputs_kernel(int N, int nmodes, int nrhs, const double2* X, const double2* b1,
                                const double2* b2, double2* u1, double2* phi1, double2* u2,
                                double2* phi2) {
@@ -1124,12 +1097,19 @@ cudaError_t launch_block_rhs(const pmlbie_problem* prob, int n_rhs, int nm, cons
     const int N = prob->P.N;
     cudaError_t e = cudaMemsetAsync(B, 0, sizeof(double2) * (size_t)nm * 2 * N * n_rhs, s);
     if (e != cudaSuccess) return e;
-    if (n_rhs >= kProductRhs)
-        return add_product_c128(2 * N, N, n_rhs, nm, A, b1, b2, (size_t)N * n_rhs, B, 1.0, nullptr, s);
-    dim3 g((unsigned)(((size_t)N * n_rhs + 255) / 256), (unsigned)((2 * N + kBrhsCols - 1) / kBrhsCols), nm);
-    block_rhs_kernel<<<g, 256, 0, s>>>(N, n_rhs, A, b1, b2, B);
-    count_launch();
-    return cudaGetLastError();
+    // B_n = [0; A_n[N:2N, 0:N] b1 + A_n[N:2N, N:2N] b2], B laid out [mode][2N][rhs]
+    ProductArgs a;
+    a.ld = a.split = a.rows = 2 * N;
+    a.row0 = a.nc = N;
+    a.nrhs = n_rhs;
+    a.A = A;
+    a.x0 = b1;
+    a.x1 = b2;
+    a.as = 4 * (size_t)N * N;
+    a.xs = (size_t)N * n_rhs;
+    a.ys = 2 * a.xs;
+    a.Y = B;
+    return add_product_c128(a, nm, s);
 }
 
 cudaError_t launch_outputs(const pmlbie_problem* prob, int n_rhs, int nm, const double2* X,
@@ -1155,12 +1135,11 @@ namespace {
 // ---------------------------------------------------------------------------
 struct FieldArgs {
     DeviceTables T;
-    int N, M, npts, mode_lo, nmodes;
+    int N, M, npts, nup, mode_lo, nmodes;
     double w1, w2, h;
-    const double* prho;   // points
+    const double* prho;   // points, those of the upper medium (nup) first
     const double* pz;
-    const int* preg;
-    double2* coef;        // [p][m][nmodes][2]
+    double2* coef;        // [nmodes][2][N][npts]
 };
 
 // S~ and K~ of one (physical point x = (rx, 0, zx), node m) pair at the M/2+1
@@ -1218,9 +1197,9 @@ __global__ void field_kernel(FieldArgs a) {
     double2* cs = smem + 3 * M / 4;
     double2* buf = cs + S1 + warp * 2 * S1;
     point_tables(a.T, M, tw, cs);
-    const int p = blockIdx.y, m = blockIdx.x * nw + warp;
-    if (m >= a.N) return;
-    const int reg = a.preg[p];
+    const int p = blockIdx.y * nw + warp, m = blockIdx.x;
+    if (p >= a.npts) return;
+    const int reg = p >= a.nup;
     const double sg = reg == 0 ? 1.0 : -1.0;
     int exS, exK;
     point_node_modes<NB>(a.T, M, reg == 0 ? a.w1 : a.w2, sg, a.prho[p], a.pz[p], m, cs, tw, a.T.ph[reg],
@@ -1228,10 +1207,11 @@ __global__ void field_kernel(FieldArgs a) {
     const longlong2* f = reinterpret_cast<const longlong2*>(buf);
     const double scale = 2.0 * kPi / M;
     const double fs = 0.5 * sg * scale * a.h * a.T.Wphi[m], fk = -0.5 * scale * a.h * a.T.Wu[m];
-    double2* o = a.coef + ((size_t)p * a.N + m) * a.nmodes * 2;
+    // [mode][S of every node, K of every node][point]: the columns of the field's product
     for (int t = lane; t < a.nmodes; t += 32) {
-        o[2 * t] = cscale(fx_to_double2(f[a.mode_lo + t], exS), fs);
-        o[2 * t + 1] = cscale(fx_to_double2(f[S1 + a.mode_lo + t], exK), fk);
+        double2* o = a.coef + ((size_t)t * 2 * a.N + m) * a.npts + p;
+        o[0] = cscale(fx_to_double2(f[a.mode_lo + t], exS), fs);
+        o[(size_t)a.N * a.npts] = cscale(fx_to_double2(f[S1 + a.mode_lo + t], exK), fk);
     }
 }
 
@@ -1268,31 +1248,11 @@ __global__ void point_rhs_kernel(DeviceTables T, int N, int M, int nrhs, int mod
     }
 }
 
-// out[t][p][r] = sum_m cS[p][m][t] phi[t][m][r] + cK[p][m][t] u[t][m][r]
-__global__ void field_contract_kernel(int N, int npts, int nmodes, int nrhs, const int* preg, const double2* coef,
-                                      const double2* u1, const double2* phi1, const double2* u2,
-                                      const double2* phi2, double2* out) {
-    const size_t tot = (size_t)nmodes * npts * nrhs;
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= tot) return;
-    const int t = (int)(k % nmodes);
-    const size_t pr = k / nmodes;
-    const int r = (int)(pr % nrhs), p = (int)(pr / nrhs);
-    const bool up = preg[p] == 0;
-    const double2* u = up ? u1 : u2;
-    const double2* ph = up ? phi1 : phi2;
-    double2 acc = c2(0.0, 0.0);
-    for (int m = 0; m < N; ++m) {
-        const double2* c = coef + (((size_t)p * N + m) * nmodes + t) * 2;
-        const size_t di = ((size_t)t * N + m) * nrhs + r;
-        acc = cadd(acc, cadd(cmul(c[0], ph[di]), cmul(c[1], u[di])));
-    }
-    out[((size_t)t * npts + p) * nrhs + r] = acc;
-}
 }  // namespace
 
-cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prho, const double* pz,
-                         const int* preg, int mode_lo, int mode_hi, int nrhs, const double2* u1,
+// points 0 .. nup - 1 lie in the upper medium; map: their places in the caller's order
+cudaError_t launch_field(const pmlbie_problem* prob, int npts, int nup, const double* prho, const double* pz,
+                         const int* map, int mode_lo, int mode_hi, int nrhs, const double2* u1,
                          const double2* phi1, const double2* u2, const double2* phi2, double2* coef, double2* out,
                          cudaStream_t s) {
     FieldArgs a;
@@ -1300,6 +1260,7 @@ cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prh
     a.N = prob->P.N;
     a.M = prob->P.M;
     a.npts = npts;
+    a.nup = nup;
     a.mode_lo = mode_lo;
     a.nmodes = mode_hi - mode_lo;
     a.w1 = prob->P.k1;
@@ -1307,23 +1268,36 @@ cudaError_t launch_field(const pmlbie_problem* prob, int npts, const double* prh
     a.h = prob->H.h;
     a.prho = prho;
     a.pz = pz;
-    a.preg = preg;
     a.coef = coef;
     const int nw = 4;
     const size_t smem = point_smem(a.M, nw);
-    const cudaError_t ef = with_half_class(a.M, [&](auto nb) {
+    cudaError_t e = with_half_class(a.M, [&](auto nb) {
         constexpr int NB = decltype(nb)::value;
         cudaError_t e = smem > 48 * 1024 ? allow_max_smem(field_kernel<NB>) : cudaSuccess;
         if (e != cudaSuccess) return e;
-        field_kernel<NB><<<dim3((a.N + nw - 1) / nw, npts), 32 * nw, smem, s>>>(a);
+        field_kernel<NB><<<dim3(a.N, (npts + nw - 1) / nw), 32 * nw, smem, s>>>(a);
         return cudaGetLastError();
     });
-    if (ef != cudaSuccess) return ef;
-    const size_t tot = (size_t)a.nmodes * npts * nrhs;
-    field_contract_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(a.N, npts, a.nmodes, nrhs, preg, coef, u1,
-                                                                        phi1, u2, phi2, out);
-    count_launch(2);
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    count_launch();
+    // out[t][p][r] = sum_m cS[t][m][p] phi[t][m][r] + cK[t][m][p] u[t][m][r]
+    ProductArgs g;
+    g.ld = g.rows = npts;
+    g.split = nup;
+    g.nc = a.N;
+    g.nrhs = nrhs;
+    g.A = coef;
+    g.x0 = phi1;
+    g.x1 = u1;
+    g.x0s = phi2;
+    g.x1s = u2;
+    g.as = 2 * (size_t)a.N * npts;
+    g.xs = (size_t)a.N * nrhs;
+    g.ys = (size_t)npts * nrhs;
+    g.Y = out;
+    g.map = map;
+    if ((e = cudaMemsetAsync(out, 0, sizeof(double2) * (size_t)a.nmodes * npts * nrhs, s)) != cudaSuccess) return e;
+    return add_product_c128(g, a.nmodes, s);
 }
 
 cudaError_t launch_point_rhs(const pmlbie_problem* prob, int n_rhs, int mode_lo, int mode_hi,

@@ -68,25 +68,19 @@ __device__ __forceinline__ unsigned mag_hi(double2 v) {
     return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
 
-// Columns 0 .. nc - 1 of A meet x0, columns nc .. 2 nc - 1 x1 (n = 2 nc; each mode's
-// [nc][nrhs], modes xs apart).  Grid (row blocks x groups of 8 right-hand sides, column
+// Grid (row blocks of either side of `split` x groups of 8 right-hand sides, column
 // splits, modes).
-struct ProductArgs {
-    int n, row0, nc, nrhs, groups;
-    const double2 *A, *x0, *x1;
-    size_t xs;
-    double2* Y;               // [mode][n][nrhs]
-    double sign;
-    const int* active;
-};
-
-__global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs a) {
+__global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs a, int groups) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const int b = blockIdx.z;
     if (a.active && !a.active[b]) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = tid & 127, hf = tid >> 7;
-    const int rb = blockIdx.x / a.groups, r0 = (blockIdx.x - rb * a.groups) * kProdRhs;
-    const int nq = min(kProdRhs, a.nrhs - r0), row = a.row0 + rb * kProdRows + r;
+    const int rb = blockIdx.x / groups, r0 = (blockIdx.x - rb * groups) * kProdRhs;
+    const int nb0 = (a.split - a.row0 + kProdRows - 1) / kProdRows;
+    const bool upper = rb < nb0;
+    const int nq = min(kProdRhs, a.nrhs - r0), end = upper ? a.split : a.rows;
+    const int row = (upper ? a.row0 + rb * kProdRows : a.split + (rb - nb0) * kProdRows) + r;
+    const double2 *x0 = upper ? a.x0 : a.x0s, *x1 = upper ? a.x1 : a.x1s;
     unsigned* rmax = reinterpret_cast<unsigned*>(sm + kProdOffMax);
     int* exq = reinterpret_cast<int*>(sm + kProdOffEx);
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kProdOffBar);
@@ -106,7 +100,7 @@ __global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs 
     const uint32_t tmem = *tm, sbase = smem_u32(sm);
     const int per = (a.nc + kProdCols - 1) / kProdCols, total = 2 * per;
     const int k0 = (int)((long long)total * blockIdx.y / gridDim.y), k1 = (int)((long long)total * (blockIdx.y + 1) / gridDim.y);
-    const double2* Ab = a.A + (size_t)b * a.n * a.n + row;
+    const double2* Ab = a.A + (size_t)b * a.as + row;
     const int quad = warp & 3;
     double sum[8];
 #pragma unroll
@@ -116,16 +110,16 @@ __global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs 
     for (int k = k0; k < k1 && !fail; ++k) {
         const bool second = k >= per;
         const int c0 = (second ? k - per : k) * kProdCols, cw = min(kProdCols, a.nc - c0);
-        const double2* Ac = Ab + (size_t)(c0 + (second ? a.nc : 0)) * a.n;
+        const double2* Ac = Ab + (size_t)(c0 + (second ? a.nc : 0)) * a.ld;
         // entries: columns 16 s + 8 hf + e, s the half
         double2 v[16];
         unsigned m = 0;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = (i >> 3) * 16 + hf * 8 + (i & 7);
-            v[i] = (row < a.n && c < cw) ? __ldg(Ac + (size_t)c * a.n) : make_double2(0.0, 0.0);
+            v[i] = (row < end && c < cw) ? __ldg(Ac + (size_t)c * a.ld) : make_double2(0.0, 0.0);
         }
-        const double2* x = (second ? a.x1 : a.x0) + (size_t)b * a.xs;
+        const double2* x = (second ? x1 : x0) + (size_t)b * a.xs;
         const double2 xv = (warp < nq && lane < cw) ? x[(size_t)(c0 + lane) * a.nrhs + r0 + warp] : make_double2(0.0, 0.0);
 #pragma unroll
         for (int i = 0; i < 16; ++i) m = max(m, mag_hi(v[i]));
@@ -221,8 +215,9 @@ __global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs 
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();         // exponents and accumulators are read before the next chunk
     }
-    if (row < a.n) {
-        double* y = reinterpret_cast<double*>(a.Y + ((size_t)b * a.n + row) * a.nrhs + r0 + 4 * hf);
+    if (row < end) {
+        const int yr = a.map ? a.map[row] : row;
+        double* y = reinterpret_cast<double*>(a.Y + (size_t)b * a.ys + (size_t)yr * a.nrhs + r0 + 4 * hf);
 #pragma unroll
         for (int c = 0; c < 8; ++c)
             if (4 * hf + (c >> 1) < nq) atomicAdd(y + c, fail ? __hiloint2double(0x7ff80000, 0) : a.sign * sum[c]);
