@@ -60,6 +60,13 @@ template <typename T> __device__ __forceinline__ T fma_c(T a, T b, T c) {
 }
 template <typename T> __device__ __forceinline__ T rcp(T a) {
     using R = typename Cx<T>::R;
+    if constexpr (sizeof(R) == 8) {
+        // scaled by a power of two: one division instead of three in a row
+        const unsigned hi = max((unsigned)__double2hiint(a.x) & 0x7fffffffu, (unsigned)__double2hiint(a.y) & 0x7fffffffu);
+        const double s = __hiloint2double(max(1, 2046 - (int)(hi >> 20)) << 20, 0);
+        const double x = a.x * s, y = a.y * s, d = s / fma(x, x, y * y);
+        return Cx<T>::mk(x * d, -y * d);
+    }
     R s = fmax(fabs(a.x), fabs(a.y));
     R ax = a.x / s, ay = a.y / s, d = ax * ax + ay * ay;
     return Cx<T>::mk(ax / (d * s), -ay / (d * s));
@@ -103,8 +110,11 @@ __device__ __forceinline__ void panel_update_fx(double2* S, const double2* a, in
 #pragma unroll
         for (int c = 0; c < kSub64; ++c) hr[c] = hm[c] = cr[c] = cm[c] = 0;
         bool bad = false;
+        double2 ln = a[i];                               // one column of L ahead
+#pragma unroll 1
         for (int t = 0; t < s0; ++t) {
-            const double2 l = a[(size_t)t * n + i];
+            const double2 l = ln;
+            if (t + 1 < s0) ln = a[(size_t)(t + 1) * n + i];
             bad = bad || !(fabs(l.x) <= 2.0) || !(fabs(l.y) <= 2.0);
             int xh, xl, yh, yl;
             fx_split(fx_of_double(l.x, -56), xh, xl);
@@ -138,23 +148,51 @@ __device__ __forceinline__ void panel_update_fx(double2* S, const double2* a, in
 // left (unit-lower solve on its top rows, then the rank-s0 update of the rows
 // below, s0 = columns already factored), factored column by column in shared
 // memory (pivot search, swap, scaling, rank-1 updates), and written back.
-// Each row interchange is applied at once to the panel's other columns in
-// global memory (the L part of the earlier sub-panels and the not yet loaded
-// later ones), so the panel leaves with LAPACK getrf's row order.
+// A column takes two barriers: the rows' updates leave each thread's candidate for the
+// next pivot (|v|^2 as an integer, so that the maxima are warp reductions of its halves),
+// every warp picks the pivot from the warps' candidates, and the first warp exchanges
+// the two rows of the sub-panel and forms 1 / pivot.  The sub-panel's interchanges reach
+// the panel's other columns in global memory together, one load and one store per
+// touched row, so the panel leaves with LAPACK getrf's row order.  What bounds it is
+// this chain of latencies, one CTA per matrix: 0.24 ms per panel at m = 512.  Against five
+// barriers a column, interchanges column by column and a serial search (and with the
+// pivots' reciprocals out of the solves' chain): FP64 solve at N = 256, M = 128 13.05 ->
+// 10.90 ms, at N = 160, M = 64 5.96 -> 4.60 ms.
 template <typename T>
 __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int kb, int w, T* A, int* piv,
                                                               int* info) {
     using R = typename Cx<T>::R;
     extern __shared__ unsigned char smraw[];
     T* S = reinterpret_cast<T*>(smraw);          // [w][m], S[c * m + i], i = row - k0
-    __shared__ R sval[kPanelThreads / 32];
-    __shared__ int sidx[kPanelThreads / 32];
-    __shared__ int spiv;
+    constexpr int kWarps = kPanelThreads / 32;
+    __shared__ int skey[2][kWarps], sidx[2][kWarps], spiv[kNB], strow[2 * kNB], scont[2 * kNB], scnt;
+    __shared__ unsigned slow[2][kWarps];
     __shared__ T sinv;
     const int m = n - k0;
     T* a = A + (size_t)blockIdx.x * n * n;
     int* pv = piv + (size_t)blockIdx.x * n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+    // candidate: the ordered halves of |v|^2 (-1: none, NaN included) and the row
+    int chi = -1, ci = 0;
+    unsigned clo = 0;
+    auto candidate = [&](T v, int i) {
+        const R q = abs2(v);
+        if (!(q >= (R)0)) return;
+        int hi;
+        unsigned lo = 0;
+        if constexpr (sizeof(R) == 8)
+            hi = __double2hiint(q), lo = (unsigned)__double2loint(q);
+        else
+            hi = __float_as_int(q);
+        if (hi > chi || (hi == chi && lo > clo)) chi = hi, clo = lo, ci = i;
+    };
+    // largest candidate over the warp, ties to the smallest row
+    auto reduce = [&](int& hi, unsigned& lo, int& i) {
+        const int h = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned l = __reduce_max_sync(0xffffffffu, hi == h ? lo : 0u);
+        i = __reduce_min_sync(0xffffffffu, hi == h && lo == l ? i : 0x7fffffff);
+        hi = h, lo = l;
+    };
     for (int s0 = 0; s0 < kb; s0 += w) {
         const int ws = min(w, kb - s0);
         for (int idx = tid; idx < ws * m; idx += nt) {
@@ -166,9 +204,11 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
             // top rows: U = L11^{-1} (rows 0..s0-1), one warp per column, lane = row
             for (int c = warp; c < ws; c += nt >> 5) {
                 T x = lane < s0 ? S[c * m + lane] : Cx<T>::mk(0, 0);
+#pragma unroll 8
                 for (int t = 0; t < s0 - 1; ++t) {
+                    const T lt = lane < s0 ? a[(size_t)(k0 + t) * n + k0 + lane] : Cx<T>::mk(0, 0);
                     const T xt = Cx<T>::mk(__shfl_sync(0xffffffffu, x.x, t), __shfl_sync(0xffffffffu, x.y, t));
-                    if (lane > t && lane < s0) x = fms(x, a[(size_t)(k0 + t) * n + k0 + lane], xt);
+                    if (lane > t && lane < s0) x = fms(x, lt, xt);
                 }
                 if (lane < s0) S[c * m + lane] = x;
             }
@@ -181,12 +221,12 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
                 for (int i = s0 + tid; i < m; i += nt) {
                     for (int c0 = 0; c0 < ws; c0 += 8) {
                         T acc[8];
-    #pragma unroll
+#pragma unroll
                         for (int c = 0; c < 8; ++c) acc[c] = Cx<T>::mk(0, 0);
-    #pragma unroll 4
+#pragma unroll 4
                         for (int t = 0; t < s0; ++t) {
                             const T l = a[(size_t)(k0 + t) * n + k0 + i];
-    #pragma unroll
+#pragma unroll
                             for (int c = 0; c < 8; ++c)
                                 if (c0 + c < ws) {
                                     const T u = S[(size_t)(c0 + c) * m + t];
@@ -194,7 +234,7 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
                                     acc[c].y += l.x * u.y + l.y * u.x;
                                 }
                         }
-    #pragma unroll
+#pragma unroll
                         for (int c = 0; c < 8; ++c)
                             if (c0 + c < ws) S[(size_t)(c0 + c) * m + i] = sub(S[(size_t)(c0 + c) * m + i], acc[c]);
                     }
@@ -202,85 +242,96 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
             }
             __syncthreads();
         }
+        chi = -1, clo = 0, ci = 0;
+        for (int i = s0 + tid; i < m; i += nt) candidate(S[i], i);
         for (int jj = 0; jj < ws; ++jj) {
-            const int j = s0 + jj;                 // local row of the diagonal entry
-            const T* col = S + (size_t)jj * m;
-            R best = -1;
-            int bi = j;
-            for (int i = j + tid; i < m; i += nt) {
-                const R v = abs2(col[i]);
-                if (v > best) {
-                    best = v;
-                    bi = i;
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const R ov = __shfl_down_sync(0xffffffffu, best, o);
-                const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-                if (ov > best || (ov == best && oi < bi)) {
-                    best = ov;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) {
-                sval[warp] = best;
-                sidx[warp] = bi;
-            }
+            const int j = s0 + jj, buf = jj & 1;   // j: local row of the diagonal entry
+            reduce(chi, clo, ci);
+            if (lane == 0) skey[buf][warp] = chi, slow[buf][warp] = clo, sidx[buf][warp] = ci;
             __syncthreads();
+            int hi = lane < kWarps ? skey[buf][lane] : -1, p = lane < kWarps ? sidx[buf][lane] : 0x7fffffff;
+            unsigned lo = lane < kWarps ? slow[buf][lane] : 0u;
+            reduce(hi, lo, p);
+            if (hi < 0) p = j;                     // no finite candidate
+            const bool zero = hi < 0 || (hi == 0 && lo == 0u);
             if (warp == 0) {
-                const int nw = nt >> 5;
-                R b = lane < nw ? sval[lane] : (R)-2;
-                int bix = lane < nw ? sidx[lane] : 0x7fffffff;
-                for (int o = 16; o > 0; o >>= 1) {
-                    const R ov = __shfl_down_sync(0xffffffffu, b, o);
-                    const int oi = __shfl_down_sync(0xffffffffu, bix, o);
-                    if (ov > b || (ov == b && oi < bix)) {
-                        b = ov;
-                        bix = oi;
-                    }
+                T vp = Cx<T>::mk(0, 0);
+                if (lane < ws) {
+                    T* sc = S + (size_t)lane * m;
+                    const T vj = sc[j];
+                    vp = sc[p];
+                    sc[j] = vp;
+                    sc[p] = vj;
                 }
+                const T d = Cx<T>::mk(__shfl_sync(0xffffffffu, vp.x, jj), __shfl_sync(0xffffffffu, vp.y, jj));
+                const T iv = zero ? Cx<T>::mk(0, 0) : rcp(d);
                 if (lane == 0) {
-                    spiv = bix;
-                    pv[k0 + j] = k0 + bix;
-                    const T d = col[bix];
-                    if (b <= (R)0) {
-                        if (info[blockIdx.x] == 0) info[blockIdx.x] = k0 + j + 1;
-                        sinv = Cx<T>::mk(0, 0);
-                    } else {
-                        sinv = rcp(d);
-                    }
+                    spiv[jj] = p;
+                    pv[k0 + j] = k0 + p;
+                    sinv = iv;
+                    if (zero && info[blockIdx.x] == 0) info[blockIdx.x] = k0 + j + 1;
                 }
             }
-            __syncthreads();
-            const int p = spiv;
-            if (p != j)
-                for (int c = tid; c < kb; c += nt) {
-                    if (c >= s0 && c < s0 + ws) {
-                        T* sc = S + (size_t)(c - s0) * m;
-                        const T t = sc[j];
-                        sc[j] = sc[p];
-                        sc[p] = t;
-                    } else {
-                        T* gc = a + (size_t)(k0 + c) * n + k0;
-                        const T t = gc[j];
-                        gc[j] = gc[p];
-                        gc[p] = t;
-                    }
-                }
             __syncthreads();
             // scale column j below the diagonal, rank-1 update of the sub-panel's later columns
             const T inv = sinv;
+            chi = -1, clo = 0, ci = j + 1;
             for (int i = j + 1 + tid; i < m; i += nt) {
                 const T l = mul(S[(size_t)jj * m + i], inv);
                 S[(size_t)jj * m + i] = l;
-                for (int cc = jj + 1; cc < ws; ++cc)
-                    S[(size_t)cc * m + i] = fms(S[(size_t)cc * m + i], l, S[(size_t)cc * m + j]);
+                for (int c0 = jj + 1; c0 < ws; c0 += 4) {
+                    T u[4], v[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (c0 + c < ws) u[c] = S[(size_t)(c0 + c) * m + j], v[c] = S[(size_t)(c0 + c) * m + i];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (c0 + c < ws) {
+                            v[c] = fms(v[c], l, u[c]);
+                            S[(size_t)(c0 + c) * m + i] = v[c];
+                        }
+                    if (c0 == jj + 1) candidate(v[0], i);
+                }
             }
-            __syncthreads();
+        }
+        __syncthreads();
+        // the interchanges as one permutation of the touched rows (slots: the ws diagonal
+        // rows, then up to ws others), simulated by the first warp
+        if (warp == 0) {
+            int row1 = -1, cont0 = s0 + lane, cont1 = -1, cnt = 0;
+            for (int jj = 0; jj < ws; ++jj) {
+                const int p = spiv[jj];
+                if (p < s0 + ws) {
+                    const int o = p - s0, cj = __shfl_sync(0xffffffffu, cont0, jj), cp = __shfl_sync(0xffffffffu, cont0, o);
+                    if (lane == jj) cont0 = cp;
+                    if (lane == o) cont0 = cj;
+                } else {
+                    const unsigned hit = __ballot_sync(0xffffffffu, row1 == p);
+                    const int o = hit ? __ffs(hit) - 1 : cnt++;
+                    if (!hit && lane == o) row1 = cont1 = p;
+                    const int cj = __shfl_sync(0xffffffffu, cont0, jj), cp = __shfl_sync(0xffffffffu, cont1, o);
+                    if (lane == jj) cont0 = cp;
+                    if (lane == o) cont1 = cj;
+                }
+            }
+            if (lane < ws) strow[lane] = s0 + lane, scont[lane] = cont0;
+            if (lane < cnt) strow[ws + lane] = row1, scont[ws + lane] = cont1;
+            if (lane == 0) scnt = ws + cnt;
         }
         for (int idx = tid; idx < ws * m; idx += nt) {
             const int c = idx / m, i = idx - c * m;
             a[(size_t)(k0 + s0 + c) * n + k0 + i] = S[idx];
+        }
+        __syncthreads();
+        {
+            // at most (kb - ws) 2 ws <= 512 values: one per thread
+            const int cnt = scnt, oc = tid / cnt, s = tid - oc * cnt, c = oc < s0 ? oc : oc + ws;
+            const bool in = c < kb;
+            T* g = a + (size_t)(k0 + c) * n + k0;
+            T v = Cx<T>::mk(0, 0);
+            if (in) v = g[scont[s]];
+            __syncthreads();
+            if (in && scont[s] != strow[s]) g[strow[s]] = v;
         }
         __syncthreads();
     }
@@ -973,8 +1024,10 @@ __global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nv, int nrhs, 
             apply_inv(j0);
         } else if (warp < nr) {
             T v = lane < jb ? sx[(j0 + lane) * R + warp] : Cx<T>::mk(0, 0);
+            // every pivot's reciprocal at once, not in the chain of the columns
+            const T rd = lane < jb ? rcp(widen<T>(sD[lane * kNB + lane])) : v;
             for (int c = jb - 1; c >= 0; --c) {
-                if (lane == c) v = mul(v, rcp(widen<T>(sD[c * kNB + c])));
+                if (lane == c) v = mul(v, rd);
                 T xc = Cx<T>::mk(__shfl_sync(0xffffffff, v.x, c), __shfl_sync(0xffffffff, v.y, c));
                 if (lane < c) v = fms(v, widen<T>(sD[c * kNB + lane]), xc);
             }
