@@ -195,10 +195,10 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
     };
     for (int s0 = 0; s0 < kb; s0 += w) {
         const int ws = min(w, kb - s0);
-        for (int idx = tid; idx < ws * m; idx += nt) {
-            const int c = idx / m, i = idx - c * m;
-            S[idx] = a[(size_t)(k0 + s0 + c) * n + k0 + i];
-        }
+        // (no divisions by m: run-time integer division issues to the FP64 pipe)
+        for (int i = tid; i < m; i += nt)
+#pragma unroll 8
+            for (int c = 0; c < ws; ++c) S[(size_t)c * m + i] = a[(size_t)(k0 + s0 + c) * n + k0 + i];
         __syncthreads();
         if (s0 > 0) {
             // top rows: U = L11^{-1} (rows 0..s0-1), one warp per column, lane = row
@@ -318,10 +318,9 @@ __global__ void __launch_bounds__(kPanelThreads) panel_kernel(int n, int k0, int
             if (lane < cnt) strow[ws + lane] = row1, scont[ws + lane] = cont1;
             if (lane == 0) scnt = ws + cnt;
         }
-        for (int idx = tid; idx < ws * m; idx += nt) {
-            const int c = idx / m, i = idx - c * m;
-            a[(size_t)(k0 + s0 + c) * n + k0 + i] = S[idx];
-        }
+        for (int i = tid; i < m; i += nt)
+#pragma unroll 8
+            for (int c = 0; c < ws; ++c) a[(size_t)(k0 + s0 + c) * n + k0 + i] = S[(size_t)c * m + i];
         __syncthreads();
         {
             // at most (kb - ws) 2 ws <= 512 values: one per thread
