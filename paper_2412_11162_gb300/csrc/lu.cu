@@ -1120,6 +1120,12 @@ __global__ void c128_to_c64_kernel(int64_t count, const double2* s, float2* d) {
     for (; i < count; i += stride) d[i] = make_float2((float)s[i].x, (float)s[i].y);
 }
 
+}  // namespace
+}  // namespace pmlbie
+#include "lu_solve32.cuh"
+namespace pmlbie {
+namespace {
+
 // The product of ProductArgs on the FP64 pipe: a thread per (row, right-hand side), one
 // chunk of kProdCols columns, added with atomics.  Grid (rows, column chunks, matrices),
 // so that a single active matrix still spreads over many SMs.  At one right-hand side it
@@ -1489,6 +1495,25 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
 template <typename T, typename TF>
 cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, const int* piv, T* B,
                              cudaStream_t s, const int* active, const TF* dinv, const int2* ptab) {
+    if constexpr (std::is_same<T, float2>::value && std::is_same<TF, float2>::value) {
+        // streamed solves: right-hand sides per CTA a power of two that shared memory holds
+        // (n up to 14000; beyond, the general kernel)
+        constexpr size_t kSmem = 227 * 1024;
+        int R = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
+        while (R > 1 && kStOffX + sizeof(T) * (size_t)R * n > kSmem) R /= 2;
+        const size_t sm = kStOffX + sizeof(T) * (size_t)R * n;
+        if (dinv && ptab && n % kNB == 0 && sm <= kSmem) {
+            auto run = [&](auto kernel) {
+                cudaError_t e = allow_max_smem(kernel);
+                if (e != cudaSuccess) return e;
+                kernel<<<dim3(batch, (nrhs + R - 1) / R), kStThreads, sm, s>>>(n, nv, nrhs, LU, B, active, dinv, ptab);
+                count_launch();
+                return cudaGetLastError();
+            };
+            return R == 8 ? run(lu_solve32_kernel<8>) : R == 4 ? run(lu_solve32_kernel<4>)
+                 : R == 2 ? run(lu_solve32_kernel<2>) : run(lu_solve32_kernel<1>);
+        }
+    }
     // right-hand sides per CTA: up to kSolveR, as many as fit in shared memory
     // (about 200 KB for the group)
     int R = std::min(nrhs, kSolveR);
