@@ -1500,13 +1500,13 @@ cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, c
         // (n up to 14000; beyond, the general kernel)
         constexpr size_t kSmem = 227 * 1024;
         int R = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
-        while (R > 1 && kStOffX + sizeof(T) * (size_t)R * n > kSmem) R /= 2;
-        const size_t sm = kStOffX + sizeof(T) * (size_t)R * n;
+        while (R > 1 && st_smem(n, R) > kSmem) R /= 2;
+        const size_t sm = st_smem(n, R);
         if (dinv && ptab && n % kNB == 0 && sm <= kSmem) {
             auto run = [&](auto kernel) {
                 cudaError_t e = allow_max_smem(kernel);
                 if (e != cudaSuccess) return e;
-                kernel<<<dim3(batch, (nrhs + R - 1) / R), kStThreads, sm, s>>>(n, nv, nrhs, LU, B, active, dinv, ptab);
+                kernel<<<dim3(batch, (nrhs + R - 1) / R), kStThreads, sm, s>>>(n, nv, nrhs, st_rows(n), LU, B, active, dinv, ptab);
                 count_launch();
                 return cudaGetLastError();
             };

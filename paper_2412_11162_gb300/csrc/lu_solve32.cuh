@@ -19,8 +19,11 @@ namespace pmlbie {
 namespace {
 
 constexpr int kStRows = 512, kStCols = 8, kStages = 3, kStThreads = 544;
-constexpr uint32_t kStBytes = kStRows * kStCols * 8, kStDiag = 32 * 32 * 8;
-constexpr uint32_t kStOffDiag = kStages * kStBytes, kStOffBar = kStOffDiag + 2 * kStDiag, kStOffX = kStOffBar + 128;
+constexpr uint32_t kStDiag = 32 * 32 * 8, kStOffDiag = 128, kStOffX = kStOffDiag + 2 * kStDiag;
+// rows of a stage (small systems leave room for another CTA) and the CTA's shared memory:
+// barriers, inverse blocks, right-hand sides, stages
+inline int st_rows(int n) { return n < kStRows ? n : kStRows; }
+inline size_t st_smem(int n, int R) { return kStOffX + 8 * (size_t)n * R + (size_t)kStages * st_rows(n) * kStCols * 8; }
 struct StreamBars {
     uint64_t full[kStages], empty[kStages], dfull[2], dempty[2];
     int err;
@@ -28,15 +31,16 @@ struct StreamBars {
 static_assert(sizeof(StreamBars) <= 128, "barrier block");
 
 template <int RM>
-__global__ void __launch_bounds__(kStThreads, 1) lu_solve32_kernel(int n, int nv, int nrhs, const float2* LU, float2* B,
+__global__ void __launch_bounds__(kStThreads, 1) lu_solve32_kernel(int n, int nv, int nrhs, int sr, const float2* LU, float2* B,
                                                                 const int* active, const float2* dinv,
                                                                 const int2* ptab) {
     using namespace tcu;
     extern __shared__ __align__(1024) unsigned char sm[];
     const int b = blockIdx.x, r0 = blockIdx.y * RM, nr = min(RM, nrhs - r0);
     if (active && !active[b]) return;
-    StreamBars* bar = reinterpret_cast<StreamBars*>(sm + kStOffBar);
+    StreamBars* bar = reinterpret_cast<StreamBars*>(sm);
     float2* sx = reinterpret_cast<float2*>(sm + kStOffX);       // [n][RM]
+    float2* stage = sx + (size_t)n * RM;                        // kStages x [kStCols][sr]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nblk = n / 32;
     const float2* a = LU + (size_t)b * n * n;
     float2* x = B + (size_t)b * nv * nrhs + r0;
@@ -71,15 +75,15 @@ __global__ void __launch_bounds__(kStThreads, 1) lu_solve32_kernel(int n, int nv
                 bulk_load(smem_u32(sm + kStOffDiag + (d & 1) * kStDiag), db + (size_t)(2 * k + back) * kStDiag, kStDiag,
                           smem_u32(&bar->dfull[d & 1]));
                 const int end = last(k, back);
-                for (int seg = first(k, back); seg < end && !*err; seg += kStRows) {
-                    const int rows = min(kStRows, end - seg);
+                for (int seg = first(k, back); seg < end && !*err; seg += sr) {
+                    const int rows = min(sr, end - seg);
                     for (int g = 0; g < 32; g += kStCols, ++i) {
                         const int s = i % kStages;
                         if (i >= kStages) wait(&bar->empty[s], i / kStages - 1);
                         if (*err) break;
                         mb_expect(&bar->full[s], (uint32_t)rows * kStCols * 8);
                         for (int c = 0; c < kStCols; ++c)
-                            bulk_load(smem_u32(sm + s * kStBytes + c * kStRows * 8), a + (size_t)(32 * k + g + c) * n + seg,
+                            bulk_load(smem_u32(stage + (s * kStCols + c) * sr), a + (size_t)(32 * k + g + c) * n + seg,
                                       (uint32_t)rows * 8, smem_u32(&bar->full[s]));
                     }
                 }
@@ -127,8 +131,8 @@ __global__ void __launch_bounds__(kStThreads, 1) lu_solve32_kernel(int n, int nv
             asm volatile("bar.sync 1, 512;" ::: "memory");
             if (tid == 0) mb_arrive(&bar->dempty[d & 1]);
             const int end = last(k, back);
-            for (int seg = first(k, back); seg < end; seg += kStRows) {
-                const bool in = r < min(kStRows, end - seg);
+            for (int seg = first(k, back); seg < end; seg += sr) {
+                const bool in = r < min(sr, end - seg);
                 float2 acc[NR][RT];
                 if (in)
 #pragma unroll
@@ -139,16 +143,16 @@ __global__ void __launch_bounds__(kStThreads, 1) lu_solve32_kernel(int n, int nv
                     const int s = i % kStages;
                     wait(&bar->full[s], i / kStages);
                     if (in) {
-                        const float2* F = reinterpret_cast<const float2*>(sm + s * kStBytes) + r;
+                        const float2* F = stage + s * kStCols * sr + r;
                         const float2* xs = sx + (j0 + g) * RM + q0;
 #pragma unroll
                         for (int c = 0; c < kStCols; ++c) {
                             float2 f[NR];
                             if constexpr (NR == 2) {
-                                const float4 v = *reinterpret_cast<const float4*>(F + c * kStRows);
+                                const float4 v = *reinterpret_cast<const float4*>(F + c * sr);
                                 f[0] = make_float2(v.x, v.y), f[1] = make_float2(v.z, v.w);
                             } else {
-                                f[0] = F[c * kStRows];
+                                f[0] = F[c * sr];
                             }
 #pragma unroll
                             for (int q = 0; q < RT; ++q) {
