@@ -9,7 +9,9 @@
 // panel), row swaps + unit-lower triangular solve for the block row, and a
 // GEMM update of the trailing matrix on the tcgen05 tensor cores from split
 // operand images formed once per step (complex64: TF32 hi / lo, tc_update.cuh;
-// complex128: exact bf16 digit slices, tc_update64.cuh).  complex128 leaves LAPACK getrf's row order (every
+// complex128: exact bf16 digit slices, tc_update64.cuh).  The complex64 solves stream the
+// factors (lu_solve32.cuh); residuals of several right-hand sides take the tensor cores
+// (tc_product64.cuh).  complex128 leaves LAPACK getrf's row order (every
 // column swapped) and a row permutation in piv; complex64 swaps only the
 // columns right of each panel, so L's column blocks keep their step's row
 // order, and the solves apply each step's interchanges (the per-step slot

@@ -1,7 +1,8 @@
 """Complex128 products with several right-hand sides on the tensor cores
 (csrc/tc_product64.cuh), which form the right-hand sides and the residuals of the
 solves: row blocks of 128 and column chunks of 32 with remainders, groups of 8
-right-hand sides with remainders.  A solution of the wrong system shows as a backward
+right-hand sides with remainders; and the streamed complex64 solves
+(csrc/lu_solve32.cuh) with 1 to 8 right-hand sides and more than one segment of 512 rows.  A solution of the wrong system shows as a backward
 error in the systems that the library's own kernels, corrections and diagonal give.
 Bars: mixed 1e-13 (the documented stop), FP64 4 n u (elimination with a growth of at
 most 4), plus the rounding n u of this test's own products, n = 2 N, u = 2^-53."""
@@ -13,7 +14,7 @@ from test_gpu_lu64 import systems
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,waves", [(47, 2), (48, 5), (64, 8), (65, 9), (80, 17), (130, 2)])
+@pytest.mark.parametrize("N,waves", [(47, 2), (48, 5), (64, 8), (65, 9), (80, 17), (130, 2), (290, 8)])
 def test_backward_error(N, waves):
     from paper_2412_11162_gb300 import Problem
     from paper_2412_11162_gb300.binding import PMLBIE_FP64, PMLBIE_MIXED
