@@ -345,6 +345,15 @@ __device__ __forceinline__ int fx_even_dft(longlong2* x, FxScale sc, int K, cons
     __syncwarp();
     return sc.ex == kFxNonfinite ? sc.ex : sc.ex + sh;
 }
+// The same out of line: the close-pair kernel holds two sizes of it, and instruction
+// misses cost it more than the calls (close pairs at N = 1024, M = 512 49.5 -> 48.1 ms,
+// 8 low modes at N = 128 1.07 -> 1.01 ms); the far and field kernels, whose
+// transforms follow a long sampling loop, are faster with it in line (field map 6.74
+// against 6.98 ms).
+template <int NB>
+__device__ __noinline__ int fx_even_dft_call(longlong2* x, FxScale sc, int K, const int4* tw, int tws, int lane) {
+    return fx_even_dft<NB>(x, sc, K, tw, tws, lane);
+}
 
 }  // namespace
 }  // namespace pmlbie

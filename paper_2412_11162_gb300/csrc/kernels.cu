@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(128) near_laplace_out_kernel(NearArgs a) {
 // index computes both; the mirror's S^ equal the pair's, and its CTA returns at once.
 //
 // Samples, transforms and phases as in the far kernel.  Modal kernels at N = 1024,
-// M = 512 through this kernel: 49.1 ms; with float-float physical pairs and FP64 PML
+// M = 512 through this kernel: 48.0 ms; with float-float physical pairs and FP64 PML
 // pairs 84.6 ms.  Bounded by the barriers between the phases of one pair and by issue
 // (IPC 1.1 at M = 256); two CTAs of 256 threads hold M = 512's shared memory.
 //

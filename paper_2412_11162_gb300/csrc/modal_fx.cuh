@@ -218,7 +218,7 @@ __device__ __forceinline__ void near_finish(const NearShape& p, int M, const int
                 const int u = t - nc - nz;
                 const int s = t < nc ? 2 * t : p.plain ? 2 * u : u < nc ? 2 * u + 1 : mirror0 + (u - nc);
                 longlong2* x = seq + s * S1;
-                const int ex = fx_even_dft<NBH>(x, quantise(x, s), K, tw, 2, lane);
+                const int ex = fx_even_dft_call<NBH>(x, quantise(x, s), K, tw, 2, lane);
                 if (lane == 0) exq[s] = ex;
                 if (t < nc) {
                     // packed: F1a + i F1b and F3a - i F3b (region b's -D^ as the conjugate)
@@ -240,7 +240,7 @@ __device__ __forceinline__ void near_finish(const NearShape& p, int M, const int
                 sc = fx_quantise(y, S2, lane);
             }
             if (y) {
-                const int ex = fx_even_dft<NB>(reinterpret_cast<longlong2*>(y), sc, M, tw, 1, lane);
+                const int ex = fx_even_dft_call<NB>(reinterpret_cast<longlong2*>(y), sc, M, tw, 1, lane);
                 if (lane == 0) *ey = ex;
             }
         }
