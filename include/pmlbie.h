@@ -408,6 +408,19 @@ int  pmlbie_selftest_wait(long long iterations, void* stream);
  * the stream.  EINVAL for an unknown fn, NULL buffers or n > 2^31; ECUDA. */
 int  pmlbie_selftest_elementary(int fn, const void* dev_x, void* dev_out, size_t n, void* stream);
 
+/* Self-tests of the dense complex128 kernels of the solves, on caller-owned
+ * device arrays of `batch` column-major n x n matrices A.
+ * pmlbie_selftest_lu: A is overwritten by its factors P A = L U (L unit lower,
+ * below the diagonal), dev_perm ([batch][n] int) receives the rows of A in the
+ * factors' order; ESINGULAR on a zero pivot.
+ * pmlbie_selftest_product: Y = A X for n_rhs right-hand sides, X and Y
+ * [batch][n][n_rhs], n even.
+ * Allocate scratch and synchronise the stream.  EINVAL (n < 1, batch outside
+ * 1 .. 65535, NULL), ENOMEM, ECUDA. */
+int  pmlbie_selftest_lu(int n, int batch, void* dev_A, int* dev_perm, void* stream);
+int  pmlbie_selftest_product(int n, int batch, int n_rhs, const void* dev_A, const void* dev_X, void* dev_Y,
+                             void* stream);
+
 /* Pipe-throughput probe (not an operation of the paper: the measured
  * denominators of the library's roofline fractions).  kind 0: FP64 FMA
  * (independent fma chains on every SM), 1: FP32 FMA, 2: TF32 tensor cores

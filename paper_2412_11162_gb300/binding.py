@@ -67,7 +67,8 @@ EXPORTS = ["pmlbie_create", "pmlbie_destroy", "pmlbie_last_error", "pmlbie_nodes
            "pmlbie_modal_kernels", "pmlbie_modal_kernels_ex", "pmlbie_close_pair_kernels",
            "pmlbie_modal_kernels_noalloc",
            "pmlbie_solve", "pmlbie_solve_ex", "pmlbie_solve_batch", "pmlbie_field", "pmlbie_solve_host",
-           "pmlbie_check_finite", "pmlbie_selftest_wait", "pmlbie_selftest_elementary", "pmlbie_selftest_peak"]
+           "pmlbie_check_finite", "pmlbie_selftest_wait", "pmlbie_selftest_elementary", "pmlbie_selftest_peak",
+           "pmlbie_selftest_lu", "pmlbie_selftest_product"]
 
 
 def _load():
@@ -112,7 +113,10 @@ def _load():
     lib.pmlbie_selftest_wait.argtypes = [ctypes.c_longlong, vp]
     lib.pmlbie_selftest_elementary.argtypes = [ctypes.c_int, vp, vp, ctypes.c_size_t, vp]
     lib.pmlbie_selftest_peak.argtypes = [ctypes.c_int, dp, vp]
-    for f in ("pmlbie_check_finite", "pmlbie_selftest_wait", "pmlbie_selftest_elementary", "pmlbie_selftest_peak", "pmlbie_nodes", "pmlbie_diagonal",
+    lib.pmlbie_selftest_lu.argtypes = [ctypes.c_int, ctypes.c_int, vp, vp, vp]
+    lib.pmlbie_selftest_product.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp, vp, vp]
+    for f in ("pmlbie_check_finite", "pmlbie_selftest_wait", "pmlbie_selftest_elementary", "pmlbie_selftest_peak",
+              "pmlbie_selftest_lu", "pmlbie_selftest_product", "pmlbie_nodes", "pmlbie_diagonal",
               "pmlbie_dims", "pmlbie_near_count", "pmlbie_near_pairs", "pmlbie_corrections", "pmlbie_node_tables",
               "pmlbie_alpert_rule",
               "pmlbie_modal_kernels", "pmlbie_modal_kernels_noalloc", "pmlbie_modal_kernels_ex",
@@ -497,3 +501,33 @@ def pmlbie_selftest_peak(kind, stream=None):
     v = ctypes.c_double(0.0)
     check(lib.pmlbie_selftest_peak(int(kind), ctypes.byref(v), _stream(stream)), "pmlbie_selftest_peak")
     return v.value
+
+
+def _dense(where, *arrays):
+    import torch
+    for name, t, dtype, want in arrays:
+        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()
+                and t.numel() == want):
+            raise PmlbieError(PMLBIE_EINVAL, where, "%s must be a contiguous %s CUDA tensor of %d elements"
+                              % (name, dtype, want))
+
+
+def pmlbie_selftest_lu(A, perm, stream=None):
+    """Complex128 LU of the matrices A[b][column][row], in place; perm[b][row] (int32) receives
+    the rows of A in the factors' order."""
+    import torch
+    batch, n = A.shape[0], A.shape[1]
+    _dense("pmlbie_selftest_lu", ("A", A, torch.complex128, batch * n * n), ("perm", perm, torch.int32, batch * n))
+    check(lib.pmlbie_selftest_lu(n, batch, _tptr(A), _tptr(perm), _stream(stream)), "pmlbie_selftest_lu")
+    return A, perm
+
+
+def pmlbie_selftest_product(A, X, Y, stream=None):
+    """Y[b] = A[b] X[b] for A[b][column][row] and X, Y [b][row][right-hand side], complex128."""
+    import torch
+    batch, n, nrhs = X.shape
+    _dense("pmlbie_selftest_product", ("A", A, torch.complex128, batch * n * n),
+           ("X", X, torch.complex128, batch * n * nrhs), ("Y", Y, torch.complex128, batch * n * nrhs))
+    check(lib.pmlbie_selftest_product(n, batch, nrhs, _tptr(A), _tptr(X), _tptr(Y), _stream(stream)),
+          "pmlbie_selftest_product")
+    return Y

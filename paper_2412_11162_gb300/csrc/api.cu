@@ -1276,6 +1276,53 @@ int pmlbie_selftest_wait(long long iterations, void* stream) {
              : PMLBIE_OK;
 }
 
+int pmlbie_selftest_lu(int n, int batch, void* dev_A, int* dev_perm, void* stream) {
+    if (n < 1 || batch < 1 || batch > 65535 || !dev_A || !dev_perm) return fail(PMLBIE_EINVAL, "bad size or NULL buffer");
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // digit images of half the matrices, so that the updates take them in two groups
+    const size_t images = lu_image64_bytes(n) * ((batch + 1) / 2), total = align256(images) + sizeof(int) * (size_t)batch;
+    char* p = nullptr;
+    if (cudaMalloc(&p, total) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(PMLBIE_ENOMEM, "scratch allocation failed");
+    }
+    int* info = reinterpret_cast<int*>(p + align256(images));
+    std::vector<int> bad(batch, 0);
+    cudaError_t e = cudaMemsetAsync(info, 0, sizeof(int) * batch, s);
+    if (e == cudaSuccess)
+        e = batched_lu<double2>(n, batch, static_cast<double2*>(dev_A), dev_perm, info, s,
+                                reinterpret_cast<unsigned char*>(p), nullptr, nullptr, nullptr, images);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(bad.data(), info, sizeof(int) * batch, cudaMemcpyDeviceToHost, s);
+    const cudaError_t es = cudaStreamSynchronize(s);
+    cudaFree(p);
+    if (e == cudaSuccess) e = es;
+    if (e != cudaSuccess) return fail(PMLBIE_ECUDA, std::string("LU self-test: ") + cudaGetErrorString(e));
+    for (int b = 0; b < batch; ++b)
+        if (bad[b]) return fail(PMLBIE_ESINGULAR, "matrix " + std::to_string(b) + ": info " + std::to_string(bad[b]));
+    return PMLBIE_OK;
+}
+
+int pmlbie_selftest_product(int n, int batch, int n_rhs, const void* dev_A, const void* dev_X, void* dev_Y,
+                            void* stream) {
+    if (n < 2 || n % 2 || batch < 1 || batch > 65535 || n_rhs < 1 || !dev_A || !dev_X || !dev_Y)
+        return fail(PMLBIE_EINVAL, "bad size or NULL buffer");
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    ProductArgs a;
+    a.ld = a.split = a.rows = n;
+    a.nc = n / 2;
+    a.nrhs = n_rhs;
+    a.A = static_cast<const double2*>(dev_A);
+    a.x0 = static_cast<const double2*>(dev_X);
+    a.x1 = a.x0 + (size_t)a.nc * n_rhs;
+    a.as = (size_t)n * n;
+    a.xs = a.ys = (size_t)n * n_rhs;
+    a.Y = static_cast<double2*>(dev_Y);
+    PMLBIE_CUDA_TRY(cudaMemsetAsync(dev_Y, 0, sizeof(double2) * a.ys * batch, s));
+    PMLBIE_CUDA_TRY(add_product_c128(a, batch, s));
+    PMLBIE_CUDA_TRY(cudaStreamSynchronize(s));
+    return PMLBIE_OK;
+}
+
 int pmlbie_selftest_peak(int kind, double* tflops, void* stream) {
     if (kind < 0 || kind > 2 || !tflops) return fail(PMLBIE_EINVAL, "kind must be 0, 1 or 2 and tflops non-NULL");
     return peak_probe(kind, tflops, static_cast<cudaStream_t>(stream));

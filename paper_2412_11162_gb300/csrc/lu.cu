@@ -80,15 +80,22 @@ constexpr int kPanelThreads = 512;
 
 // complex128 panels: S[c][i] -= sum_{t < s0} L[i][t] U[t][c] for the rows i >= s0 of a
 // sub-panel of ws <= kSub64 columns (S in shared memory, column stride m; U its first
-// s0 rows; L the panel's finished columns in global memory), on the integer pipe: L
-// in units of 2^-56 (|L| <= 1 by the pivoting), column c of U in units of 2^-57 of
-// its largest entry, three 32 x 32 -> 64 multiply-adds per real product, the sum
-// rounded once to 2^-57 of that entry and subtracted in FP64.  The FP64 pipe (2 per
-// SM per clock, and one CTA per matrix) keeps the rank-1 updates inside the
-// sub-panels only.  A NaN or an infinity in a row of L or a column of U gives NaN.
-// Measured with kSub64 = 8, against sub-panels of 16 updated in FP64: FP64 solve at N =
-// 256, M = 128 (64 systems of 512) 15.2 -> 14.3 ms, at N = 160, M = 64 6.65 -> 6.50 ms.
+// s0 rows; L the panel's finished columns in global memory), on the integer pipe: the
+// row of L in units of 2^-55 of its largest entry, the column of U likewise, both split
+// into digits of 28 and 27 bits, three 32 x 32 -> 64 multiply-adds per real product (the
+// low x low ones are dropped: about 2^-57 of the product of the largest entries together,
+// 2^-52 at worst), the sum rounded to 2^-55 or less of that product and subtracted in
+// FP64; entries that this unit is too coarse for (weak_sum) are formed in FP64.  The FP64
+// pipe (2 per SM per clock, and one CTA per matrix) keeps those and the rank-1 updates
+// inside the sub-panels only.  A NaN or an infinity in a row of L or a column of U gives
+// NaN.  All panels of 64 systems of 512 (FP64 solve at N = 256, M = 128): 2.99 ms; 4.22 ms
+// with the products in FP64 and sub-panels of 16, 4.69 ms with sub-panels of 8.
 constexpr int kSub64 = 8;
+// x = h 2^27 + l, |l| <= 2^26
+__device__ __forceinline__ void split27(i64 x, int& h, int& l) {
+    l = (int)((unsigned)(u64)x << 5) >> 5;
+    h = (int)(x >> 27) - (l >> 31);
+}
 __device__ __forceinline__ void panel_update_fx(double2* S, const double2* a, int n, int m, int s0, int ws, int tid,
                                                 int nt) {
     __shared__ int4 uq[kNB][kSub64];
@@ -96,31 +103,32 @@ __device__ __forceinline__ void panel_update_fx(double2* S, const double2* a, in
     const int lane = tid & 31, warp = tid >> 5;
     if (warp < ws) {      // one warp per column, lane = row of U
         const double2 u = lane < s0 ? S[(size_t)warp * m + lane] : make_double2(0.0, 0.0);
-        const unsigned hi = max((unsigned)__double2hiint(u.x) & 0x7fffffffu, (unsigned)__double2hiint(u.y) & 0x7fffffffu);
-        const int top = (int)(__reduce_max_sync(0xffffffffu, hi) >> 20);
-        const int ex = top - 1079;                      // |u| 2^-ex < 2^57
+        const int top = (int)(__reduce_max_sync(0xffffffffu, tcu::mag_hi(u)) >> 20);
+        const int ex = top - 1077;                      // |u| 2^-ex < 2^55
         int h0, l0, h1, l1;
-        fx_split(fx_of_double(u.x, ex), h0, l0);
-        fx_split(fx_of_double(u.y, ex), h1, l1);
+        split27(fx_of_double(u.x, ex), h0, l0);
+        split27(fx_of_double(u.y, ex), h1, l1);
         uq[lane][warp] = make_int4(h0, l0, h1, l1);
         if (lane == 0) ue[warp] = top == 0x7ff ? kFxNonfinite : ex;
     }
     __syncthreads();
     for (int i = s0 + tid; i < m; i += nt) {
-        // sums of the high x high products, and of the mixed ones (times 2^-32)
+        unsigned hi = 0;
+#pragma unroll 8
+        for (int t = 0; t < s0; ++t) hi = max(hi, tcu::mag_hi(a[(size_t)t * n + i]));
+        const int top = (int)(hi >> 20), el = top - 1077;
+        // sums of the high x high products, and of the mixed ones
         i64 hr[kSub64], hm[kSub64], cr[kSub64], cm[kSub64];
 #pragma unroll
         for (int c = 0; c < kSub64; ++c) hr[c] = hm[c] = cr[c] = cm[c] = 0;
-        bool bad = false;
         double2 ln = a[i];                               // one column of L ahead
 #pragma unroll 1
         for (int t = 0; t < s0; ++t) {
             const double2 l = ln;
             if (t + 1 < s0) ln = a[(size_t)(t + 1) * n + i];
-            bad = bad || !(fabs(l.x) <= 2.0) || !(fabs(l.y) <= 2.0);
             int xh, xl, yh, yl;
-            fx_split(fx_of_double(l.x, -56), xh, xl);
-            fx_split(fx_of_double(l.y, -56), yh, yl);
+            split27(fx_of_double(l.x, el), xh, xl);
+            split27(fx_of_double(l.y, el), yh, yl);
 #pragma unroll
             for (int c = 0; c < kSub64; ++c) {
                 const int4 u = uq[t][c];
@@ -130,16 +138,27 @@ __device__ __forceinline__ void panel_update_fx(double2* S, const double2* a, in
                 cm[c] += mul_wide(xl, u.z) + mul_wide(xh, u.w) + mul_wide(yl, u.x) + mul_wide(yh, u.y);
             }
         }
+        unsigned weak = 0;
 #pragma unroll
         for (int c = 0; c < kSub64; ++c)
             if (c < ws) {
-                // sum = (h 2^64 + c 2^32) 2^(ex - 56) = T 2^(ex), T = h 2^8 + c 2^-24 in units of 2^56
-                const int ex = bad ? kFxNonfinite : ue[c];
-                const double2 v = fx_to_double2(fx2((hr[c] << 8) + ((cr[c] + (1 << 23)) >> 24),
-                                                    (hm[c] << 8) + ((cm[c] + (1 << 23)) >> 24)), ex);
+                // (h 2^54 + c 2^27) 2^(el + eu) in units of 2^(el + eu + 53)
+                const int ex = (top == 0x7ff || ue[c] == kFxNonfinite) ? kFxNonfinite : el + ue[c] + 53;
+                const double2 v = fx_to_double2(fx2((hr[c] << 1) + ((cr[c] + (1 << 25)) >> 26),
+                                                    (hm[c] << 1) + ((cm[c] + (1 << 25)) >> 26)), ex);
                 double2& d = S[(size_t)c * m + i];
-                d = make_double2(d.x - v.x, d.y - v.y);
+                if (tcu::weak_sum(ex, max(tcu::mag_hi(d), tcu::mag_hi(v))))
+                    weak |= 1u << c;
+                else
+                    d = make_double2(d.x - v.x, d.y - v.y);
             }
+        for (; weak; weak &= weak - 1) {
+            double2* sc = S + (size_t)(__ffs(weak) - 1) * m;
+            double2 v = make_double2(0.0, 0.0);
+#pragma unroll 4
+            for (int t = 0; t < s0; ++t) v = fma_c(v, a[(size_t)t * n + i], sc[t]);
+            sc[i] = sub(sc[i], v);
+        }
     }
 }
 

@@ -156,6 +156,18 @@ __device__ __forceinline__ int acc_int(uint32_t bits) {
     return (m ^ sg) - sg;
 }
 
+// A sum in units of 2^ex where 2^ex exceeds 2^-kWeakBits of the values that it meets (hi:
+// the largest of their high words, signs off) has lost bits that a double would keep: the
+// digits lie below the row's and the column's largest entry, and the entry itself can be
+// smaller by any factor (the modal kernels of high modes fall off like (rho / rho')^n
+// next to the axis).  Such entries are formed again in FP64.
+constexpr int kWeakBits = 50;
+__device__ __forceinline__ bool weak_sum(int ex, unsigned hi) {
+    return ex != kFxNonfinite && ex + kWeakBits > (int)(hi >> 20) - 1023;
+}
+__device__ __forceinline__ unsigned mag_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned mag_hi(double2 v) { return max(mag_hi(v.x), mag_hi(v.y)); }
+
 struct Upd64Bars {
     uint64_t a_full, a_empty, b_full[2], b_empty[2], acc_full[2], acc_empty[2];
     uint32_t tmem;
