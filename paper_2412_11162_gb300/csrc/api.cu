@@ -726,8 +726,8 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
     std::vector<double> mres(nm, 0.0), mbwd(nm, 0.0);
     if (precision == PMLBIE_FP64) {
         // the close-pair scratch is free after the assembly: the digit images of the
-        // updates live in it (about 20 corrections per node and more, 32 M bytes of
-        // Laplace modes each: more than one mode's images, 3 KB per row of the system)
+        // updates live in it (about 40 close pairs per node, 32 M bytes of Laplace modes each:
+        // at least three times one mode's images, 3 KB per row of the system)
         if ((rc = batched_lu_graphed(prob, PMLBIE_FP64, n2, nm, w.A, w.piv, w.info, (unsigned char*)w.zd, nullptr, s,
                                      w.near_bytes)))
             return rc;

@@ -1380,12 +1380,14 @@ size_t lu_image_bytes(int n, int batch) {
     return (size_t)batch * nblk * (tcu::kAImg + tcu::kBImg);
 }
 
-// complex128: per mode the first step's digit images and 2 n exponents
+// complex128: per mode the first step's digit images, 2 n exponents, the list of the
+// entries to form in FP64 (one per 16 x 16 block at most), and a counter
+static size_t lu_list64(int rem) { return (size_t)tcu::row_blocks64(rem) * 4 * tcu::col_blocks64(rem) * 2; }
 size_t lu_image64_bytes(int n) {
     if (n <= kNB) return 0;
     const int rem = n - kNB;
     return (size_t)tcu::row_blocks64(rem) * tcu::kAImg64 + (size_t)tcu::col_blocks64(rem) * tcu::kBImg64 +
-           sizeof(int) * 2 * (size_t)n;
+           sizeof(int) * 2 * ((size_t)n + 8) + sizeof(uint2) * lu_list64(rem);
 }
 
 template <typename T>
@@ -1492,14 +1494,20 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
                 // complex128: digit images and update, as many modes at a time as the
                 // scratch holds images of (the exponents behind the images)
                 const int nra = tcu::row_blocks64(rem), nca = tcu::col_blocks64(rem);
-                int* expo = reinterpret_cast<int*>(img + (size_t)group * (lu_image64_bytes(n) - sizeof(int) * 2 * (size_t)n));
+                // behind the images: the counter, the exponents and the list
+                int* count = reinterpret_cast<int*>(
+                    img + (size_t)group * ((size_t)tcu::row_blocks64(n - kNB) * tcu::kAImg64 +
+                                           (size_t)tcu::col_blocks64(n - kNB) * tcu::kBImg64));
+                int* expo = count + 2;
+                uint2* list = reinterpret_cast<uint2*>(expo + 2 * (size_t)group * n);
                 for (int b0 = 0; b0 < batch; b0 += group) {
                     const int g = std::min(group, batch - b0);
                     double2* Ab = reinterpret_cast<double2*>(A) + (size_t)b0 * n * n;
-                    tcu::operand_image64_kernel<<<dim3(nra + nca, g), 256, 0, s>>>(n, k0, nra, Ab, img, nca, expo);
+                    tcu::operand_image64_kernel<<<dim3(nra + nca, g), 256, 0, s>>>(n, k0, nra, Ab, img, nca, expo, count);
                     tcu::update64_kernel<<<std::min(g * nra, sms), tcu::kUpd64Threads, tcu::kUpd64Smem, s>>>(
-                        n, k0, g, Ab, img, expo, info + b0);
-                    count_launch(2);
+                        n, k0, g, Ab, img, expo, info + b0, list, count);
+                    tcu::weak64_kernel<<<2 * sms, tcu::kWeakThreads, 0, s>>>(n, k0, Ab, list, count);
+                    count_launch(3);
                 }
             }
             if (upd_ev && (ee = record_update_event(upd_ev[2 * (k0 / kNB) + 1], s)) != cudaSuccess) return ee;

@@ -13,12 +13,14 @@
 // the row's or column's largest entry, so entries are represented to 2^-63 of it).
 // Digit products are integers of at most 2^14; those of one weight s + t = q, summed
 // over at most 8 pairs and the real depth 64, stay below 2^23 and are exact in the
-// FP32 accumulators.  The 36 pairs with s + t <= 7 are kept (the dropped ones are
-// below 2^-60 of the row's times the column's largest entry).  An element of the
-// product is the combination of its eight accumulators in a 64-bit integer (unit
-// 2^{e_i + f_j - 56}), converted to double and subtracted from A22 with one rounding,
-// against 128 roundings of the FP64 dot product it replaces.  Rows or columns holding
-// a NaN or an infinity give NaN.
+// FP32 accumulators.  The 36 pairs with s + t <= 7 are kept; the dropped ones come to
+// about 2^-59 of the row's times the column's largest entry, 2^-51 at worst (all digits
+// of weight 8 at their largest and of one sign).  An element of the product is the
+// combination of its eight accumulators in a 64-bit integer, in units of 2^-54 or less
+// of the row's times the column's largest entry, converted to double and subtracted
+// from A22.  Elements that this unit is too coarse for (weak_sum) are left as they are
+// and formed in FP64 by weak64_kernel, so that every entry keeps what the FP64 dot
+// product gives it.  Rows or columns holding a NaN or an infinity give NaN.
 //
 // The complex product is one real GEMM of depth 64 (as in tc_update.cuh): A' row 2i =
 // (Re L, -Im L), row 2i + 1 = (Im L, Re L); B' = [Re U; Im U].  operand_image64_kernel
@@ -33,9 +35,10 @@
 // waited for).  Bounded waits as in tc_update.cuh; an expiry marks info[b] = -1.
 //
 // Measured (GB300), all updates of one factorisation, CUDA-core FP64 -> this: n = 512,
-// 64 modes 28.8 -> 2.6 ms, n = 320, 32 modes 3.6 -> 0.54 ms; FP64 solve at N = 256,
-// M = 128 41.5 -> 15.2 ms, N = 160, M = 64 9.7 -> 6.65 ms.  The operand images are
-// what the MMAs wait for next (A' is re-read from shared memory for every 32 columns).
+// 64 modes 28.8 -> 4.3 ms (of it the FP64 entries, 4 % of them, 1.7 ms, the operand
+// images 0.35), n = 320, 32 modes 3.6 -> 1.2 ms (0.64, 0.11).  The FP64 entries are bounded
+// by the FP64 pipe; the MMAs wait for the operand images next (A' is re-read from shared
+// memory for every 32 columns).
 #pragma once
 
 #include "fxdft.cuh"
@@ -74,8 +77,9 @@ __device__ __forceinline__ uint32_t digit_pair(u64 a, u64 b, int s) {
 // expo: per mode n entries, the exponent of row r at [r] and of column c at [n + c]
 // (kFxNonfinite for a row or column with a NaN or an infinity).
 __global__ void __launch_bounds__(256) operand_image64_kernel(int n, int k0, int nra, const double2* A,
-                                                              unsigned char* img, int nca, int* expo) {
+                                                              unsigned char* img, int nca, int* expo, int* count) {
     const int b = blockIdx.y, first = k0 + 32;
+    if (blockIdx.x == 0 && b == 0 && threadIdx.x == 0) *count = 0;
     const double2* a = A + (size_t)b * n * n;
     const bool rows = (int)blockIdx.x < nra;
     const int blk = rows ? blockIdx.x : blockIdx.x - nra;
@@ -177,7 +181,7 @@ static_assert(sizeof(Upd64Bars) <= 256, "barrier block");
 
 __global__ void __launch_bounds__(kUpd64Threads, 1) update64_kernel(int n, int k0, int batch, double2* A,
                                                                     const unsigned char* img, const int* expo,
-                                                                    int* info) {
+                                                                    int* info, uint2* list, int* count) {
     extern __shared__ __align__(1024) unsigned char sm[];
     Upd64Bars* bar = reinterpret_cast<Upd64Bars*>(sm + kOff64Bar);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -342,12 +346,23 @@ __global__ void __launch_bounds__(kUpd64Threads, 1) update64_kernel(int n, int k
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mb_arrive(&bar->acc_empty[s]);
+                unsigned weak = 0;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     // sum of 2^-12 2^-8q 2^(e + f) v_q with q = 2^62-scaled digits: exponent er + ec + 68
                     const int ex = (er == kFxNonfinite || ec[c] == kFxNonfinite) ? kFxNonfinite : er + ec[c] + 68;
-                    if (row < n && c0 + c < n) a[(size_t)(c0 + c) * n * 2] = cv[c] - fx_to_double(acc[c], ex);
+                    const double v = fx_to_double(acc[c], ex);
+                    unsigned hi = max(mag_hi(cv[c]), mag_hi(v));
+                    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, 1));      // the entry's other part
+                    if (row < n && c0 + c < n && weak_sum(ex, hi)) weak |= 1u << c;
+                    cv[c] -= v;
                 }
+                weak = __reduce_or_sync(0xffffffffu, weak);
+                if (weak && lane == 0)
+                    list[atomicAdd(count, 1)] = make_uint2((unsigned)b << 16 | weak, (unsigned)(row >> 4) << 16 | (c0 >> 4));
+#pragma unroll
+                for (int c = 0; c < 16; ++c)
+                    if (row < n && c0 + c < n && !(weak >> c & 1)) a[(size_t)(c0 + c) * n * 2] = cv[c];
             }
         }
     }
@@ -356,6 +371,38 @@ __global__ void __launch_bounds__(kUpd64Threads, 1) update64_kernel(int n, int k
     if (failed() && tid == 0)
         for (int u = blockIdx.x; u < U; u += G) info[u / nra] = -1;
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// The columns of 16 rows that update64_kernel left as they were, in FP64: a warp takes
+// one entry of the list (mode and mask of 16 columns, row / 16 and first column / 16);
+// two lanes share a row, half of the depth each.  An own launch, because the entries
+// lie in few row blocks: formed in the update's epilogue, one column after the other,
+// they held up the CTAs that own those rows.
+constexpr int kWeakThreads = 256;
+__global__ void __launch_bounds__(kWeakThreads) weak64_kernel(int n, int k0, double2* A, const uint2* list,
+                                                              const int* count) {
+    const int lane = threadIdx.x & 31, part = lane & 1, d0 = k0 + 16 * part, total = *count;
+    for (int i = (blockIdx.x * kWeakThreads + threadIdx.x) >> 5; i < total; i += gridDim.x * (kWeakThreads >> 5)) {
+        const uint2 e = list[i];
+        double2* m = A + (size_t)(e.x >> 16) * n * n;
+        const int row = (int)(e.y >> 16) * 16 + (lane >> 1), c0 = (int)(e.y & 0xffffu) * 16;
+        double2 l[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) l[k] = m[(size_t)(d0 + k) * n + min(row, n - 1)];
+        for (unsigned cols = e.x & 0xffffu; cols; cols &= cols - 1) {
+            double2* col = m + (size_t)(c0 + __ffs(cols) - 1) * n;
+            double re = 0.0, im = 0.0;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const double2 u = col[d0 + k];
+                re = fma(l[k].x, u.x, fma(-l[k].y, u.y, re));
+                im = fma(l[k].x, u.y, fma(l[k].y, u.x, im));
+            }
+            re += __shfl_xor_sync(0xffffffffu, re, 1);
+            im += __shfl_xor_sync(0xffffffffu, im, 1);
+            if (row < n) reinterpret_cast<double*>(col + row)[part] -= part ? im : re;
+        }
+    }
 }
 
 }  // namespace tcu

@@ -35,6 +35,13 @@ def test_factors_of_one_panel(n):
     check_factors(n)
 
 
+# tensor-core updates of 64 x 32 tiles: trailing blocks of 1 .. 66 rows, whole tiles, several
+# row blocks (of the three matrices two are updated together, then one)
+@pytest.mark.parametrize("n", [33, 34, 48, 64, 65, 96, 97, 98, 130, 160, 258])
+def test_factors_of_several_panels(n):
+    check_factors(n)
+
+
 def check_factors(n):
     import torch
     from paper_2412_11162_gb300 import binding as B
