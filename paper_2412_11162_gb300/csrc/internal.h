@@ -327,7 +327,7 @@ struct ProductArgs {
 };
 // From two right-hand sides on, the tensor cores (tc_product64.cuh): their time hardly
 // depends on the number up to 8 (n = 1600, 128 modes, one: 1.87 ms against 1.58 ms of the
-// FP64 kernel, whose time grows with them; n = 768, 96 modes, eight: 0.41 against 2.19 ms).
+// FP64 kernel, whose time grows with them; n = 768, 96 modes, eight: 0.70 against 2.19 ms).
 cudaError_t add_product_c128(const ProductArgs& a, int batch, cudaStream_t s);
 // R = B - A X with |R|^2, |B|^2, |X|^2 per (matrix, rhs)
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,

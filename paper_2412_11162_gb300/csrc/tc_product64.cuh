@@ -8,9 +8,10 @@
 // balanced base-256 digits (62 bits) below their largest entry in the chunk; the digits
 // are exact in fp16 (1024 + byte by a byte permutation, less 1152), the digit products of
 // one weight, summed over the real depth 64, stay below 2^23 and are exact in the FP32
-// accumulators; the weights are combined in a 64-bit integer (unit 2^-56 of the row's
-// times the column's largest entry), and the chunks' sums are added in FP64: one rounding
-// per chunk, against 64 of the dot product's.
+// accumulators; the weights are combined in a 64-bit integer (unit 2^-54 or less of the
+// row's times the column's largest entry in the chunk, the dropped pairs of digits as in the
+// update) and the chunks' sums are added in FP64.  A chunk's element that this unit is too
+// coarse for (weak_sum: large entries of A meet small ones of X) is formed in FP64.
 //
 // A CTA holds 128 rows and walks its chunks.  The complex product is a real one of depth
 // 64, A' = (Re A, Im A), and X' has, per right-hand side, the columns (Re x, -Im x) and
@@ -20,10 +21,11 @@
 // 16 depths instead of 36.  The digits of A are formed in shared memory in two halves of
 // 16 columns (64 KB), two CTAs to an SM cover each other's waits.
 // What bounds it is the integer work of the digits, about 50 instructions per entry, once
-// for up to 8 right-hand sides: n = 768, 96 modes, residual of 8 right-hand sides 2.19 ->
-// 0.41 ms (2.2 TB/s of the matrix).  Mixed solve for 64 waves (8 solved) at N = 384, M =
-// 192 29.7 -> 21.3 ms, four instances with 4 waves at N = 256 24.4 -> 20.0 ms.  Waits are
-// bounded; an expiry gives NaN.
+// for up to 8 right-hand sides, and the elements in FP64, some 10 % there: n = 768, 96 modes,
+// residual of 8 right-hand sides 2.19 -> 0.70 ms (0.51 without those elements).  Mixed solve
+// for 64 waves (8 solved) at N = 384, M = 192 15.9 -> 16.6 ms by those elements, four
+// instances with 4 waves at N = 256 16.5 -> 17.7 ms (all on the FP64 pipe about 7 and 3 ms more).
+// Waits are bounded; an expiry gives NaN.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -40,6 +42,9 @@ constexpr uint32_t kProdOffB = kProdA, kProdOffMax = kProdOffB + 2 * kProdBHalf;
 constexpr uint32_t kProdOffEx = kProdOffMax + 2 * kProdRows * 4, kProdOffBar = kProdOffEx + 32;
 constexpr uint32_t kProdSmem = kProdOffBar + 32;
 constexpr uint32_t kProdTmem = 128;
+// as kWeakBits, per chunk: the largest error by entry on the oracle's systems is below the
+// FP64 product's with 49, about equal with 48, twice with 47
+constexpr int kProdWeakBits = 49;
 
 // fp16 pair of digit s (0: top) of two values in digit_bytes form
 __device__ __forceinline__ uint32_t digit_half2(u64 a, u64 b, int s) {
@@ -203,10 +208,34 @@ __global__ void __launch_bounds__(kProdThreads, 2) product64_kernel(ProductArgs 
                         acc[c] = (acc[c] << 4) + ((w + 2048) >> 12);
                 }
             }
+            unsigned weak = 0;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int eq = exq[4 * hf + (c >> 1)];
-                sum[c] += fx_to_double(acc[c], (top == 0x7ff || eq == kFxNonfinite) ? kFxNonfinite : ex + eq + 68);
+            for (int q = 0; q < 4; ++q) {
+                const int eq = exq[4 * hf + q];
+                const int e = (top == 0x7ff || eq == kFxNonfinite) ? kFxNonfinite : ex + eq + 68;
+                const double vr = fx_to_double(acc[2 * q], e), vi = fx_to_double(acc[2 * q + 1], e);
+                const unsigned hi = max(max(mag_hi(vr), mag_hi(vi)), max(mag_hi(sum[2 * q]), mag_hi(sum[2 * q + 1])));
+                if (row < end && 4 * hf + q < nq && weak_sum(e, hi, kProdWeakBits)) {
+                    weak |= 1u << q;
+                } else {
+                    sum[2 * q] += vr;
+                    sum[2 * q + 1] += vi;
+                }
+            }
+            if (weak) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (weak >> q & 1) {
+                        double sr = 0.0, si = 0.0;
+#pragma unroll 8
+                        for (int c = 0; c < cw; ++c) {
+                            const double2 w = __ldg(Ac + (size_t)c * a.ld), y = x[(size_t)(c0 + c) * a.nrhs + r0 + 4 * hf + q];
+                            sr = fma(w.x, y.x, fma(-w.y, y.y, sr));
+                            si = fma(w.x, y.y, fma(w.y, y.x, si));
+                        }
+                        sum[2 * q] += sr;
+                        sum[2 * q + 1] += si;
+                    }
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -165,9 +165,11 @@ __device__ __forceinline__ int acc_int(uint32_t bits) {
 // digits lie below the row's and the column's largest entry, and the entry itself can be
 // smaller by any factor (the modal kernels of high modes fall off like (rho / rho')^n
 // next to the axis).  Such entries are formed again in FP64.
+// (50: the factors of the oracle's systems then are as close to P A entry by entry as in
+// FP64; with 48 and 46 two and five to twenty times as far.)
 constexpr int kWeakBits = 50;
-__device__ __forceinline__ bool weak_sum(int ex, unsigned hi) {
-    return ex != kFxNonfinite && ex + kWeakBits > (int)(hi >> 20) - 1023;
+__device__ __forceinline__ bool weak_sum(int ex, unsigned hi, int bits = kWeakBits) {
+    return ex != kFxNonfinite && ex + bits > (int)(hi >> 20) - 1023;
 }
 __device__ __forceinline__ unsigned mag_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 __device__ __forceinline__ unsigned mag_hi(double2 v) { return max(mag_hi(v.x), mag_hi(v.y)); }

@@ -4,7 +4,8 @@ bits relative to a row's and a column's largest entry, a double relative to the 
 Bar for every entry of P A - L U: (8 sqrt(n) + 16) u of the entry of |L| |U| (u = 2^-53).
 A complex multiply-add errs by at most (1 + sqrt 5) u of its terms, a sum of n of them by
 4 sqrt(n) u with errors of independent signs, in the elimination and again in the test's
-own product; a pivot's reciprocal and the product with it by 16 u.
+own product; a pivot's reciprocal and the product with it by 16 u.  Products A X against
+the same bar times the entry of |A| |X|.
 """
 import numpy as np
 import pytest
@@ -55,3 +56,19 @@ def check_factors(n):
         assert np.max(np.abs(L)) <= 1 + 4 * U            # partial pivoting
         ratio = np.abs(A[b][perm[b]] - L @ R) / (np.abs(L) @ np.abs(R))
         assert np.max(ratio) <= bar(n), (b, np.max(ratio) / U, np.unravel_index(np.argmax(ratio), ratio.shape))
+
+
+# row blocks of 128 and column chunks of 32 (of either half of the columns) with remainders,
+# groups of 8 right-hand sides with remainders, one right-hand side; X of any scale from
+# row to row
+@pytest.mark.parametrize("n,waves", [(2, 2), (62, 2), (64, 3), (66, 8), (130, 9), (190, 16), (258, 17), (258, 1)])
+def test_products(n, waves):
+    import torch
+    from paper_2412_11162_gb300 import binding as B
+    A, rng = matrices(n, n), np.random.default_rng(waves)
+    X = rng.standard_normal((3, n, waves)) + 1j * rng.standard_normal((3, n, waves))
+    X *= 2.0 ** rng.integers(-40, 41, (3, n, 1))
+    Y = torch.empty((3, n, waves), dtype=torch.complex128, device="cuda")
+    B.pmlbie_selftest_product(torch.tensor(A.transpose(0, 2, 1).copy(), device="cuda"), torch.tensor(X, device="cuda"), Y)
+    ratio = np.abs(Y.cpu().numpy() - A @ X) / (np.abs(A) @ np.abs(X))
+    assert np.max(ratio) <= bar(n), (np.max(ratio) / U, np.unravel_index(np.argmax(ratio), ratio.shape))
