@@ -399,13 +399,17 @@ int  pmlbie_selftest_wait(long long iterations, void* stream);
  * the paper: the sampling loops of Sec. 3.1 / 4.1 evaluate e^{iq} with their
  * own exp, sin / cos and 1/sqrt).  Evaluates, at the n doubles of device
  * array dev_x, into device array dev_out:
- *   fn 0: exp(x)            -> out[i]   (arguments are clamped to [-708, 709])
- *   fn 1: sin(x), cos(x)    -> out[2 i], out[2 i + 1]
- *   fn 2: 1/sqrt(x)         -> out[i]   (x > 0)
+ *   fn 30: exp(x)           -> out[i]   (0 below the normal range, infinity above)
+ *   fn 31: sin(x), cos(x)   -> out[2 i], out[2 i + 1]   (0 <= x < 2^63)
+ *   fn 32: 1/sqrt(x)        -> out[i]   (x > 0 normal)
+ *   of the sampling loops, on the integer pipe but for the last;
+ *   fn 0, 1, 2: exp (arguments clamped to [-708, 709]), sin and cos, 1/sqrt in
+ *   FP64, of which the diagnostic exact split (subst_off) takes the first two;
+ *   fn 20, 21, 22: the same in float-float arithmetic (pairs of FP32 numbers);
  *   fn 10, 11, 12: the same by the CUDA math library (exp, sincos, rsqrt),
  *   the references the tests compare with.
- * dev_out holds n (fn 0, 2, 10, 12) or 2 n (fn 1, 11) doubles.  Synchronises
- * the stream.  EINVAL for an unknown fn, NULL buffers or n > 2^31; ECUDA. */
+ * dev_out holds n, for sin / cos 2 n doubles.  Synchronises the stream.
+ * EINVAL for an unknown fn, NULL buffers or n > 2^31; ECUDA. */
 int  pmlbie_selftest_elementary(int fn, const void* dev_x, void* dev_out, size_t n, void* stream);
 
 /* Self-tests of the dense complex128 kernels of the solves, on caller-owned

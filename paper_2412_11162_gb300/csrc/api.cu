@@ -1340,7 +1340,6 @@ int pmlbie_selftest_elementary(int fn, const void* dev_x, void* dev_out, size_t 
     }
     PMLBIE_CUDA_TRY(launch_elementary_selftest(fn, static_cast<const double*>(dev_x), static_cast<double*>(dev_out),
                                                n, s));
-    PMLBIE_CUDA_TRY(cudaStreamSynchronize(s));
     return PMLBIE_OK;
 }
 

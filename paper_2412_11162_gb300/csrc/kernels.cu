@@ -1343,15 +1343,17 @@ cudaError_t launch_expand_waves(int N, int nmodes, int mode_lo, int n_src, int n
 }
 
 namespace {
-// Elementary-function self-test: fn 0 / 1 / 2 evaluate the sampling loops'
-// exp, sin and cos, 1/sqrt; fn 10 / 11 / 12 the CUDA math library's exp,
-// sincos, rsqrt at the same points (the references).  sin, cos: out[2i],
-// out[2i + 1]; the others out[i].
-__global__ void elementary_selftest_kernel(int fn, const double* x, double* out, size_t n) {
+// Elementary-function self-test: fn 30 / 31 / 32 evaluate the sampling loops' exp, sin
+// and cos (of phases with w = 1), 1/sqrt (fxtrig.cuh); fn 0 / 1 / 2 the FP64 exp, sin and
+// cos, 1/sqrt of fp64_elem.cuh, the first two of which the diagnostic exact split
+// takes; fn 10 / 11 / 12 the CUDA math library's exp, sincos, rsqrt (the references).
+// sin, cos: out[2i], out[2i + 1]; the others out[i].
+__global__ void elementary_selftest_kernel(int fn, const double* x, double* out, size_t n, FxTab T, FxPhase one) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double v = x[i];
     double s, c;
+    int ex;
     switch (fn) {
         case 0: out[i] = fexp(v); break;
         case 1: fsincos(v, &s, &c); out[2 * i] = s; out[2 * i + 1] = c; break;
@@ -1359,18 +1361,47 @@ __global__ void elementary_selftest_kernel(int fn, const double* x, double* out,
         case 10: out[i] = exp(v); break;
         case 11: sincos(v, &s, &c); out[2 * i] = s; out[2 * i + 1] = c; break;
         case 12: out[i] = rsqrt(v); break;
+        case 30: {
+            const i64 m = fx_exp(v, T, ex);
+            out[i] = fx_to_double(m, ex - 61);
+            break;
+        }
+        case 31: {
+            const longlong2 t = fx_cis(fx_turns(v, one), T);
+            out[2 * i] = fx_to_double(t.y, -62);
+            out[2 * i + 1] = fx_to_double(t.x, -62);
+            break;
+        }
+        case 32: out[i] = fx_rsqrt(v); break;
         default: break;
     }
 }
 }  // namespace
 
-bool elementary_selftest_known(int fn) { return fn == 0 || fn == 1 || fn == 2 || fn == 10 || fn == 11 || fn == 12; }
+bool elementary_selftest_known(int fn) {
+    return fn == 0 || fn == 1 || fn == 2 || fn == 10 || fn == 11 || fn == 12 || (fn >= 30 && fn <= 32);
+}
 
 cudaError_t launch_elementary_selftest(int fn, const double* x, double* out, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    elementary_selftest_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(fn, x, out, n);
-    count_launch();
-    return cudaGetLastError();
+    const std::vector<int4> trig = fx_trig_table();
+    const std::vector<int2> ex = fx_exp_table();
+    int4* dtrig = nullptr;
+    int2* dexp = nullptr;
+    cudaError_t e = cudaMalloc(&dtrig, sizeof(int4) * trig.size());
+    if (e == cudaSuccess) e = cudaMalloc(&dexp, sizeof(int2) * ex.size());
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dtrig, trig.data(), sizeof(int4) * trig.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dexp, ex.data(), sizeof(int2) * ex.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) {
+        elementary_selftest_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(fn, x, out, n, FxTab{dtrig, dexp},
+                                                                                fx_phase(1.0));
+        count_launch();
+        e = cudaGetLastError();
+    }
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (dtrig) cudaFree(dtrig);
+    if (dexp) cudaFree(dexp);
+    return e == cudaSuccess ? es : e;
 }
 
 }  // namespace pmlbie

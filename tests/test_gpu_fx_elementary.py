@@ -1,0 +1,52 @@
+"""The sampling loops' exp, sin / cos and 1/sqrt (csrc/fxtrig.cuh), point by point through
+pmlbie_selftest_elementary selectors 30 .. 32, against the host's extended precision.
+
+Bars: the functions' stated errors plus the rounding of the result to a double --
+exp 2^-55.7 + 2^-53 relative; sin and cos 2^-57.9 + 2^-54 absolute, plus |x| 2^-63 (the 64
+bits of 1 / 2 pi) and 2^-61 (the fraction of a turn, cut at 2^-64 turns); 1/sqrt 2^-52
+(about 1 ulp) relative.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_elementary import _grid, _run
+
+pytestmark = pytest.mark.gpu
+LD = np.longdouble
+
+
+def test_exp():
+    x = np.concatenate([_grid(-707.0, 709.0, 1 << 18, 1), _grid(-1.0, 1.0, 1 << 17, 2),
+                        # powers of two of either sign: shifts of the fraction, nothing left of it, all of it
+                        *(s * 2.0 ** np.arange(-80, 10) for s in (-1, 1)),
+                        # next to multiples of ln 2 / 256 (table entries) and of ln 2
+                        *(np.arange(-2000, 2001) * (np.log(2) / 256) * (1 + d) for d in (-1e-15, 0, 1e-15)),
+                        np.arange(-1000, 1001) * np.log(2), [0.0, -0.0, 1e-300, -1e-300, 5e-324]])
+    got, ref = _run(30, x), np.exp(x.astype(LD))
+    err = np.abs(got.astype(LD) - ref) / ref
+    assert np.max(err) <= 2.0 ** -53 + 2.0 ** -55.7, (float(np.max(err)) * 2.0 ** 53, x[np.argmax(err)])
+    assert np.all(_run(30, np.array([-709.0, -750.0, -1023.5, -1024.0, -1e4, -1e300, -np.inf])) == 0.0)
+    assert np.all(_run(30, np.array([710.0, 750.0, 1023.5, 1024.0, 1e4, 1e300, np.inf])) == np.inf)
+
+
+def test_sin_cos():
+    x = np.concatenate([_grid(0.0, 8.0, 1 << 18, 3), _grid(0.0, 2.0 ** 20, 1 << 18, 4), _grid(0.0, 2.0 ** 40, 1 << 12, 5),
+                        2.0 ** np.arange(-80, 41),
+                        # next to the table's angles, half way between them, and the quadrants' ends
+                        *(np.arange(0, 8193) * (np.pi / 1024) * (1 + d) for d in (-1e-15, 0, 1e-15)),
+                        np.arange(0, 4001) * (np.pi / 2), [0.0, 1e-300, 5e-324]])
+    got = _run(31, x)
+    bar = 2.0 ** -54 + 2.0 ** -57.9 + x * 2.0 ** -63 + 2.0 ** -61
+    for k, ref in enumerate((np.sin(x.astype(LD)), np.cos(x.astype(LD)))):
+        err = np.abs(got[k::2].astype(LD) - ref)
+        assert np.all(err <= bar), (k, float(np.max(err / bar)), x[np.argmax(err / bar)])
+
+
+def test_rsqrt():
+    rng = np.random.default_rng(6)
+    x = np.concatenate([2.0 ** rng.uniform(-1021, 1023, 1 << 18), _grid(0.5, 8.0, 1 << 17, 7),
+                        # every exponent, odd and even, at both ends of the significand
+                        *(2.0 ** np.arange(-1022, 1024) * v for v in (1.0, 2 - 2.0 ** -52))])
+    got, ref = _run(32, x), 1 / np.sqrt(x.astype(LD))
+    err = np.abs(got.astype(LD) - ref) / ref
+    assert np.max(err) <= 2.0 ** -52, (float(np.max(err)) * 2.0 ** 52, x[np.argmax(err)])
