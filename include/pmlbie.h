@@ -402,7 +402,8 @@ int  pmlbie_selftest_wait(long long iterations, void* stream);
  *   fn 30: exp(x)           -> out[i]   (0 below the normal range, infinity above)
  *   fn 31: sin(x), cos(x)   -> out[2 i], out[2 i + 1]   (0 <= x < 2^63)
  *   fn 32: 1/sqrt(x)        -> out[i]   (x > 0 normal)
- *   of the sampling loops, on the integer pipe but for the last;
+ *   of the sampling loops, on the integer pipe but for the last,
+ *   fn 33, 34: sin(x)/x, (sin x - x cos x)/x^3 -> out[i]   (x > 0) of the close pairs;
  *   fn 0, 1, 2: exp (arguments clamped to [-708, 709]), sin and cos, 1/sqrt in
  *   FP64, of which the diagnostic exact split (subst_off) takes the first two;
  *   fn 20, 21, 22: the same in float-float arithmetic (pairs of FP32 numbers);

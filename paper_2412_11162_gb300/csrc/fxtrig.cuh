@@ -143,5 +143,25 @@ __device__ __forceinline__ double2 fx_expi(double2 R, double qy, FxPhase w, cons
     return c2(fx_to_double(fx_mul(c.x, h, l), ex - 61), fx_to_double(fx_mul(c.y, h, l), ex - 61));
 }
 
+// sin(q)/q and (sin q - q cos q)/q^3 of a real phase q from its sine and cosine and iq = 1/q;
+// below kSmallPhase, where the differences would magnify the rounding of sn and cs
+// (absolute, about 2^-54) by 1/q and 3/q^2, their power series (terms left out below 2^-60)
+constexpr double kSmallPhase = 0.5;
+__device__ __forceinline__ void fx_sinc_h4(double q, double iq, double sn, double cs, double& sinc, double& h4) {
+    if (fabs(q) < kSmallPhase) {
+        const double x = -q * q;
+        constexpr double s[8] = {1.0, 1.0 / 6, 1.0 / 120, 1.0 / 5040, 1.0 / 362880, 1.0 / 39916800, 1.0 / 6227020800.0,
+                                 1.0 / 1307674368000.0};
+        constexpr double h[8] = {1.0 / 3, 1.0 / 30, 1.0 / 840, 1.0 / 45360, 1.0 / 3991680, 1.0 / 518918400.0,
+                                 1.0 / 93405312000.0, 1.0 / 22230464256000.0};
+        sinc = s[7], h4 = h[7];
+#pragma unroll
+        for (int k = 6; k >= 0; --k) sinc = fma(sinc, x, s[k]), h4 = fma(h4, x, h[k]);
+    } else {
+        sinc = sn * iq;
+        h4 = fma(-q, cs, sn) * (iq * iq * iq);
+    }
+}
+
 }  // namespace
 }  // namespace pmlbie

@@ -539,11 +539,8 @@ __global__ void __launch_bounds__(near_threads(NB), NB <= 2 ? 4 : NB <= 4 ? 2 : 
                 const double qr = w * R.x, iq = iR.x / w;
                 const longlong2 t = fx_cis(fx_turns(R.x, a.T.ph[r]), TB);
                 const double cs = fx_to_double(t.x, -62), sn = fx_to_double(t.y, -62);
-                const double q2 = qr * qr;
-                const double sinc = fabs(qr) < 1e-3 ? 1.0 - q2 / 6.0 + q2 * q2 / 120.0 : sn * iq;
-                const double h4 = fabs(qr) < 1e-2
-                                      ? 1.0 / 3.0 - q2 / 30.0 + q2 * q2 / 840.0 - q2 * q2 * q2 / 45360.0
-                                      : (sn - qr * cs) * (iq * iq * iq);
+                double sinc, h4;
+                fx_sinc_h4(qr, iq, sn, cs, sinc, h4);
                 f1[r] = cs;
                 r1[r] = w * kInv4Pi * sinc;
                 f3[r] = fma(qr, sn, cs);
@@ -1344,7 +1341,8 @@ cudaError_t launch_expand_waves(int N, int nmodes, int mode_lo, int n_src, int n
 
 namespace {
 // Elementary-function self-test: fn 30 / 31 / 32 evaluate the sampling loops' exp, sin
-// and cos (of phases with w = 1), 1/sqrt (fxtrig.cuh); fn 0 / 1 / 2 the FP64 exp, sin and
+// and cos (of phases with w = 1), 1/sqrt (fxtrig.cuh), fn 33 / 34 the close pairs' sin(q)/q
+// and (sin q - q cos q)/q^3; fn 0 / 1 / 2 the FP64 exp, sin and
 // cos, 1/sqrt of fp64_elem.cuh, the first two of which the diagnostic exact split
 // takes; fn 10 / 11 / 12 the CUDA math library's exp, sincos, rsqrt (the references).
 // sin, cos: out[2i], out[2i + 1]; the others out[i].
@@ -1373,13 +1371,20 @@ __global__ void elementary_selftest_kernel(int fn, const double* x, double* out,
             break;
         }
         case 32: out[i] = fx_rsqrt(v); break;
+        case 33:
+        case 34: {
+            const longlong2 t = fx_cis(fx_turns(v, one), T);
+            fx_sinc_h4(v, 1.0 / v, fx_to_double(t.y, -62), fx_to_double(t.x, -62), s, c);
+            out[i] = fn == 33 ? s : c;
+            break;
+        }
         default: break;
     }
 }
 }  // namespace
 
 bool elementary_selftest_known(int fn) {
-    return fn == 0 || fn == 1 || fn == 2 || fn == 10 || fn == 11 || fn == 12 || (fn >= 30 && fn <= 32);
+    return fn == 0 || fn == 1 || fn == 2 || fn == 10 || fn == 11 || fn == 12 || (fn >= 30 && fn <= 34);
 }
 
 cudaError_t launch_elementary_selftest(int fn, const double* x, double* out, size_t n, cudaStream_t s) {

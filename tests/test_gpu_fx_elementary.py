@@ -4,7 +4,9 @@ pmlbie_selftest_elementary selectors 30 .. 32, against the host's extended preci
 Bars: the functions' stated errors plus the rounding of the result to a double --
 exp 2^-55.7 + 2^-53 relative; sin and cos 2^-57.9 + 2^-54 absolute, plus |x| 2^-63 (the 64
 bits of 1 / 2 pi) and 2^-61 (the fraction of a turn, cut at 2^-64 turns); 1/sqrt 2^-52
-(about 1 ulp) relative.
+(about 1 ulp) relative.  sin(q)/q, at most 1, to 2^-51 and (sin q - q cos q)/q^3, at most
+1/3, to 2^-50: their series below q = 1/2 to an ulp; above, the sine's rounding over q
+and, of the difference, (2^-57.9 + 2^-53 q) 8 at q = 1/2.
 """
 import numpy as np
 import pytest
@@ -50,3 +52,20 @@ def test_rsqrt():
     got, ref = _run(32, x), 1 / np.sqrt(x.astype(LD))
     err = np.abs(got.astype(LD) - ref) / ref
     assert np.max(err) <= 2.0 ** -52, (float(np.max(err)) * 2.0 ** 52, x[np.argmax(err)])
+
+
+def test_small_phase_quotients():
+    q = np.concatenate([np.exp(_grid(np.log(1e-12), np.log(30.0), 1 << 18, 8)), _grid(0.0005, 2.0, 1 << 17, 9),
+                        *(v * (1 + np.array([-1e-9, 0.0, 1e-9])) for v in (1e-3, 1e-2, 0.5))])
+    x = q.astype(LD)
+    s, k = np.zeros_like(x), np.zeros_like(x)
+    ts, tk = np.ones_like(x), np.ones_like(x) / 3          # power series, all terms that count for q < 1
+    for j in range(16):
+        s, k = s + ts, k + tk
+        ts = ts * -x * x / ((2 * j + 2) * (2 * j + 3))
+        tk = tk * -x * x / ((2 * j + 2) * (2 * j + 5))
+    big = x > 1
+    s[big], k[big] = np.sin(x[big]) / x[big], (np.sin(x[big]) - x[big] * np.cos(x[big])) / x[big] ** 3
+    for fn, ref, bar in ((33, s, 2.0 ** -51), (34, k, 2.0 ** -50)):
+        err = np.abs(_run(fn, q).astype(LD) - ref)
+        assert np.max(err) <= bar, (fn, float(np.max(err)) * 2.0 ** 53, q[np.argmax(err)])
