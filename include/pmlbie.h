@@ -296,11 +296,17 @@ int  pmlbie_modal_kernels_noalloc(pmlbie_problem* prob, int mode_lo, int mode_hi
  * refinement with FP64 residuals of those matrices until, for
  * every mode and right-hand side, the relative residual is <= 1e-13, or the
  * normwise backward error |B - A x| / (|A|_F |x| + |B|) is <= 1e-16, or it has
- * stopped decreasing (the FP64 floor) at <= 4e-16 in refinement or <= 1e-14 in
- * GMRES; modes whose refinement stalls above that (condition number x FP32 LU error near 1 or above)
- * are restarted and solved by flexible GMRES in FP64 preconditioned by the
- * same LU.  Errors: EINVAL, ENOMEM, ECUDA, ESINGULAR, ENOCONVERGE (mixed: a
- * mode missed both tolerances after the iteration caps; outputs still
+ * stopped decreasing at <= 4e-16 (the FP64 floor); modes whose refinement
+ * stalls above that (condition number x FP32 LU error near 1 or above) are
+ * solved by flexible GMRES in FP64 preconditioned by the same LU, up to the
+ * same tolerances or a backward error <= 1e-14 that a cycle lowers by less
+ * than 10 % or that is left after the last cycle (modes that refinement left
+ * at <= 1e-14 keep its result when there is no memory for the Krylov bases).
+ * FP64: factorisation and products as accurate, entry by entry, as in
+ * complex128 arithmetic.  Both: entries of the modal kernels are accurate
+ * relative to the largest sample of their node pair.
+ * Errors: EINVAL, ENOMEM, ECUDA, ESINGULAR, ENOCONVERGE (mixed: a
+ * mode missed the tolerances after the iteration caps; outputs still
  * written), ETIMEOUT (a bounded wait of the tensor-core LU update expired),
  * ENAN (NaN or Inf in an output; outputs written).  Inside the call some
  * kernels run on the problem's own streams (the close-pair kernels beside

@@ -8,6 +8,7 @@
 #include <thread>
 
 #include "internal.h"
+#include "refine_rules.h"
 
 using namespace pmlbie;
 
@@ -198,19 +199,6 @@ struct Workspace {
 
 constexpr int kGmresM = 20;          // FGMRES restart length
 constexpr int kGmresCycles = 10;     // FGMRES restarts at most
-// a mode's refinement is done when, for every rhs, the relative residual
-// |B - A x| / |B| <= kTolRel or the normwise backward error
-// |B - A x| / (|A|_F |x| + |B|) <= kTolBwd, or when the backward error is
-// below kTolFloor and stopped decreasing (the FP64 floor of ill-conditioned
-// modes, whose |A| |x| >> |B|)
-constexpr double kTolRel = 1e-13;
-constexpr double kTolBwd = 1e-16;
-constexpr double kTolFloor = 1e-14;
-// a refinement that no longer halves its backward error is at the FP64 floor only below
-// kTolFloorIr: above it the FP32 factors contract too slowly (a factor near 1 a step
-// looks the same), and FGMRES takes the mode over, which stops on kTolFloor when a cycle
-// gains less than 10 %
-constexpr double kTolFloorIr = 4e-16;
 
 // order of the complex64 factors of an n x n system: whole 32-row blocks
 int padded_order(int n) { return (n + 31) / 32 * 32; }
@@ -777,15 +765,10 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
                     }
                     mres[mo] = worst;
                     mbwd[mo] = wbwd;
-                    const bool stalled = iters >= 2 && !(wbwd < 0.5 * prev[mo]);
-                    if (ok || (stalled && wbwd <= kTolFloorIr)) {
-                        act[mo] = 0;     // done, or at the FP64 floor
-                    } else if (stalled) {
-                        act[mo] = 0;     // contraction too slow or divergent: FGMRES
-                        slow[mo] = 1;
-                    } else {
-                        ++nact;
-                    }
+                    const RefineStep step = refine_rule(iters, ok, wbwd, prev[mo]);
+                    act[mo] = step == RefineStep::kContinue;
+                    slow[mo] = step == RefineStep::kSlow;     // FGMRES
+                    nact += act[mo];
                     prev[mo] = wbwd;
                     if (iters == 1) first[mo] = wbwd;
                 }
@@ -799,34 +782,42 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
             }
             PMLBIE_CUDA_TRY(refine_step(n2, np2, nm, n_rhs, w.A32, w.piv, w.R, w.w32, w.X, s, w.active, w.dinv, w.ptab));
         }
-        const int nslow = (int)std::count(slow.begin(), slow.end(), 1);
-        if (nslow > 0) {
-            const size_t per = (size_t)n2 * n_rhs * sizeof(double2);
-            for (int mo = 0; mo < nm; ++mo)
-                // FGMRES starts from the refinement's last iterate when that
-                // improved on the first one, else (divergence) from zero
-                if (slow[mo] && !(mbwd[mo] < first[mo]))
-                    PMLBIE_CUDA_TRY(cudaMemsetAsync((char*)w.X + per * mo, 0, per, s));
-            int git = 0;
-            // FGMRES on the contiguous range of modes [g0, g1) holding every
-            // slow mode (its Krylov bases allocated for that range only)
-            int g0 = nm, g1 = 0;
+        int nslow = (int)std::count(slow.begin(), slow.end(), 1), g0 = 0, g1 = 0;
+        // FGMRES on the contiguous range of modes [g0, g1) holding every slow mode (its
+        // Krylov bases allocated for that range only); without memory for it, on the
+        // modes that refinement left above the level that FGMRES accepts
+        void* gm = nullptr;
+        for (int tries = 0; nslow > 0 && !gm; ++tries) {
+            g0 = nm, g1 = 0;
             for (int mo = 0; mo < nm; ++mo)
                 if (slow[mo]) g0 = std::min(g0, mo), g1 = mo + 1;
-            const int gn = g1 - g0;
-            void* gm = nullptr;
-            const size_t gbytes = gmres_scratch_bytes(n2, gn, n_rhs, kGmresM);
+            const size_t gbytes = gmres_scratch_bytes(n2, g1 - g0, n_rhs, kGmresM);
             if (cudaMalloc(&gm, gbytes) != cudaSuccess) {
                 cudaGetLastError();
-                return fail(PMLBIE_ENOMEM, "FGMRES scratch allocation failed (" + std::to_string(gbytes) + " bytes)");
+                gm = nullptr;
+                if (tries > 0) return fail(PMLBIE_ENOMEM, "FGMRES scratch allocation failed (" + std::to_string(gbytes) + " bytes)");
+                nslow = accept_refined(slow, mbwd);
+            }
+        }
+        if (nslow > 0) {
+            const size_t per = (size_t)n2 * n_rhs * sizeof(double2);
+            int git = 0;
+            const int gn = g1 - g0;
+            cudaError_t ez = cudaSuccess;
+            for (int mo = g0; mo < g1 && ez == cudaSuccess; ++mo)
+                if (slow[mo] && restart_from_zero(mbwd[mo], first[mo]))
+                    ez = cudaMemsetAsync((char*)w.X + per * mo, 0, per, s);
+            if (ez != cudaSuccess) {
+                cudaFree(gm);
+                return fail(PMLBIE_ECUDA, std::string("FGMRES start: ") + cudaGetErrorString(ez));
             }
             std::vector<int> gslow(slow.begin() + g0, slow.begin() + g1);
             std::vector<double> gan(an.begin() + g0, an.begin() + g1), gres(mres.begin() + g0, mres.begin() + g1),
                 gbwd(mbwd.begin() + g0, mbwd.begin() + g1);
             const size_t mat = (size_t)n2 * n2, vec = (size_t)n2 * n_rhs;
             rc = gmres_refine(n2, np2, gn, n_rhs, w.A + g0 * mat, w.A32 + (size_t)g0 * np2 * np2, w.piv + (size_t)g0 * np2,
-                              w.B + g0 * vec, w.X + g0 * vec, gslow, w.active, gm, kGmresM, kGmresCycles, kTolRel,
-                              kTolBwd, kTolFloor, gan, s, git, gres, gbwd,
+                              w.B + g0 * vec, w.X + g0 * vec, gslow, w.active, gm, kGmresM, kGmresCycles, gan, s, git,
+                              gres, gbwd,
                               w.dinv + (size_t)g0 * diag_inv_elems(np2), w.ptab + (size_t)g0 * lu_ptab_elems(np2, 1));
             cudaStreamSynchronize(s);
             cudaFree(gm);

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "refine_rules.h"
 
 namespace pmlbie {
 
@@ -280,7 +281,7 @@ size_t gmres_scratch_bytes(int n, int batch, int nrhs, int m) {
 
 int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const float2* LU32, const int* piv,
                  const double2* B, double2* X, std::vector<int>& act, int* active_dev, void* scratch, int m,
-                 int max_cycles, double tol, double tol_bw, double tol_floor, const std::vector<double>& an2,
+                 int max_cycles, const std::vector<double>& an2,
                  cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
                  const float2* dinv, const int2* ptab) {
     const size_t vec = (size_t)batch * n * nrhs, ninst = (size_t)batch * nrhs;
@@ -331,8 +332,8 @@ int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const flo
         GM_TRY(cudaMemcpyAsync(rn2.data(), beta2, sizeof(double) * ninst, cudaMemcpyDeviceToHost, s));
         GM_TRY(cudaMemcpyAsync(xn2.data(), xn2d, sizeof(double) * ninst, cudaMemcpyDeviceToHost, s));
         GM_TRY(cudaStreamSynchronize(s));
-        // converged: relative residual <= tol or normwise backward error
-        // |r| / (|A|_F |x| + |b|) <= tol_bw, for every rhs of the mode
+        // converged: relative residual <= kTolRel or normwise backward error
+        // |r| / (|A|_F |x| + |b|) <= kTolBwd, for every rhs of the mode
         int nact = 0;
         for (int b = 0; b < batch; ++b) {
             if (!act[b]) continue;
@@ -345,16 +346,14 @@ int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const flo
                 const double rel = bn > 0 ? rn / bn : 0.0, bwd = den > 0 ? rn / den : 0.0;
                 worst = std::max(worst, rel);
                 wbwd = std::max(wbwd, bwd);
-                if (!(rel <= tol || bwd <= tol_bw)) ok = false;
-                target[t] = 0.5 * std::max(tol * bn, tol_bw * den);
+                if (!(rel <= kTolRel || bwd <= kTolBwd)) ok = false;
+                target[t] = 0.5 * std::max(kTolRel * bn, kTolBwd * den);
                 hist[t].clear();
             }
-            // after a cycle: also done at the FP64 floor (backward error below
-            // tol_floor that the last cycle did not lower by 10 %)
-            const bool floor = cyc > 0 && wbwd <= tol_floor && wbwd >= 0.9 * mode_bwd[b];
+            const bool done = gmres_rule(ok, cyc, max_cycles, wbwd, mode_bwd[b]);
             mode_res[b] = worst;
             mode_bwd[b] = wbwd;
-            if (ok || floor) act[b] = 0;
+            if (done) act[b] = 0;
             else ++nact;
         }
         if (nact == 0 || cyc == max_cycles) break;

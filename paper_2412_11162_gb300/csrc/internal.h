@@ -304,13 +304,12 @@ cudaError_t convert_to_c64(int64_t count, const double2* src, float2* dst, cudaS
 cudaError_t convert_fro2_c128(int n, int np, int batch, const double2* A, float2* A32, double* out, cudaStream_t s);
 // Flexible GMRES (FP64, right-preconditioned by the FP32 LU) for the modes with
 // act[b] = 1; X holds the start and receives the solution; act is cleared for
-// converged modes (relative residual <= tol or normwise backward error
-// |r| / (|A|_F |x| + |b|) <= tol_bw; an2 = |A_b|_F^2), mode_res / mode_bwd
+// converged modes (gmres_rule of refine_rules.h; an2 = |A_b|_F^2), mode_res / mode_bwd
 // receive their final relative residuals and backward errors.
 size_t gmres_scratch_bytes(int n, int batch, int nrhs, int m);
 int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const float2* LU32, const int* piv,
                  const double2* B, double2* X, std::vector<int>& act, int* active_dev, void* scratch, int m,
-                 int max_cycles, double tol, double tol_bw, double tol_floor, const std::vector<double>& an2,
+                 int max_cycles, const std::vector<double>& an2,
                  cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
                  const float2* dinv = nullptr, const int2* ptab = nullptr);
 // Y[b] += sign A[b] [x0; x1] for the rows row0 .. rows - 1 of `batch` matrices A[b] of 2 nc
