@@ -721,7 +721,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
             return rc;
         PMLBIE_CUDA_TRY(cudaEventRecord(ev[2], s));
         PMLBIE_CUDA_TRY(cudaMemcpyAsync(w.X, w.B, xbytes, cudaMemcpyDeviceToDevice, s));
-        PMLBIE_CUDA_TRY((batched_lu_solve<double2, double2>(n2, n2, nm, n_rhs, w.A, w.piv, w.X, s)));
+        PMLBIE_CUDA_TRY(batched_lu_solve(n2, nm, n_rhs, w.A, w.piv, w.X, s));
     } else {
         PMLBIE_CUDA_TRY(convert_fro2_c128(n2, np2, nm, w.A, w.A32, w.an, slu));
         if ((rc = batched_lu_graphed(prob, PMLBIE_MIXED, np2, nm, w.A32, w.piv, w.info, w.img, w.ptab, slu)))
@@ -780,7 +780,7 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
                 }
                 PMLBIE_CUDA_TRY(cudaMemcpyAsync(w.active, act.data(), sizeof(int) * nm, cudaMemcpyHostToDevice, s));
             }
-            PMLBIE_CUDA_TRY(refine_step(n2, np2, nm, n_rhs, w.A32, w.piv, w.R, w.w32, w.X, s, w.active, w.dinv, w.ptab));
+            PMLBIE_CUDA_TRY(refine_step(n2, np2, nm, n_rhs, w.A32, w.R, w.w32, w.X, s, w.active, w.dinv, w.ptab));
         }
         int nslow = (int)std::count(slow.begin(), slow.end(), 1), g0 = 0, g1 = 0;
         // FGMRES on the contiguous range of modes [g0, g1) holding every slow mode (its
@@ -815,9 +815,8 @@ static int solve_chunk(pmlbie_problem* prob, int precision, int n_rhs, bool poin
             std::vector<double> gan(an.begin() + g0, an.begin() + g1), gres(mres.begin() + g0, mres.begin() + g1),
                 gbwd(mbwd.begin() + g0, mbwd.begin() + g1);
             const size_t mat = (size_t)n2 * n2, vec = (size_t)n2 * n_rhs;
-            rc = gmres_refine(n2, np2, gn, n_rhs, w.A + g0 * mat, w.A32 + (size_t)g0 * np2 * np2, w.piv + (size_t)g0 * np2,
-                              w.B + g0 * vec, w.X + g0 * vec, gslow, w.active, gm, kGmresM, kGmresCycles, gan, s, git,
-                              gres, gbwd,
+            rc = gmres_refine(n2, np2, gn, n_rhs, w.A + g0 * mat, w.A32 + (size_t)g0 * np2 * np2, w.B + g0 * vec,
+                              w.X + g0 * vec, gslow, w.active, gm, kGmresM, kGmresCycles, gan, s, git, gres, gbwd,
                               w.dinv + (size_t)g0 * diag_inv_elems(np2), w.ptab + (size_t)g0 * lu_ptab_elems(np2, 1));
             cudaStreamSynchronize(s);
             cudaFree(gm);

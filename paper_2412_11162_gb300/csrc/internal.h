@@ -283,17 +283,14 @@ size_t lu_image_bytes(int n, int batch);
 // kernel attributes of batched_lu<T>, set once (call before capturing it)
 template <typename T>
 cudaError_t lu_prepare();
-// active: optional per-matrix flags (0 = skip), used to leave converged modes alone
-// factors in TF, right-hand sides and arithmetic in T (T = double2 with TF = float2:
-// FP64 solves with the FP32 factors)
-// dinv: optional inverses of the 32 x 32 diagonal blocks (batched_diag_inv),
-// used when n is a multiple of 32
-template <typename T, typename TF>
-// ptab: the complex64 factorisation's interchange mapping (batched_lu); then
-// piv is not read.  The right-hand sides have nv <= n rows (padded factors)
-cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, const int* piv, T* B,
-                             cudaStream_t s, const int* active = nullptr, const TF* dinv = nullptr,
-                             const int2* ptab = nullptr);
+// complex128 solves with the factors and the row permutation of batched_lu
+cudaError_t batched_lu_solve(int n, int batch, int nrhs, const double2* LU, const int* perm, double2* B, cudaStream_t s);
+// complex64 solves, n a multiple of 32: the right-hand sides have nv <= n rows (padded
+// factors); active: optional per-matrix flags (0 = skip), used to leave converged modes
+// alone; dinv: the inverses of the 32 x 32 diagonal blocks (batched_diag_inv); ptab: the
+// factorisation's interchange mapping (batched_lu)
+cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const float2* LU, float2* B, cudaStream_t s,
+                             const int* active, const float2* dinv, const int2* ptab);
 // inverses of the 32 x 32 diagonal blocks of L (unit lower) and U of every
 // complex64 factor, [b][n / 32][2][32 x 32] column-major (n a multiple of 32)
 cudaError_t batched_diag_inv(int n, int batch, const float2* LU, float2* dinv, cudaStream_t s);
@@ -307,11 +304,10 @@ cudaError_t convert_fro2_c128(int n, int np, int batch, const double2* A, float2
 // converged modes (gmres_rule of refine_rules.h; an2 = |A_b|_F^2), mode_res / mode_bwd
 // receive their final relative residuals and backward errors.
 size_t gmres_scratch_bytes(int n, int batch, int nrhs, int m);
-int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const float2* LU32, const int* piv,
-                 const double2* B, double2* X, std::vector<int>& act, int* active_dev, void* scratch, int m,
-                 int max_cycles, const std::vector<double>& an2,
-                 cudaStream_t s, int& iters, std::vector<double>& mode_res, std::vector<double>& mode_bwd,
-                 const float2* dinv = nullptr, const int2* ptab = nullptr);
+int gmres_refine(int n, int np, int batch, int nrhs, const double2* A, const float2* LU32, const double2* B,
+                 double2* X, std::vector<int>& act, int* active_dev, void* scratch, int m, int max_cycles,
+                 const std::vector<double>& an2, cudaStream_t s, int& iters, std::vector<double>& mode_res,
+                 std::vector<double>& mode_bwd, const float2* dinv, const int2* ptab);
 // Y[b] += sign A[b] [x0; x1] for the rows row0 .. rows - 1 of `batch` matrices A[b] of 2 nc
 // columns (column-major, leading dimension ld, as apart): columns 0 .. nc - 1 meet x0[b],
 // the others x1[b] ([nc][nrhs], xs apart); rows from `split` on take x0s, x1s instead.
@@ -332,8 +328,7 @@ cudaError_t add_product_c128(const ProductArgs& a, int batch, cudaStream_t s);
 cudaError_t residual_c128(int n, int batch, int nrhs, const double2* A, const double2* X,
                           const double2* B, double2* R, double* rnorm, double* bnorm, double* xnorm,
                           cudaStream_t s, const int* active = nullptr);
-cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const int* piv,
-                        const double2* R, float2* work32, double2* X, cudaStream_t s,
-                        const int* active = nullptr, const float2* dinv = nullptr, const int2* ptab = nullptr);
+cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const double2* R, float2* work32,
+                        double2* X, cudaStream_t s, const int* active, const float2* dinv, const int2* ptab);
 
 }  // namespace pmlbie

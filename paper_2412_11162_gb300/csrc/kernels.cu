@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256, NB == 1 ? 3 : 2) far_kernel(FarArgs a) {
     extern __shared__ double2 smem[];
     const int M = a.M, N = a.N, K = M / 2, S1 = K + 1;
     const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int TM = far_tile_m(nw), TL = nw / TM;
+    const int TM = kFarTileM, TL = nw / TM;
     const int l0 = blockIdx.x * TL, m0 = blockIdx.y * TM;
     if (l0 + TL - 1 < m0) return;               // the whole tile has l < m: mirrored elsewhere
     int4* tw = reinterpret_cast<int4*>(smem);   // 3M/4: e^{-2 pi i e / M}
@@ -907,7 +907,7 @@ cudaError_t launch_far(const pmlbie_problem* prob, const FarLaunch& fl, cudaStre
     if (e != cudaSuccess) return e;
     auto run = [&](int nw) {
         g_far_pairs_per_cta = nw;
-        const int tm = far_tile_m(nw), tl = nw / tm;
+        const int tm = kFarTileM, tl = nw / tm;
         dim3 grid((N + tl - 1) / tl, (N + tm - 1) / tm);
         return with_half_class(M, [&](auto nb) {
             far_kernel<decltype(nb)::value><<<grid, 32 * nw, far_smem(M, nw), s>>>(a);

@@ -815,280 +815,163 @@ __global__ void __launch_bounds__(256) swap_trsm_kernel(int n, int k0, int kb, i
     }
 }
 
-// Solve LU x = b for every matrix and rhs: the row permutation (gathered
+// Complex128 solves L U x = b for every matrix and rhs: the row permutation (gathered
 // while loading), then blocked unit-lower forward and upper backward
 // substitution.  One CTA (512 threads) per (matrix, group of up to kSolveR
 // right-hand sides); B is [b][n][nrhs].  The group's right-hand sides live in
 // shared memory ([row][R]) for the whole solve, so each factor element read
 // from memory serves all of them; each 32-row diagonal block is solved by one
-// warp per right-hand side, then the rows outside it are updated.  When n is
-// a multiple of 32 (and, with several right-hand sides, the arithmetic is
-// complex64) the update takes two adjacent rows per thread and issues a
-// block's column loads in chunks (256 bytes per thread with one right-hand
-// side; 16-byte loads for complex64 factors), so that enough bytes are in
-// flight to stream the factors at HBM speed; each factor pair then serves
-// every right-hand side of the group, and the next diagonal block is fetched
-// into registers during the update.  With `dinv` (the inverses of the 32 x 32
-// diagonal blocks of L and U, diag_inv_kernel; n a multiple of 32) a
-// diagonal block is applied as a matrix-vector product by one warp per
-// right-hand side, 32 independent products instead of a 32-step dependent
-// substitution that the other warps wait for.  The right-hand sides have nv <= n rows
-// (a factor padded to whole 32-row blocks by an identity; the rows beyond nv are zero
-// and stay so).  Matrices whose active flag is 0 are skipped (converged modes).
+// warp per right-hand side, then the rows outside it are updated.  With one
+// right-hand side and n a multiple of 32 the update takes two adjacent rows per
+// thread and issues a block's column loads in chunks of 256 bytes per thread, so
+// that enough bytes are in flight to stream the factors at HBM speed, and the next
+// diagonal block is fetched into registers during the update.
 constexpr int kSolveR = 8;
 
-template <typename T> __device__ __forceinline__ T widen(float2 v) { return Cx<T>::mk(v.x, v.y); }
-template <typename T> __device__ __forceinline__ T widen(double2 v) { return Cx<T>::mk(v.x, v.y); }
-
-// two adjacent column entries p[0], p[1] (p 16-byte aligned for complex64)
-__device__ __forceinline__ void load_pair(const float2* p, float2& u, float2& v) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
-    u = make_float2(q.x, q.y);
-    v = make_float2(q.z, q.w);
-}
-__device__ __forceinline__ void load_pair(const double2* p, double2& u, double2& v) {
-    u = __ldg(p);
-    v = __ldg(p + 1);
-}
-
-// x[i][q], x[i+1][q] -= sum_{c < kNB} F[c][i..i+1] xs[c][q] for the group's
-// right-hand sides q < nr (a full 32-column block; xs row stride R), factor
+// x[i], x[i+1] -= sum_{c < kNB} F[c][i..i+1] xs[c] (a full 32-column block), factor
 // loads issued in chunks of 256 bytes per thread
-template <typename T, typename TF, int RM>
-__device__ __forceinline__ void block_pair_update(const TF* col, int n, const T* xs, int R, int nr, T (&acc0)[RM],
-                                                  T (&acc1)[RM]) {
-    constexpr int CH = RM == 1 ? (int)(256 / (2 * sizeof(TF))) : 2;
+__device__ __forceinline__ void block_pair_update(const double2* col, int n, const double2* xs, double2& x0, double2& x1) {
+    constexpr int CH = 8;
 #pragma unroll
     for (int c0 = 0; c0 < kNB; c0 += CH) {
-        TF l0[CH], l1[CH];
-#pragma unroll
-        for (int c = 0; c < CH; ++c) load_pair(col + (size_t)(c0 + c) * n, l0[c], l1[c]);
+        double2 l0[CH], l1[CH];
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            const T f0 = widen<T>(l0[c]), f1 = widen<T>(l1[c]);
+            l0[c] = __ldg(col + (size_t)(c0 + c) * n);
+            l1[c] = __ldg(col + (size_t)(c0 + c) * n + 1);
+        }
 #pragma unroll
-            for (int q = 0; q < RM; ++q)
-                if (q < nr) {
-                    const T xc = xs[(c0 + c) * R + q];
-                    acc0[q] = fms(acc0[q], f0, xc);
-                    acc1[q] = fms(acc1[q], f1, xc);
-                }
+        for (int c = 0; c < CH; ++c) {
+            const double2 xc = xs[c0 + c];
+            x0 = fms(x0, l0[c], xc);
+            x1 = fms(x1, l1[c], xc);
         }
     }
 }
 
-template <typename T, typename TF, int RM>
-__global__ void __launch_bounds__(512) lu_solve_kernel(int n, int nv, int nrhs, int Rg, const TF* LU, const int* perm,
-                                                       T* B, const int* active, const TF* dinv, const int2* ptab) {
+template <int RM>
+__global__ void __launch_bounds__(512) lu_solve64_kernel(int n, int nrhs, int Rg, const double2* LU, const int* perm,
+                                                         double2* B) {
+    using T = double2;
     const int R = RM == 1 ? 1 : Rg;    // compile-time 1 in the single-wave variant
     const int b = blockIdx.x, r0 = blockIdx.y * R, nr = RM == 1 ? 1 : min(R, nrhs - r0);
-    if (active && !active[b]) return;
     extern __shared__ unsigned char smraw[];
     T* sx = reinterpret_cast<T*>(smraw);                     // n x R entries, sx[i * R + q]
-    const TF* a = LU + (size_t)b * n * n;
+    const T* a = LU + (size_t)b * n * n;
     const int* pm = perm + (size_t)b * n;
-    T* x = B + (size_t)b * nv * nrhs;
-    __shared__ __align__(16) TF sD[kNB * kNB];     // diagonal block, sD[col * kNB + row]
-    constexpr int kDiagPer = (int)(kNB * kNB * sizeof(TF) / (512 * 16));   // 16-byte pieces per thread
+    T* x = B + (size_t)b * n * nrhs;
+    __shared__ __align__(16) T sD[kNB * kNB];      // diagonal block, sD[col * kNB + row]
+    constexpr int kDiagPer = kNB * kNB / 512;      // of its entries per thread
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nblk = (n + kNB - 1) / kNB;
-    // with ptab the factor's L columns keep the row order of their step: the
-    // right-hand sides are loaded as they are and each step's interchanges are
-    // applied when the forward solve reaches its block; else loaded permuted
-    const int2* pt = ptab ? ptab + (size_t)b * nblk * 2 * kNB : nullptr;
     for (int idx = tid; idx < n * nr; idx += blockDim.x) {
         const int i = idx / nr, q = idx - i * nr;
-        sx[i * R + q] = i < nv ? x[(size_t)(pt ? i : pm[i]) * nrhs + r0 + q] : Cx<T>::mk(0, 0);
+        sx[i * R + q] = x[(size_t)pm[i] * nrhs + r0 + q];
     }
-    // the pair path: full blocks only, and with several right-hand sides only
-    // for complex64 accumulators (register budget of 512 threads)
-    const bool vec = (n % kNB) == 0 && (RM == 1 || sizeof(T) == 8);
-    // (complex64 factors only: the FP64 path keeps the substitution)
-    const bool inv = std::is_same<TF, float2>::value && vec && dinv != nullptr;
-    // diagonal block j0 into registers (16-byte pieces, column by column): the
-    // factor's block, or with inv the inverse of its L (t = 0) or U (t = 1) part
-    const TF* dinv_b = inv ? dinv + (size_t)b * nblk * 2 * kNB * kNB : nullptr;
-    auto fetch_diag = [&](int j0, int jb, int t, float4 (&reg)[kDiagPer]) {
-        if (inv) {
-            // the inverse blocks are contiguous: full 16-byte pieces
-            const float4* src = reinterpret_cast<const float4*>(dinv_b + ((size_t)(j0 / kNB) * 2 + t) * kNB * kNB);
-#pragma unroll
-            for (int q = 0; q < kDiagPer; ++q) reg[q] = __ldg(src + tid + q * 512);
-            return;
-        }
+    // the pair path: full blocks only, one right-hand side (register budget of 512 threads)
+    const bool vec = (n % kNB) == 0 && RM == 1;
+    // diagonal block j0 into registers, or (not vec) straight into sD
+    auto fetch_diag = [&](int j0, T (&reg)[kDiagPer]) {
 #pragma unroll
         for (int q = 0; q < kDiagPer; ++q) {
-            const int e = (tid + q * 512) * (int)(16 / sizeof(TF));     // first element of the piece
-            const int c = e / kNB, i = e - c * kNB;
-            reg[q] = (c < jb && i < jb) ? __ldg(reinterpret_cast<const float4*>(a + (size_t)(j0 + c) * n + j0 + i))
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            const int e = tid + q * 512, c = e / kNB;
+            reg[q] = __ldg(a + (size_t)(j0 + c) * n + j0 + (e - c * kNB));
         }
     };
-    // x_blk <- Inv x_blk for the warp's right-hand side (inv path)
-    auto apply_inv = [&](int j0) {
-        if (warp < nr) {
-            const T v = sx[(j0 + lane) * R + warp];
-            T acc0 = Cx<T>::mk(0, 0), acc1 = acc0;
+    auto store_diag = [&](const T (&reg)[kDiagPer]) {
 #pragma unroll
-            for (int c = 0; c < kNB; c += 2) {
-                const T x0 = Cx<T>::mk(__shfl_sync(0xffffffff, v.x, c), __shfl_sync(0xffffffff, v.y, c));
-                const T x1 = Cx<T>::mk(__shfl_sync(0xffffffff, v.x, c + 1), __shfl_sync(0xffffffff, v.y, c + 1));
-                acc0 = fma_c(acc0, widen<T>(sD[c * kNB + lane]), x0);
-                acc1 = fma_c(acc1, widen<T>(sD[(c + 1) * kNB + lane]), x1);
+        for (int q = 0; q < kDiagPer; ++q) sD[tid + q * 512] = reg[q];
+    };
+    auto load_diag = [&](int j0, int jb) {
+        for (int idx = tid; idx < jb * jb; idx += blockDim.x) {
+            const int c = idx / jb, i = idx % jb;
+            sD[c * kNB + i] = a[(size_t)(j0 + c) * n + j0 + i];
+        }
+        __syncthreads();
+    };
+    // rows [first, last) less the block's columns times its solution
+    auto update = [&](int j0, int jb, int first, int last) {
+        if (vec) {
+            for (int i = first + 2 * tid; i < last; i += 2 * blockDim.x) {
+                T x0 = sx[i], x1 = sx[i + 1];
+                block_pair_update(a + (size_t)j0 * n + i, n, sx + j0, x0, x1);
+                sx[i] = x0;
+                sx[i + 1] = x1;
             }
-            sx[(j0 + lane) * R + warp] = add(acc0, acc1);
+            return;
+        }
+        for (int i = first + tid; i < last; i += blockDim.x) {
+            T acc[RM];
+#pragma unroll
+            for (int q = 0; q < RM; ++q)
+                if (q < nr) acc[q] = sx[i * R + q];
+#pragma unroll 8
+            for (int c = 0; c < jb; ++c) {
+                const T l = a[(size_t)(j0 + c) * n + i];
+#pragma unroll
+                for (int q = 0; q < RM; ++q)
+                    if (q < nr) acc[q] = fms(acc[q], l, sx[(j0 + c) * R + q]);
+            }
+#pragma unroll
+            for (int q = 0; q < RM; ++q)
+                if (q < nr) sx[i * R + q] = acc[q];
         }
     };
-    auto store_diag = [&](const float4 (&reg)[kDiagPer]) {
-#pragma unroll
-        for (int t = 0; t < kDiagPer; ++t) reinterpret_cast<float4*>(sD)[tid + t * 512] = reg[t];
-    };
-    float4 dreg[kDiagPer];
-    int2 pn0 = make_int2(-1, -1), pn1 = pn0;   // interchange entries of the next block (ptab)
-    if (pt && warp < nr) {
-        pn0 = pt[lane];
-        pn1 = pt[32 + lane];
-    }
+    T dreg[kDiagPer];
     // forward: L y = x (unit diagonal)
     if (vec) {
-        fetch_diag(0, kNB, 0, dreg);
+        fetch_diag(0, dreg);
         store_diag(dreg);
     }
     __syncthreads();
     for (int j0 = 0; j0 < n; j0 += kNB) {
         const int jb = min(kNB, n - j0);
-        if (!vec) {
-            for (int idx = tid; idx < jb * jb; idx += blockDim.x) {
-                const int c = idx / jb, i = idx % jb;
-                sD[c * kNB + i] = a[(size_t)(j0 + c) * n + j0 + i];
-            }
-            __syncthreads();
-        }
-        if (pt && warp < nr) {
-            // this step's interchanges on the warp's right-hand side: slots lane, lane + 32
-            // (entries loaded one block ahead, off the critical path)
-            const int2 e0 = pn0, e1 = pn1;
-            if (j0 + kNB < n) {
-                pn0 = pt[(size_t)(j0 / kNB + 1) * 2 * kNB + lane];
-                pn1 = pt[(size_t)(j0 / kNB + 1) * 2 * kNB + 32 + lane];
-            }
-            const T v0 = e0.x >= 0 ? sx[e0.y * R + warp] : Cx<T>::mk(0, 0);
-            const T v1 = e1.x >= 0 ? sx[e1.y * R + warp] : Cx<T>::mk(0, 0);
-            __syncwarp();
-            if (e0.x >= 0) sx[e0.x * R + warp] = v0;
-            if (e1.x >= 0) sx[e1.x * R + warp] = v1;
-            __syncwarp();
-        }
-        if (inv) {
-            apply_inv(j0);
-        } else if (warp < nr) {
+        if (!vec) load_diag(j0, jb);
+        if (warp < nr) {
             T v = lane < jb ? sx[(j0 + lane) * R + warp] : Cx<T>::mk(0, 0);
             for (int c = 0; c < jb; ++c) {
                 T xc = Cx<T>::mk(__shfl_sync(0xffffffff, v.x, c), __shfl_sync(0xffffffff, v.y, c));
-                if (lane > c && lane < jb) v = fms(v, widen<T>(sD[c * kNB + lane]), xc);
+                if (lane > c && lane < jb) v = fms(v, sD[c * kNB + lane], xc);
             }
             if (lane < jb) sx[(j0 + lane) * R + warp] = v;
         }
         __syncthreads();
-        if (vec) {
-            const bool more = j0 + kNB < n;
-            if (more) fetch_diag(j0 + kNB, kNB, 0, dreg);
-            for (int i = j0 + kNB + 2 * tid; i < n; i += 2 * blockDim.x) {
-                T acc0[RM], acc1[RM];
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) acc0[q] = sx[i * R + q], acc1[q] = sx[(i + 1) * R + q];
-                block_pair_update<T, TF, RM>(a + (size_t)j0 * n + i, n, sx + (size_t)j0 * R, R, nr, acc0, acc1);
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) sx[i * R + q] = acc0[q], sx[(i + 1) * R + q] = acc1[q];
-            }
-            __syncthreads();
-            if (more) store_diag(dreg);
-        } else {
-            for (int i = j0 + jb + tid; i < n; i += blockDim.x) {
-                T acc[RM];
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) acc[q] = sx[i * R + q];
-#pragma unroll 8
-                for (int c = 0; c < jb; ++c) {
-                    const T l = widen<T>(a[(size_t)(j0 + c) * n + i]);
-#pragma unroll
-                    for (int q = 0; q < RM; ++q)
-                        if (q < nr) acc[q] = fms(acc[q], l, sx[(j0 + c) * R + q]);
-                }
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) sx[i * R + q] = acc[q];
-            }
-        }
+        const bool more = vec && j0 + kNB < n;
+        if (more) fetch_diag(j0 + kNB, dreg);
+        update(j0, jb, j0 + jb, n);
+        if (vec) __syncthreads();
+        if (more) store_diag(dreg);
         __syncthreads();
     }
     // backward: U x = y
     if (vec) {
-        fetch_diag((nblk - 1) * kNB, kNB, 1, dreg);
+        fetch_diag((nblk - 1) * kNB, dreg);
         store_diag(dreg);
         __syncthreads();
     }
     for (int bi = nblk - 1; bi >= 0; --bi) {
         const int j0 = bi * kNB, jb = min(kNB, n - j0);
-        if (!vec) {
-            for (int idx = tid; idx < jb * jb; idx += blockDim.x) {
-                const int c = idx / jb, i = idx % jb;
-                sD[c * kNB + i] = a[(size_t)(j0 + c) * n + j0 + i];
-            }
-            __syncthreads();
-        }
-        if (inv) {
-            apply_inv(j0);
-        } else if (warp < nr) {
+        if (!vec) load_diag(j0, jb);
+        if (warp < nr) {
             T v = lane < jb ? sx[(j0 + lane) * R + warp] : Cx<T>::mk(0, 0);
             // every pivot's reciprocal at once, not in the chain of the columns
-            const T rd = lane < jb ? rcp(widen<T>(sD[lane * kNB + lane])) : v;
+            const T rd = lane < jb ? rcp(sD[lane * kNB + lane]) : v;
             for (int c = jb - 1; c >= 0; --c) {
                 if (lane == c) v = mul(v, rd);
                 T xc = Cx<T>::mk(__shfl_sync(0xffffffff, v.x, c), __shfl_sync(0xffffffff, v.y, c));
-                if (lane < c) v = fms(v, widen<T>(sD[c * kNB + lane]), xc);
+                if (lane < c) v = fms(v, sD[c * kNB + lane], xc);
             }
             if (lane < jb) sx[(j0 + lane) * R + warp] = v;
         }
         __syncthreads();
-        if (vec) {
-            if (bi > 0) fetch_diag(j0 - kNB, kNB, 1, dreg);
-            for (int i = 2 * tid; i < j0; i += 2 * blockDim.x) {
-                T acc0[RM], acc1[RM];
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) acc0[q] = sx[i * R + q], acc1[q] = sx[(i + 1) * R + q];
-                block_pair_update<T, TF, RM>(a + (size_t)j0 * n + i, n, sx + (size_t)j0 * R, R, nr, acc0, acc1);
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) sx[i * R + q] = acc0[q], sx[(i + 1) * R + q] = acc1[q];
-            }
-            __syncthreads();
-            if (bi > 0) store_diag(dreg);
-        } else {
-            for (int i = tid; i < j0; i += blockDim.x) {
-                T acc[RM];
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) acc[q] = sx[i * R + q];
-#pragma unroll 8
-                for (int c = 0; c < jb; ++c) {
-                    const T u = widen<T>(a[(size_t)(j0 + c) * n + i]);
-#pragma unroll
-                    for (int q = 0; q < RM; ++q)
-                        if (q < nr) acc[q] = fms(acc[q], u, sx[(j0 + c) * R + q]);
-                }
-#pragma unroll
-                for (int q = 0; q < RM; ++q)
-                    if (q < nr) sx[i * R + q] = acc[q];
-            }
-        }
+        const bool more = vec && bi > 0;
+        if (more) fetch_diag(j0 - kNB, dreg);
+        update(j0, jb, 0, j0);
+        if (vec) __syncthreads();
+        if (more) store_diag(dreg);
         __syncthreads();
     }
-    for (int idx = tid; idx < nv * nr; idx += blockDim.x) {
+    for (int idx = tid; idx < n * nr; idx += blockDim.x) {
         const int i = idx / nr, q = idx - i * nr;
         x[(size_t)i * nrhs + r0 + q] = sx[i * R + q];
     }
@@ -1521,51 +1404,45 @@ cudaError_t batched_lu(int n, int batch, T* A, int* piv, int* info, cudaStream_t
     return cudaGetLastError();
 }
 
-template <typename T, typename TF>
-cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const TF* LU, const int* piv, T* B,
-                             cudaStream_t s, const int* active, const TF* dinv, const int2* ptab) {
-    if constexpr (std::is_same<T, float2>::value && std::is_same<TF, float2>::value) {
-        // streamed solves: right-hand sides per CTA a power of two that shared memory holds
-        // (n up to 14000; beyond, the general kernel)
-        constexpr size_t kSmem = 227 * 1024;
-        int R = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
-        while (R > 1 && st_smem(n, R) > kSmem) R /= 2;
-        const size_t sm = st_smem(n, R);
-        if (dinv && ptab && n % kNB == 0 && sm <= kSmem) {
-            auto run = [&](auto kernel) {
-                cudaError_t e = allow_max_smem(kernel);
-                if (e != cudaSuccess) return e;
-                kernel<<<dim3(batch, (nrhs + R - 1) / R), kStThreads, sm, s>>>(n, nv, nrhs, st_rows(n), LU, B, active, dinv, ptab);
-                count_launch();
-                return cudaGetLastError();
-            };
-            return R == 8 ? run(lu_solve32_kernel<8>) : R == 4 ? run(lu_solve32_kernel<4>)
-                 : R == 2 ? run(lu_solve32_kernel<2>) : run(lu_solve32_kernel<1>);
-        }
-    }
+cudaError_t batched_lu_solve(int n, int batch, int nrhs, const double2* LU, const int* perm, double2* B, cudaStream_t s) {
     // right-hand sides per CTA: up to kSolveR, as many as fit in shared memory
     // (about 200 KB for the group)
     int R = std::min(nrhs, kSolveR);
-    while (R > 1 && sizeof(T) * (size_t)R * (size_t)n > 200 * 1024) --R;
-    dim3 g(batch, (nrhs + R - 1) / R);
+    while (R > 1 && sizeof(double2) * (size_t)R * (size_t)n > 200 * 1024) --R;
+    const dim3 g(batch, (nrhs + R - 1) / R);
     // dynamic: right-hand sides; static: the 32 x 32 diagonal block
-    size_t sm = sizeof(T) * (size_t)R * (size_t)n;
-    const bool big = sm + sizeof(TF) * kNB * kNB > 48 * 1024;
-    if (R == 1) {   // the common single-wave case, without the group loops
-        if (big) {
-            cudaError_t e = allow_max_smem(lu_solve_kernel<T, TF, 1>);
+    const size_t sm = sizeof(double2) * (size_t)R * (size_t)n;
+    auto run = [&](auto kernel) {
+        if (sm + sizeof(double2) * kNB * kNB > 48 * 1024) {
+            cudaError_t e = allow_max_smem(kernel);
             if (e != cudaSuccess) return e;
         }
-        lu_solve_kernel<T, TF, 1><<<g, 512, sm, s>>>(n, nv, nrhs, R, LU, piv, B, active, dinv, ptab);
-    } else {
-        if (big) {
-            cudaError_t e = allow_max_smem(lu_solve_kernel<T, TF, kSolveR>);
-            if (e != cudaSuccess) return e;
-        }
-        lu_solve_kernel<T, TF, kSolveR><<<g, 512, sm, s>>>(n, nv, nrhs, R, LU, piv, B, active, dinv, ptab);
-    }
-    count_launch();
-    return cudaGetLastError();
+        kernel<<<g, 512, sm, s>>>(n, nrhs, R, LU, perm, B);
+        count_launch();
+        return cudaGetLastError();
+    };
+    // the common single-wave case without the group loops
+    return R == 1 ? run(lu_solve64_kernel<1>) : run(lu_solve64_kernel<kSolveR>);
+}
+
+cudaError_t batched_lu_solve(int n, int nv, int batch, int nrhs, const float2* LU, float2* B, cudaStream_t s,
+                             const int* active, const float2* dinv, const int2* ptab) {
+    if (n % kNB) return cudaErrorInvalidValue;
+    // right-hand sides per CTA a power of two that shared memory holds beside whole stages
+    // (8 up to n = 1838, one from 7353 on); from n = 14705 on the stages shrink
+    int R = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
+    while (R > 1 && st_rows(n, R) < std::min(n, kStRows)) R /= 2;
+    const int sr = st_rows(n, R);
+    if (sr == 0) return cudaErrorInvalidValue;
+    auto run = [&](auto kernel) {
+        cudaError_t e = allow_max_smem(kernel);
+        if (e != cudaSuccess) return e;
+        kernel<<<dim3(batch, (nrhs + R - 1) / R), kStThreads, st_smem(n, R, sr), s>>>(n, nv, nrhs, sr, LU, B, active, dinv, ptab);
+        count_launch();
+        return cudaGetLastError();
+    };
+    return R == 8 ? run(lu_solve32_kernel<8>) : R == 4 ? run(lu_solve32_kernel<4>)
+         : R == 2 ? run(lu_solve32_kernel<2>) : run(lu_solve32_kernel<1>);
 }
 
 template cudaError_t lu_prepare<double2>();
@@ -1574,13 +1451,6 @@ template cudaError_t batched_lu<double2>(int, int, double2*, int*, int*, cudaStr
                                           const LuSide*, cudaEvent_t*, size_t);
 template cudaError_t batched_lu<float2>(int, int, float2*, int*, int*, cudaStream_t, unsigned char*, int2*,
                                          const LuSide*, cudaEvent_t*, size_t);
-template cudaError_t batched_lu_solve<double2, double2>(int, int, int, int, const double2*, const int*, double2*,
-                                                        cudaStream_t, const int*, const double2*, const int2*);
-template cudaError_t batched_lu_solve<float2, float2>(int, int, int, int, const float2*, const int*, float2*,
-                                                      cudaStream_t, const int*, const float2*, const int2*);
-template cudaError_t batched_lu_solve<double2, float2>(int, int, int, int, const float2*, const int*, double2*,
-                                                       cudaStream_t, const int*, const float2*, const int2*);
-
 cudaError_t convert_to_c64(int64_t count, const double2* src, float2* dst, cudaStream_t s) {
     int blocks = (int)std::min<int64_t>((count + 255) / 256, 152 * 32);
     c128_to_c64_kernel<<<blocks, 256, 0, s>>>(count, src, dst);
@@ -1651,13 +1521,12 @@ cudaError_t batched_diag_inv(int n, int batch, const float2* LU, float2* dinv, c
     return cudaGetLastError();
 }
 
-cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const int* piv,
-                        const double2* R, float2* work32, double2* X, cudaStream_t s, const int* active,
-                        const float2* dinv, const int2* ptab) {
+cudaError_t refine_step(int n, int np, int batch, int nrhs, const float2* LU32, const double2* R, float2* work32,
+                        double2* X, cudaStream_t s, const int* active, const float2* dinv, const int2* ptab) {
     int64_t cnt = (int64_t)batch * n * nrhs;
     cudaError_t e = convert_to_c64(cnt, R, work32, s);
     if (e != cudaSuccess) return e;
-    e = batched_lu_solve<float2, float2>(np, n, batch, nrhs, LU32, piv, work32, s, active, dinv, ptab);
+    e = batched_lu_solve(np, n, batch, nrhs, LU32, work32, s, active, dinv, ptab);
     if (e != cudaSuccess) return e;
     add_correction_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(cnt, (int64_t)n * nrhs, work32, X, active);
     count_launch();

@@ -20,10 +20,15 @@ namespace {
 
 constexpr int kStRows = 512, kStCols = 8, kStages = 3, kStThreads = 544;
 constexpr uint32_t kStDiag = 32 * 32 * 8, kStOffDiag = 128, kStOffX = kStOffDiag + 2 * kStDiag;
-// rows of a stage (small systems leave room for another CTA) and the CTA's shared memory:
-// barriers, inverse blocks, right-hand sides, stages
-inline int st_rows(int n) { return n < kStRows ? n : kStRows; }
-inline size_t st_smem(int n, int R) { return kStOffX + 8 * (size_t)n * R + (size_t)kStages * st_rows(n) * kStCols * 8; }
+// the CTA's shared memory: barriers, inverse blocks, right-hand sides, stages of `rows` rows
+// (small systems leave room for another CTA; large ones leave less for the stages; 0: none)
+constexpr size_t kStSmemMax = 227 * 1024;
+inline size_t st_smem(int n, int R, int rows) { return kStOffX + 8 * (size_t)n * R + (size_t)kStages * rows * kStCols * 8; }
+inline int st_rows(int n, int R) {
+    int rows = n < kStRows ? n : kStRows;
+    while (rows > 0 && st_smem(n, R, rows) > kStSmemMax) rows -= 32;
+    return rows;
+}
 struct StreamBars {
     uint64_t full[kStages], empty[kStages], dfull[2], dempty[2];
     int err;

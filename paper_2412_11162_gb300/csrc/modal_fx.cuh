@@ -84,8 +84,8 @@ struct FarArgs {
     double2* raw;   // [mode][kernel][l][m]
 };
 
-// targets x sources of a CTA with nw pairs
-__host__ __device__ __forceinline__ int far_tile_m(int nw) { return 2; }
+// sources of a far CTA's tile (its pairs over this: targets)
+constexpr int kFarTileM = 2;
 
 // Pair of lane `lane` (< nw) of a far CTA: target l = l0 + lane % TL, source m =
 // m0 + lane / TL.  Returns its flags (bit 0: (l, m) is far; bit 1: (m, l) is far;
@@ -112,7 +112,7 @@ __device__ __forceinline__ int far_pair_setup(const FarArgs& a, int l, int m, Pa
 // fixed point with exponents exs[4 w ..].
 __device__ __forceinline__ void far_scatter(const FarArgs& a, int nw, int l0, int m0, const longlong2* spec,
                                             const int* exs, const FarPairFx* pf, const int* act) {
-    const int N = a.N, S1 = a.M / 2 + 1, TM = far_tile_m(nw), TL = nw / TM;
+    const int N = a.N, S1 = a.M / 2 + 1, TM = kFarTileM, TL = nw / TM;
     const int nmodes = a.mode_hi - a.mode_lo;
     const int lg = __ffs(nw) - 1, lgl = __ffs(TL) - 1;
     const int total = nmodes << lg;
