@@ -407,7 +407,7 @@ int  pmlbie_selftest_wait(long long iterations, void* stream);
  * array dev_x, into device array dev_out:
  *   fn 30: exp(x)           -> out[i]   (0 below the normal range, infinity above)
  *   fn 31: sin(x), cos(x)   -> out[2 i], out[2 i + 1]   (0 <= x < 2^63)
- *   fn 32: 1/sqrt(x)        -> out[i]   (x > 0 normal)
+ *   fn 32: 1/sqrt(x)        -> out[i]   (x > 0 normal; else NaN)
  *   of the sampling loops, on the integer pipe but for the last,
  *   fn 33, 34: sin(x)/x, (sin x - x cos x)/x^3 -> out[i]   (x > 0) of the close pairs;
  *   fn 0, 1, 2: exp (arguments clamped to [-708, 709]), sin and cos, 1/sqrt in

@@ -107,9 +107,10 @@ __device__ __forceinline__ i64 fx_exp(double x, const FxTab& T, int& ex) {
     return ((i64)t2.x << 32) + t2.y + (fx_mul(p, t2.x, t2.y) >> 7);
 }
 
-// 1/sqrt(x), x > 0 normal
+// 1/sqrt(x), x > 0 normal; NaN for zero (a receiver on a node), denormals, x < 0, infinity
 __device__ __forceinline__ double fx_rsqrt(double x) {
     const int hw = __double2hiint(x), e = (hw >> 20) - 1023;
+    if ((unsigned)hw - 0x00100000u >= 0x7fe00000u) return __hiloint2double(0x7ff80000, 0);
     const unsigned mant = ((unsigned)hw << 12) | ((unsigned)__double2loint(x) >> 20);
     float y;      // estimate for the significand in [1, 4)
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(((127u + (e & 1)) << 23) | (mant >> 9))));

@@ -52,6 +52,21 @@ def test_rsqrt():
     got, ref = _run(32, x), 1 / np.sqrt(x.astype(LD))
     err = np.abs(got.astype(LD) - ref) / ref
     assert np.max(err) <= 2.0 ** -52, (float(np.max(err)) * 2.0 ** 52, x[np.argmax(err)])
+    # outside: NaN
+    assert np.all(np.isnan(_run(32, np.array([0.0, -0.0, 5e-324, 2.0 ** -1023, -1.0, -np.inf, np.inf, np.nan]))))
+
+
+def test_field_on_a_node_is_not_a_number():
+    """The kernels are infinite there: every mode of that receiver, and of no other, is NaN."""
+    import torch
+    from paper_2412_11162_gb300 import Problem
+    P = Problem(2 * np.pi, 3 * np.pi, 64, 32)
+    node, m = P.nodes(), 20
+    one = torch.ones((P.n_modes, P.N, 1), dtype=torch.complex128, device="cuda")
+    rho, z = np.array([node["rho"][m], 0.7]), np.array([node["z"][m], 0.9])
+    for region in ([0, 0], [1, 0]):
+        got = P.field(rho, z, np.array(region), dict(u1=one, phi1=one, u2=one, phi2=one)).cpu().numpy()
+        assert np.all(np.isnan(got[:, 0])) and np.all(np.isfinite(got[:, 1]))
 
 
 def test_small_phase_quotients():
