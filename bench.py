@@ -343,8 +343,8 @@ def run_ours(args, rank, world):
               "near_modes_kernel": last.ms_near - last.ms_near_laplace,
               "assemble": last.ms_assemble, "lu_fp32": last.ms_lu, "solve_refine": last.ms_solve}
     clocks = clk.summary()
-    roof = near_roofline(w, last, pk, clocks, ncounts, pipes)
-    roof_far = roofline(w, last, pk, clocks, pipes)
+    roof = near_roofline(w, last, pk, ncounts)
+    roof_far = roofline(w, last, pk)
     roof_lu = lu_update_roofline(w, last, pk)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -603,9 +603,9 @@ def run_batched(args, rank, world):
     d2h = sum(4 * o["u1"].numel() * 16 for o in outs)
     big = max(range(8), key=lambda i: reps[i].ms_far)
     clocks = clk.summary()
-    roof = near_roofline(inst[big], reps[big], peaks(), clocks, near_counts(probs[big]), pipes)
+    roof = near_roofline(inst[big], reps[big], peaks(), near_counts(probs[big]))
     roof["kernel"] += " of the N=%d instance" % inst[big]["N"]
-    roof_far = roofline(inst[big], reps[big], peaks(), clocks, pipes)
+    roof_far = roofline(inst[big], reps[big], peaks())
     roof_far["kernel"] += " of the N=%d instance" % inst[big]["N"]
     line = {
         "metric": METRIC, "value": job_value(world, ent, ms), "unit": UNIT, "n_gpus": world, "steps": steps,
@@ -726,7 +726,7 @@ def profile_traffic(path, src_name, units):
     return float(vals["dram_bytes_per_unit"]) * units
 
 
-def near_roofline(w, rep, pk, clk, counts, pipes=None):
+def near_roofline(w, rep, pk, counts):
     """Roofline of the close-pair modes kernel (all close pairs, one launch per
     mode chunk), the HBM view: algorithmic bytes = per pair the 2 M Laplace
     modes read and the 4 kernels' modes written.  The kernel is bounded by
@@ -742,17 +742,19 @@ def near_roofline(w, rep, pk, clk, counts, pipes=None):
     nbytes = float(n) * (2 * M + 4 * rep.chunk_modes) * 16
     hbm = pk.get("hbm_gbs", 6794.1)
     ach = nbytes / (ms1 / 1e3) / 1e9
+    traffic = profile_traffic("near_modes_kernel_n512_m256.md", "kernels.cu", nbytes)
     return {"kernel": "near_modes_kernel (close pairs: split samples, even DFTs in block fixed point, convolution with "
                       "the exact Laplace modes)",
-            "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": None,
+            "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": traffic,
             "flops_per_launch": near_flops_per_launch(M, rep.chunk_modes, packed, npml, plain, couples),
             "ms_per_launch": ms1, "launches_per_step": launches, "pairs": n, "pml_couples": couples,
             "algorithmic_bytes": nbytes, "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)",
             "time_note": "span in the step, where it runs beside the far-pair kernel",
-            "traffic_note": "null: no ncu capture of the current kernels.cu"}
+            "traffic_note": ("ncu dram read+write per algorithmic byte (profiles/near_modes_kernel_n512_m256.md)"
+                             if traffic else "null: no ncu capture of the current kernels.cu")}
 
 
-def roofline(w, rep, pk, clk, pipes=None):
+def roofline(w, rep, pk):
     """Roofline of the far-pair kernel (sampling, fixed-point transforms and
     block scatter), the HBM view of
     SURVEY-style stage a3: algorithmic bytes = the 4 N^2 (M/2) complex128
@@ -768,7 +770,7 @@ def roofline(w, rep, pk, clk, pipes=None):
     wbytes = 4.0 * w["N"] ** 2 * rep.chunk_modes * 16
     hbm = pk.get("hbm_gbs", 6794.1)
     ach = wbytes / (ms1 / 1e3) / 1e9
-    traffic = None
+    traffic = profile_traffic("far_kernel_n512_m256.md", "kernels.cu", wbytes)
     return {"kernel": "far_kernel (S~, K~ sampling of both media per unordered pair + 4 even DFTs in block fixed point "
                       "+ block scatter of both orientations)",
             "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": traffic,
@@ -777,7 +779,8 @@ def roofline(w, rep, pk, clk, pipes=None):
                           "step it runs beside the close-pair kernels" if alone > 0 else
                           "span of the launch in the step (runs beside the close-pair kernels)"),
             "peak_note": "measured HBM copy bandwidth (MEASURED_PEAKS.json)",
-            "traffic_note": "null: no ncu capture of the current kernels.cu"}
+            "traffic_note": ("ncu dram read+write per algorithmic byte (profiles/far_kernel_n512_m256.md)"
+                             if traffic else "null: no ncu capture of the current kernels.cu")}
 
 
 def lu_update_roofline(w, rep, pk):
