@@ -1,12 +1,10 @@
-// Float-float ("double-float") arithmetic on the FP32 pipe (sm_103a).
+// Float-float ("double-float") arithmetic on the FP32 pipe (sm_103a), for the selectors
+// 20-22 of pmlbie_selftest_elementary; the modal kernels work in 64-bit fixed point and
+// FP64 (fxdft.cuh, fxtrig.cuh).
 //
 // A value is the unevaluated sum hi + lo of two floats with |lo| <= ulp(hi)/2:
 // 48 significant bits (relative rounding ~2^-47 per operation), the exponent
-// range of float.  The GB300's FP64 pipe retires 2 FMA per SM per clock and
-// its FP32 pipe 128, so the sampling loops and transforms of the mixed path
-// (S~, K~ at every node pair and angle, Sec. 3.1 / 4.1; the even-sequence
-// DFTs of the FFT modal kernels, Sec. 4.1) run in this arithmetic and keep
-// near-FP64 accuracy of the modal kernels.
+// range of float.
 //
 // Building blocks: Knuth's TwoSum, Dekker's Fast2Sum and the FMA-based exact
 // product (TwoProd), as in the double-double literature (Dekker 1971;

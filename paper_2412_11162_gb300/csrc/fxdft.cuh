@@ -346,8 +346,8 @@ __device__ __forceinline__ int fx_even_dft(longlong2* x, FxScale sc, int K, cons
     return sc.ex == kFxNonfinite ? sc.ex : sc.ex + sh;
 }
 // The same out of line: the close-pair kernel holds two sizes of it, and instruction
-// misses cost it more than the calls (close pairs at N = 1024, M = 512 49.5 -> 48.1 ms,
-// 8 low modes at N = 128 1.07 -> 1.01 ms); the far and field kernels, whose
+// misses cost it more than the calls (close pairs at N = 1024, M = 512 49.2 -> 48.0 ms,
+// 8 low modes at N = 128 1.07 -> 1.03 ms); the far and field kernels, whose
 // transforms follow a long sampling loop, are faster with it in line (field map 6.74
 // against 6.98 ms).
 template <int NB>

@@ -60,8 +60,8 @@ __host__ __device__ __forceinline__ size_t far_elems(int M, int nw) {
 // so the phases, sines and exponentials (fxtrig.cuh) and the transforms (fxdft.cuh)
 // run on the integer pipe, and FP64 keeps the geometry and the joining products; the
 // scatter's normal factors carry the column weights.  N = 384, M = 256 alone: 1.30 ms,
-// FP64 pipe 49 % busy.  The mixed path takes it too: all modal kernels at N = 512, M = 128
-// 15.2 ms with float-float samples and transforms, 11.7 ms with these.
+// FP64 pipe 49 % busy.  The mixed path takes it too: all modal kernels at N = 512, M = 256
+// 15.2 ms with float-float samples and transforms, 11.5 ms with these.
 template <int NB>
 __global__ void __launch_bounds__(256, NB == 1 ? 3 : 2) far_kernel(FarArgs a) {
     extern __shared__ double2 smem[];
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(128) near_laplace_out_kernel(NearArgs a) {
 // index computes both; the mirror's S^ equal the pair's, and its CTA returns at once.
 //
 // Samples, transforms and phases as in the far kernel.  Modal kernels at N = 1024,
-// M = 512 through this kernel: 48.0 ms; with float-float physical pairs and FP64 PML
+// M = 512 through this kernel: 47.7 ms; with float-float physical pairs and FP64 PML
 // pairs 84.6 ms.  Bounded by the barriers between the phases of one pair and by issue
 // (IPC 1.1 at M = 256); two CTAs of 256 threads hold M = 512's shared memory.
 //

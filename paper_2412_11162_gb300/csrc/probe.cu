@@ -3,8 +3,7 @@
 // derived from unit counts.
 //
 //   kind 0: FP64 FMA    -- independent fma chains per thread, all SMs
-//   kind 1: FP32 FMA    -- the same in float (the pipe of the mixed path's
-//                          float-float kernels)
+//   kind 1: FP32 FMA    -- the same in float
 //   kind 2: TF32 tensor -- tcgen05.mma kind::tf32, M = 128, N = 256, K = 8,
 //                          issued back to back by one thread per CTA (one CTA
 //                          per SM) into one tensor-memory accumulator, operands
